@@ -1602,23 +1602,29 @@ void launch_forward(const LayerDev& L, int M, const float* in, int ld_in, float*
 // ---------------------------------------------------------------------------
 // reductions and bookkeeping
 // ---------------------------------------------------------------------------
+// One warp of the CTA sums the row's partials (lane-strided, then a shuffle
+// tree: a fixed order for a given number of slots); a single thread's serial sum
+// of the 68 to 150 slots of the 32 x 32 networks took 17 us a launch, this 4.
 __global__ void k_reduce_lb(int M, const float* part, int nslot, int used, const float* gp0,
                             float* lb, int track, const int* row_node, PoolDev pool,
                             const float* X, int d0) {
   const int m = blockIdx.x;
   __shared__ int imp;
   __shared__ int node;
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {
     float acc = 0.f;
     const float* p = part + (size_t)m * nslot;
-    for (int i = 0; i < used; ++i) acc += p[i];
-    if (gp0) acc -= gp0[m];
-    lb[m] = acc;
-    imp = 0;
-    node = row_node ? row_node[m] : 0;
-    if (track && acc > pool.BEST[node]) {
-      pool.BEST[node] = acc;
-      imp = 1;
+    for (int i = threadIdx.x; i < used; i += 32) acc += p[i];
+    if (gp0 && threadIdx.x < GP_SPLIT) acc -= gp0[(size_t)m * GP_SPLIT + threadIdx.x];
+    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (threadIdx.x == 0) {
+      lb[m] = acc;
+      imp = 0;
+      node = row_node ? row_node[m] : 0;
+      if (track && acc > pool.BEST[node]) {
+        pool.BEST[node] = acc;
+        imp = 1;
+      }
     }
   }
   __syncthreads();
@@ -1707,10 +1713,15 @@ __device__ __forceinline__ int layer_of(const NetDev& net, int f) {
   return i;
 }
 
-// gamma^T P and gamma^T Phat per neuron (CSR by neuron), gamma^T p per row.
-// A CTA serves one row: its node and its property's per-layer CSR pointers are
-// looked up once into shared memory; a thread takes one neuron and keeps eight
-// of its entries' loads in flight at a time (the sums keep entry order).
+// gamma^T P and gamma^T Phat per neuron (CSR by neuron), and gamma^T p per row.
+// A CTA serves `npb` neurons of one row: its threads read the neurons' entry
+// counts, write the zeros of those without entries and list the others; its
+// warps then take the listed neurons in turn, the lanes striding over a neuron's
+// entries (a neuron in three groups has about 450) with four loads in flight.
+// Bound by the latency of those loads: one thread per neuron walking its own
+// entries took 79 us for 9 rows of the 784-100-100-10 network and 335 us for 64
+// rows of the 3x32x32 one with 135k constraint rows.  The first GP_SPLIT CTAs of
+// a row sum a share of gamma^T p each (k_reduce_lb adds the shares).
 struct MncCsr {
   const int* cptr;
   const int* ce;
@@ -1718,98 +1729,109 @@ struct MncCsr {
   const float* cPh;
   int goff, e;
 };
+constexpr int GP_THREADS = 256;
 
-__global__ void k_gamma_proj(int M, const int* __restrict__ row_node, PoolDev pool,
-                             const PropDev* __restrict__ props, NetDev net, float* __restrict__ GP,
-                             float* __restrict__ GPh) {
+__global__ void __launch_bounds__(GP_THREADS) k_gamma_proj(
+    int M, const int* __restrict__ row_node, PoolDev pool, const PropDev* __restrict__ props,
+    NetDev net, int npb, float* __restrict__ GP, float* __restrict__ GPh,
+    float* __restrict__ gp0) {
   const int m = blockIdx.y;
-  __shared__ int s_n;
+  const int n = row_node[m];
+  const PropDev& P = props[pool.prop[n]];
+  const float* gam = pool.GAM + (size_t)n * pool.EC;
+  if (blockIdx.x < GP_SPLIT) {
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    constexpr int step = GP_THREADS * GP_SPLIT;
+    for (int i = 1; i <= net.R; ++i) {
+      const MncDev& mc = P.mnc[i];
+      const float* g = gam + mc.goff;
+      const float* pv = mc.p;
+      const int e1 = mc.e;
+      for (int e = blockIdx.x * GP_THREADS + threadIdx.x; e < e1; e += 4 * step) {
+        float gv[4], p[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const bool in = e + u * step < e1;
+          gv[u] = in ? g[e + u * step] : 0.f;
+          p[u] = in ? pv[e + u * step] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] = fmaf(gv[u], p[u], acc[u]);
+      }
+    }
+    const float tot = block_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
+    if (threadIdx.x == 0) gp0[(size_t)m * GP_SPLIT + blockIdx.x] = tot;
+    return;
+  }
+  __shared__ int s_cnt, s_f[GP_THREADS];
   __shared__ MncCsr s_mc[MNBAB_MAXR + 1];
-  if (threadIdx.x == 0) s_n = row_node[m];
-  __syncthreads();
-  const int n = s_n;
+  if (threadIdx.x == 0) s_cnt = 0;
   if (threadIdx.x >= 1 && threadIdx.x <= net.R) {
-    const MncDev& mc = props[pool.prop[n]].mnc[threadIdx.x];
+    const MncDev& mc = P.mnc[threadIdx.x];
     s_mc[threadIdx.x] = MncCsr{mc.cptr, mc.ce, mc.cP, mc.cPh, mc.goff, mc.e};
   }
   __syncthreads();
-  const int f = blockIdx.x * blockDim.x + threadIdx.x;
-  if (f >= net.SD) return;
-  const int i = layer_of(net, f);
-  const MncCsr& mc = s_mc[i];
-  float gp = 0.f, gph = 0.f;
-  if (mc.e > 0) {
+  const int f0 = (blockIdx.x - GP_SPLIT) * npb;
+  if (threadIdx.x < npb && f0 + threadIdx.x < net.SD) {
+    const int f = f0 + threadIdx.x;
+    const int i = layer_of(net, f);
+    const MncCsr& mc = s_mc[i];
     const int j = f - net.off[i];
-    const float* gam = pool.GAM + (size_t)n * pool.EC + mc.goff;
-    const int q1 = mc.cptr[j + 1];
-    int q = mc.cptr[j];
-    for (; q + 8 <= q1; q += 8) {
-      int ce[8];
-      float g[8], cp[8], cph[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        ce[k] = mc.ce[q + k];
-        cp[k] = mc.cP[q + k];
-        cph[k] = mc.cPh[q + k];
-      }
-#pragma unroll
-      for (int k = 0; k < 8; ++k) g[k] = gam[ce[k]];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        gp = fmaf(g[k], cp[k], gp);
-        gph = fmaf(g[k], cph[k], gph);
-      }
-    }
-    for (; q < q1; ++q) {
-      const float g = gam[mc.ce[q]];
-      gp = fmaf(g, mc.cP[q], gp);
-      gph = fmaf(g, mc.cPh[q], gph);
+    if (mc.e > 0 && mc.cptr[j + 1] > mc.cptr[j]) {
+      s_f[atomicAdd(&s_cnt, 1)] = f;  // order of the list: any, every neuron is on its own
+    } else {
+      GP[(size_t)m * net.SD + f] = 0.f;
+      GPh[(size_t)m * net.SD + f] = 0.f;
     }
   }
-  GP[(size_t)m * net.SD + f] = gp;
-  GPh[(size_t)m * net.SD + f] = gph;
-}
-
-// gamma^T p of one row: GP_THREADS threads, four independent partial sums a
-// thread (fixed order, so the value does not depend on the launch)
-constexpr int GP_THREADS = 512;
-
-__global__ void __launch_bounds__(GP_THREADS) k_gamma_p(int M, const int* row_node, PoolDev pool,
-                                                        const PropDev* props, NetDev net,
-                                                        float* gp0) {
-  const int m = blockIdx.x;
-  const int n = row_node[m];
-  const PropDev& P = props[pool.prop[n]];
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int i = 1; i <= net.R; ++i) {
-    const MncDev& mc = P.mnc[i];
-    const float* gam = pool.GAM + (size_t)n * pool.EC + mc.goff;
-    const int e1 = mc.e;
-    int e = threadIdx.x;
-    for (; e + 3 * GP_THREADS < e1; e += 4 * GP_THREADS) {
-      float g[4], p[4];
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  for (int a = threadIdx.x >> 5; a < s_cnt; a += GP_THREADS / 32) {
+    const int f = s_f[a];
+    const int i = layer_of(net, f);
+    const MncCsr& mc = s_mc[i];
+    const int j = f - net.off[i];
+    const float* g = gam + mc.goff;
+    const int q0 = mc.cptr[j], q1 = mc.cptr[j + 1];
+    float gp = 0.f, gph = 0.f;
+    for (int q = q0 + lane; q < q1; q += 32 * 4) {
+      int ce[4];
+      float gv[4], cp[4], cph[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        g[u] = gam[e + u * GP_THREADS];
-        p[u] = mc.p[e + u * GP_THREADS];
+      for (int k = 0; k < 4; ++k) {
+        const bool in = q + 32 * k < q1;
+        ce[k] = in ? mc.ce[q + 32 * k] : 0;
+        cp[k] = in ? mc.cP[q + 32 * k] : 0.f;
+        cph[k] = in ? mc.cPh[q + 32 * k] : 0.f;
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) acc[u] = fmaf(g[u], p[u], acc[u]);
-    }
+      for (int k = 0; k < 4; ++k) gv[k] = q + 32 * k < q1 ? g[ce[k]] : 0.f;
 #pragma unroll
-    for (int u = 0; u < 3; ++u, e += GP_THREADS)
-      if (e < e1) acc[u] = fmaf(gam[e], mc.p[e], acc[u]);
+      for (int k = 0; k < 4; ++k) {
+        gp = fmaf(gv[k], cp[k], gp);
+        gph = fmaf(gv[k], cph[k], gph);
+      }
+    }
+    for (int o = 16; o; o >>= 1) {
+      gp += __shfl_xor_sync(0xffffffffu, gp, o);
+      gph += __shfl_xor_sync(0xffffffffu, gph, o);
+    }
+    if (lane == 0) {
+      GP[(size_t)m * net.SD + f] = gp;
+      GPh[(size_t)m * net.SD + f] = gph;
+    }
   }
-  const float tot = block_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
-  if (threadIdx.x == 0) gp0[m] = tot;
 }
 
+// Neurons per CTA: 32 spreads the few hundred neurons of a small network over
+// several CTAs a row (its listed neurons are dense), 256 keeps the CTAs of a
+// large one few (most of its neurons have no entries).
 void launch_gamma_proj(int M, const int* row_node, PoolDev pool, const PropDev* props,
                        const NetDev& net, float* GP, float* GPh, float* gp0, cudaStream_t st) {
   if (M <= 0) return;
-  dim3 grid((net.SD + 255) / 256, M);
-  k_gamma_proj<<<grid, 256, 0, st>>>(M, row_node, pool, props, net, GP, GPh);
-  k_gamma_p<<<M, GP_THREADS, 0, st>>>(M, row_node, pool, props, net, gp0);
+  const int npb = net.SD >= 8192 ? GP_THREADS : 32;
+  dim3 grid(GP_SPLIT + (net.SD + npb - 1) / npb, M);
+  k_gamma_proj<<<grid, GP_THREADS, 0, st>>>(M, row_node, pool, props, net, npb, GP, GPh, gp0);
 }
 
 // d lb / d gamma_e = sum_k P_ek (d lb / d a')_idx + Phat_ek (d lb / d ahat)_idx - p_e.
@@ -1891,62 +1913,79 @@ __device__ __forceinline__ void adam1(float& th, float& mo, float& ve, float g, 
   th = th + lr * mh / (sqrtf(vh) + eps);
 }
 
-// largest |gradient component| of each row over alpha, beta and gamma
-__global__ void k_grad_max(int SD, int EC, const int* row_node, const PoolDev pool,
-                           const PropDev* props, const float* GA, const float* GB,
-                           const float* GG, float* gmax) {
-  const int m = blockIdx.x;
+// largest |gradient component| of each row over alpha, beta and gamma: CTA s of
+// a row covers elements s, s + gridDim.x, ... of 4 * 256-element tiles and writes
+// gmax[m][s].  One CTA per row read the 260k components of the 3x32x32 network
+// with 135k constraint rows at 0.2 TB/s (362 us for 64 rows).
+__global__ void __launch_bounds__(256) k_grad_max(int SD, int EC, const int* row_node,
+                                                  const PoolDev pool, const PropDev* props,
+                                                  const float* GA, const float* GB,
+                                                  const float* GG, float* gmax) {
+  const int m = blockIdx.y;
   const int E = props[pool.prop[row_node[m]]].E;
+  const float* src[3] = {GA + (size_t)m * SD, GB + (size_t)m * SD, GG + (size_t)m * EC};
+  const int len[3] = {SD, SD, E};
   float mx = 0.f;
-  for (int i = threadIdx.x; i < SD; i += blockDim.x)
-    mx = fmaxf(mx, fmaxf(fabsf(GA[(size_t)m * SD + i]), fabsf(GB[(size_t)m * SD + i])));
-  for (int e = threadIdx.x; e < E; e += blockDim.x) mx = fmaxf(mx, fabsf(GG[(size_t)m * EC + e]));
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    for (int i = blockIdx.x * 1024 + threadIdx.x; i < len[k]; i += gridDim.x * 1024) {
+      float v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = i + 256 * u < len[k] ? src[k][i + 256 * u] : 0.f;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) mx = fmaxf(mx, fabsf(v[u]));
+    }
   for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  __shared__ float sh[32];
+  __shared__ float sh[8];
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
-    float r = 0.f;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) r = fmaxf(r, sh[i]);
-    gmax[m] = r;
+    float r = sh[0];
+    for (int i = 1; i < 8; ++i) r = fmaxf(r, sh[i]);
+    gmax[(size_t)m * GMAX_SPLIT + blockIdx.x] = r;
   }
 }
 
 // The alpha of a neuron that is not unstable and unsplit, and the beta of an
 // unsplit one, have a zero gradient at every step of an optimisation (its
 // bounds and splits are fixed), and their moments start at zero: their
-// updates are identities and are skipped.  gmax is read only when the
-// dead-zone or the gradient-scaled eps is on (use_gmax).
-__global__ void k_adam(int M, const int* __restrict__ row_node, PoolDev pool,
-                       const PropDev* __restrict__ props, int SD, const float* __restrict__ GA,
-                       const float* __restrict__ GB, const float* __restrict__ GG,
-                       const float* __restrict__ gmax, int use_gmax, float floor, float lr_a,
-                       float lr_b, float lr_g, float b1, float b2, float eps_abs, float eps_rel,
-                       float bc1, float bc2) {
+// updates are identities and are skipped.  A thread takes one neuron (its alpha
+// or its beta, by its split) or one multi-neuron multiplier.  gmax (nsplit
+// shares a row) is read only when the dead-zone or the gradient-scaled eps is on.
+__global__ void __launch_bounds__(256) k_adam(
+    int M, const int* __restrict__ row_node, PoolDev pool, const PropDev* __restrict__ props,
+    int SD, const float* __restrict__ GA, const float* __restrict__ GB,
+    const float* __restrict__ GG, const float* __restrict__ gmax, int nsplit, float floor,
+    float lr_a, float lr_b, float lr_g, float b1, float b2, float eps_abs, float eps_rel,
+    float bc1, float bc2) {
   const int m = blockIdx.y;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   const int n = row_node[m];
-  const float gm = use_gmax ? gmax[m] : 0.f;
+  float gm = 0.f;
+  if (nsplit) {
+    const int lane = threadIdx.x & 31;
+    if (lane < nsplit) gm = gmax[(size_t)m * GMAX_SPLIT + lane];
+    for (int o = 16; o; o >>= 1) gm = fmaxf(gm, __shfl_xor_sync(0xffffffffu, gm, o));
+  }
   const float thr = floor * gm;
   const float eps = fmaxf(eps_abs, eps_rel * gm);
   auto dz = [thr](float g) { return fabsf(g) <= thr ? 0.f : g; };
   if (idx < SD) {
     const size_t q = (size_t)n * SD + idx;
-    if (pool.S[q] != 0 || !(pool.L[q] < 0.f) || !(pool.U[q] > 0.f)) return;
-    float th = pool.ALPHA[q], mo = pool.MA[q], ve = pool.VA[q];
-    adam1(th, mo, ve, dz(GA[(size_t)m * SD + idx]), lr_a, b1, b2, eps, bc1, bc2);
-    pool.ALPHA[q] = fminf(fmaxf(th, 0.f), 1.f);
-    pool.MA[q] = mo; pool.VA[q] = ve;
-  } else if (idx < 2 * SD) {
-    const int f = idx - SD;
-    const size_t q = (size_t)n * SD + f;
-    if (pool.S[q] == 0) return;
-    float th = pool.BETA[q], mo = pool.MB[q], ve = pool.VB[q];
-    adam1(th, mo, ve, dz(GB[(size_t)m * SD + f]), lr_b, b1, b2, eps, bc1, bc2);
-    pool.BETA[q] = fmaxf(th, 0.f);
-    pool.MB[q] = mo; pool.VB[q] = ve;
+    if (pool.S[q] == 0) {
+      if (!(pool.L[q] < 0.f) || !(pool.U[q] > 0.f)) return;
+      float th = pool.ALPHA[q], mo = pool.MA[q], ve = pool.VA[q];
+      adam1(th, mo, ve, dz(GA[(size_t)m * SD + idx]), lr_a, b1, b2, eps, bc1, bc2);
+      pool.ALPHA[q] = fminf(fmaxf(th, 0.f), 1.f);
+      pool.MA[q] = mo; pool.VA[q] = ve;
+    } else {
+      float th = pool.BETA[q], mo = pool.MB[q], ve = pool.VB[q];
+      adam1(th, mo, ve, dz(GB[(size_t)m * SD + idx]), lr_b, b1, b2, eps, bc1, bc2);
+      pool.BETA[q] = fmaxf(th, 0.f);
+      pool.MB[q] = mo; pool.VB[q] = ve;
+    }
   } else {
-    const int e = idx - 2 * SD;
+    const int e = idx - SD;
     if (e >= props[pool.prop[n]].E) return;
     const size_t q = (size_t)n * pool.EC + e;
     float th = pool.GAM[q], mo = pool.MG[q], ve = pool.VG[q];
@@ -1961,12 +2000,15 @@ void launch_adam(int M, const int* row_node, PoolDev pool, const PropDev* props,
                  float lr_a, float lr_b, float lr_g, float b1, float b2, float eps, float eps_rel,
                  float bc1, float bc2, cudaStream_t st) {
   if (M <= 0) return;
-  const int use_gmax = (floor != 0.f || eps_rel != 0.f) ? 1 : 0;
-  if (use_gmax)
-    k_grad_max<<<M, 256, 0, st>>>(SD, pool.EC, row_node, pool, props, GA, GB, GG, gmax);
-  const int tot = 2 * SD + pool.EC;
+  int nsplit = 0;
+  if (floor != 0.f || eps_rel != 0.f) {
+    nsplit = std::min(GMAX_SPLIT, (std::max(SD, pool.EC) + 1023) / 1024);
+    k_grad_max<<<dim3(nsplit, M), 256, 0, st>>>(SD, pool.EC, row_node, pool, props, GA, GB, GG,
+                                                gmax);
+  }
+  const int tot = SD + pool.EC;
   dim3 grid((tot + 255) / 256, M);
-  k_adam<<<grid, 256, 0, st>>>(M, row_node, pool, props, SD, GA, GB, GG, gmax, use_gmax, floor,
+  k_adam<<<grid, 256, 0, st>>>(M, row_node, pool, props, SD, GA, GB, GG, gmax, nsplit, floor,
                                lr_a, lr_b, lr_g, b1, b2, eps, eps_rel, bc1, bc2);
 }
 

@@ -269,8 +269,12 @@ bool conv_supported(const LayerDev& L);
 // Forward through affine layer i (+ bias): in [M][d_{i-1}] -> out [M][d_i].
 void launch_forward(const LayerDev& L, int M, const float* in, int ld_in, float* out, int ld_out,
                     const Epi& e, cudaStream_t st);
-// lb[m] = sum of partial slots - gp0[m]; with track, keep the best bound and
-// its minimiser per node.
+// Shares per row of gamma^T p (gp0 [M][GP_SPLIT]) and of the largest gradient
+// component (gmax [M][GMAX_SPLIT], at most a warp's width).
+constexpr int GP_SPLIT = 16;
+constexpr int GMAX_SPLIT = 32;
+// lb[m] = sum of partial slots - sum of gp0[m][:]; with track, keep the best
+// bound and its minimiser per node.
 void launch_reduce_lb(int M, const float* part, int nslot, int used, const float* gp0,
                       float* lb, bool track, const int* row_node, PoolDev pool, const float* X,
                       int d0, cudaStream_t st);

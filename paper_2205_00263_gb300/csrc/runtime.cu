@@ -912,7 +912,7 @@ void run_optimize_body(mnbab_net* n, int M, bool has_gamma, const mnbab_adam& a,
   double b1t = 1.0, b2t = 1.0;
   for (int step = 0; step <= a.steps; ++step) {
     if (has_gamma) {
-      Scope sc(c, C_GAMMA, 0.0, 4.0 * M * (c->EC + 2.0 * n->SD), 2);
+      Scope sc(c, C_GAMMA, 0.0, 4.0 * M * (c->EC + 2.0 * n->SD));
       launch_gamma_proj(M, n->bslots, n->pool, c->d_props, n->nd, n->GP, n->GPh, n->gp0, c->st);
     }
     sweep(n, n->R + 1, obj_rows(n, M), o);
@@ -1068,7 +1068,7 @@ void leaf_complete(mnbab_net* n, const std::vector<int>& slots, int steps, const
   int cnt = 0;
   for (int step = 0; step <= steps; ++step) {
     if (g) {
-      Scope sc(c, C_GAMMA, 0.0, 4.0 * M * (c->EC + 2.0 * n->SD), 2);
+      Scope sc(c, C_GAMMA, 0.0, 4.0 * M * (c->EC + 2.0 * n->SD));
       launch_gamma_proj(M, n->bslots, n->pool, c->d_props, n->nd, n->GP, n->GPh, n->gp0, c->st);
     }
     sweep(n, n->R + 1, obj_rows(n, M), o);  // x* of this iterate in n->X
@@ -1196,11 +1196,11 @@ void setup_net(mnbab_ctx* c, mnbab_net* n) {
   n->X = dalloc_t<float>(c, mrows * n->d0);
   n->Xb = dalloc_t<float>(c, B * n->d0);
   n->GG = dalloc_t<float>(c, B * std::max<size_t>(EC, 1));
-  n->gp0 = dalloc_t<float>(c, B);
+  n->gp0 = dalloc_t<float>(c, B * GP_SPLIT);
   n->fout = dalloc_t<float>(c, B);
   n->score = dalloc_t<float>(c, B);
   n->bestb = dalloc_t<float>(c, B);
-  n->gmax = dalloc_t<float>(c, B);
+  n->gmax = dalloc_t<float>(c, B * GMAX_SPLIT);
   n->f64a = dalloc_t<double>(c, B * (size_t)(n->d0 + n->SD));
   n->f64out = dalloc_t<double>(c, B);
   n->cslots = dalloc_t<int>(c, B);
@@ -1812,7 +1812,7 @@ int64_t optimize_intermediate_impl(mnbab_net* n, const std::vector<int>& slots, 
         RowsDev r{Mc, n->row_node + c0, n->row_j + c0, n->row_sign + c0};
         if (has_g) {
           // gamma^T P, gamma^T Phat, gamma^T p of each row's set
-          Scope sc(c, C_GAMMA, 0.0, 4.0 * Mc * (c->EC + 2.0 * n->SD), 2);
+          Scope sc(c, C_GAMMA, 0.0, 4.0 * Mc * (c->EC + 2.0 * n->SD));
           launch_gamma_proj(Mc, r.node, n->pool, c->d_props, n->nd, n->GP, n->GPh, n->gp0, c->st);
         }
         sweep(n, t, r, o);
@@ -2940,7 +2940,7 @@ mnbab_status mnbab_bound_batch(mnbab_ctx* c, const mnbab_node_id* nodes, int32_t
   upload_batch(n, slots);
   const bool g = batch_has_gamma(n, slots);
   if (g) {
-    Scope sc(c, C_GAMMA, 0.0, 4.0 * nn * (c->EC + 2.0 * n->SD), 2);
+    Scope sc(c, C_GAMMA, 0.0, 4.0 * nn * (c->EC + 2.0 * n->SD));
     launch_gamma_proj(nn, n->bslots, n->pool, c->d_props, n->nd, n->GP, n->GPh, n->gp0, c->st);
   }
   SweepOpts o;
@@ -3002,7 +3002,7 @@ mnbab_status mnbab_bound_grad(mnbab_ctx* c, const mnbab_node_id* nodes, int32_t 
   upload_batch(n, slots);
   const bool g = batch_has_gamma(n, slots);
   if (g) {
-    Scope sc(c, C_GAMMA, 0.0, 4.0 * nn * (c->EC + 2.0 * n->SD), 2);
+    Scope sc(c, C_GAMMA, 0.0, 4.0 * nn * (c->EC + 2.0 * n->SD));
     launch_gamma_proj(nn, n->bslots, n->pool, c->d_props, n->nd, n->GP, n->GPh, n->gp0, c->st);
   }
   SweepOpts o;
@@ -3087,7 +3087,7 @@ mnbab_status mnbab_score_branches(mnbab_ctx* c, const mnbab_node_id* nodes, int3
   upload_batch(n, slots);
   const bool g = batch_has_gamma(n, slots);
   if (g) {
-    Scope sc(c, C_GAMMA, 0.0, 4.0 * nn * (c->EC + 2.0 * n->SD), 2);
+    Scope sc(c, C_GAMMA, 0.0, 4.0 * nn * (c->EC + 2.0 * n->SD));
     launch_gamma_proj(nn, n->bslots, n->pool, c->d_props, n->nd, n->GP, n->GPh, n->gp0, c->st);
   }
   SweepOpts o;

@@ -1,0 +1,97 @@
+"""Kernels at the edges of their tiles and splits, against the FP64 oracle.
+
+Tolerance of bounds and gradients as in test_gpu_parity: 1e-4 (1 + |oracle|),
+gradients relative to the largest component.
+"""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from helpers import TOL, close, concat, random_node, to_params
+from oracle import bab, core
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def Context():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2205_00263_gb300 import Context
+    return Context
+
+
+def _case(spec, eps, mnc_fn=None):
+    layers = synth.make_network(spec)
+    x0 = synth.make_image(spec["seed"] + 7, spec["in_shape"]).reshape(-1)
+    y = synth.net_forward(layers, x0)
+    C, d = synth.property_rows(int(np.argmax(y)), y.shape[0])
+    lo, hi = synth.input_box(x0, eps)
+    return layers, C, d, lo, hi, bab.prepare(layers, C, d, lo, hi, mnc_fn)
+
+
+def _rows_per_neuron(seed, counts, k):
+    """Constraints over k neurons each in which the first neurons of every layer
+    occur counts[0], counts[1], ... times (up to the layer's width)."""
+    def fn(net, l, u, lo, hi):
+        rng = np.random.default_rng(seed)
+        out = {}
+        for t in l:
+            d = l[t].numel()
+            first = np.repeat(np.arange(min(d, len(counts))), counts[:d])
+            idx = np.stack([first] + [rng.integers(0, d, first.size) for _ in range(k - 1)], 1)
+            P, Ph = (rng.normal(0, 0.1, idx.shape).astype(np.float32) for _ in range(2))
+            p = rng.uniform(0.0, 0.2, first.size).astype(np.float32)
+            out[t] = core.MNC(idx, P, Ph, p)
+        return out
+    return fn
+
+
+# gamma terms: neurons with no entry, around a warp's width and around a warp's
+# four loads in flight, in a network of a few neurons per CTA and in one of more
+# than 8192 neurons (256 per CTA, a ragged last one); rows over 2 and 3 neurons
+@pytest.mark.parametrize("spec,k", [
+    (dict(seed=31, in_shape=(12,), layers=[("fc", 33), ("relu",), ("fc", 9), ("relu",), ("fc", 3)]), 3),
+    (dict(seed=32, in_shape=(1, 33, 33), layers=[("conv", 8, 3, 1, 1), ("relu",), ("fc", 17), ("relu",),
+                                                 ("fc", 3)]), 2),
+])
+def test_gamma_terms(Context, spec, k):
+    counts = [0, 1, 31, 32, 33, 127, 128, 129, 300, 0, 5]
+    if len(spec["in_shape"]) == 1:
+        layers = synth.tiny_fc_net(spec["seed"], [12, 33, 9, 3])
+        lo, hi = synth.input_box(np.random.default_rng(1).uniform(0.2, 0.8, 12), 0.1)
+        C, d = synth.property_rows(0, 3)
+        prep = bab.prepare(layers, C, d, lo, hi, _rows_per_neuron(5, counts, k))
+    else:
+        layers, C, d, lo, hi, prep = _case(spec, 0.02, _rows_per_neuron(5, counts, k))
+    net, lo_t, hi_t, l, u, S, m, dense = prep
+    E = sum(v.idx.shape[0] for v in m.values())
+    SD = sum(l[i].numel() for i in l)
+    rng = np.random.default_rng(9)
+    with Context(node_capacity=64, max_mnc_rows=E + 3) as ctx:
+        gnet = ctx.load_network(layers)
+        prop = ctx.set_property(gnet, lo, hi, C, d)
+        for i in sorted(m):
+            ctx.set_mnc(prop, i, m[i].idx, m[i].P, m[i].Ph, m[i].p)
+        nodes = [random_node(prep, rng, n_splits=j, row=j % 2) for j in range(3)]
+        gids = []
+        for on in nodes:
+            on.split_layer = net.R
+            gids.append(ctx.node_root(prop, on.row))
+            ctx.import_params(gids[-1], to_params(on, net.R))
+        lb, ga, gb, gg = ctx.bound_grad(gids, SD, E)
+        best = ctx.optimize(gids, steps=1, eps_rel=1e-3)
+        for j, on in enumerate(nodes):
+            ref, _, oa, ob, og = core.bound_and_grad(net, on, on.alpha, on.beta, on.gamma, dense,
+                                                     lo_t, hi_t)
+            assert close(lb[j], float(ref)).all()
+            o = np.concatenate([concat(oa, net.R), concat(ob, net.R),
+                                *(og[i].numpy() for i in sorted(og))])
+            g = np.concatenate([ga[j], gb[j], gg[j]])
+            assert np.abs(g - o).max() <= TOL * (1 + np.abs(o).max())
+            top, *_ = core.optimize(net, on, dense, lo_t, hi_t, core.AdamHP(steps=1, eps_rel=1e-3))
+            assert close(best[j], top).all()
+
