@@ -229,7 +229,8 @@ void launch_first_rows(const NetDev& net, const PoolDev& pool, const PropDev* pr
 // window with origin (y0 s - p, x0 s - p); relative output position yy takes
 // input position Y = (yy - kh) / s wherever that is an integer in [0, h).
 // Positions outside the layer (padding) carry no coefficient.
-constexpr int WIN_MAX_FLOATS = 12288;  // per buffer: two buffers = 96 KB
+constexpr int WIN_MAX_FLOATS = 12288;  // per buffer of one row
+constexpr int WIN_RB_MAX = 8;
 
 bool win_plan(const NetDev& net, int t, WinPlan& wp) {
   if (t < 2 || t > net.R) return false;  // rows at layer 1 are direct in k_init_rows
@@ -249,225 +250,335 @@ bool win_plan(const NetDev& net, int t, WinPlan& wp) {
     wp.w[i - 1] = w;
     mx = std::max(mx, L.ci * h * w);
   }
-  wp.maxw = mx;
-  return mx <= WIN_MAX_FLOATS;
+  if (mx > WIN_MAX_FLOATS) return false;
+  // planes of the two buffers (16-byte multiples) and the padded weights
+  wp.plane[0] = wp.plane[1] = wp.wpad = 0;
+  for (int i = t - 1; i >= 0; --i) {
+    const int n = (net.aff[i + 1].ci * wp.h[i] * wp.w[i] + 3) / 4 * 4, side = (t - 1 - i) & 1;
+    wp.plane[side] = std::max(wp.plane[side], n);
+    if (i >= 1 && (net.aff[i].ci == 2 || net.aff[i].ci == 3))
+      wp.wpad += net.aff[i].co * net.aff[i].k * net.aff[i].k * 4;
+  }
+  // rows per CTA: 8 where two CTAs still fit on an SM, else 4 or 1
+  auto bytes = [&](int rb) { return (rb * (wp.plane[0] + wp.plane[1]) + wp.wpad) * 4; };
+  wp.rb = bytes(WIN_RB_MAX) <= 112 * 1024 ? WIN_RB_MAX : bytes(4) <= 224 * 1024 ? 4 : 1;
+  return bytes(wp.rb) <= 224 * 1024;
 }
 
-__global__ void k_win_rows(NetDev net, WinPlan wp, RowsDev rows, Epi e) {
+// x / d for the small operands of window indices (x d < 2^32), by the rounded-up
+// reciprocal `magic` = ceil(2^32 / d) (0 stands for d = 1)
+__device__ __forceinline__ unsigned win_magic(int d) {
+  return d == 1 ? 0u : 0xffffffffu / (unsigned)d + 1u;
+}
+__device__ __forceinline__ int win_div(int x, unsigned magic) {
+  return magic ? (int)__umulhi((unsigned)x, magic) : x;
+}
+
+// two FP32 FMAs in one instruction, each rounded as fmaf
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(r)
+      : "l"(*reinterpret_cast<unsigned long long*>(&a)),
+        "l"(*reinterpret_cast<unsigned long long*>(&b)),
+        "l"(*reinterpret_cast<unsigned long long*>(&c)));
+  return *reinterpret_cast<float2*>(&r);
+}
+
+struct WinRow {
+  int y0, x0;  // window origin at the current layer
+};
+
+// Output positions are enumerated phase-major (ih mod s, iw mod s) so that the
+// threads of a warp share kernel taps, and with them their weight loads.
+__device__ __forceinline__ void decode_phase(int pidx, int hi, int wi, int s, int& ih, int& iw) {
+  for (int ph = 0; ph < s; ++ph) {
+    const int nh = (hi - ph + s - 1) / s;
+    for (int pw = 0; pw < s; ++pw) {
+      const int nw = (wi - pw + s - 1) / s;
+      const int cnt = nh * nw;
+      if (pidx < cnt) {
+        ih = ph + s * (pidx / nw);
+        iw = pw + s * (pidx % nw);
+        return;
+      }
+      pidx -= cnt;
+    }
+  }
+  ih = iw = -1;
+}
+
+// Transposed convolution of the CTA's row windows, A (h x w) to B (h2 x w2),
+// both [channel][position][RB rows].  An item is one output position x CB
+// channels x four rows: a 16-byte load brings a coefficient of the four rows,
+// and its CB weights serve all of them, so three loads feed 32 FMAs (CB = 8).
+// Where the items leave threads idle, 2 or 4 adjacent lanes split an item's
+// reduction.  SM: the weights are in shared memory, else in global memory.
+template <int THREADS, int RG, int CB, bool SM>
+__device__ __forceinline__ void win_conv(const LayerDev& L, const float* __restrict__ Wt, int wci,
+                                         const float* A, float* B, int RB, int h, int w,
+                                         const WinRow* rows) {
+  const int s = L.s, k = L.k, h2 = (h - 1) * s + k, w2 = (w - 1) * s + k;
+  const int hw = h * w, hw2 = h2 * w2;
+  const int items = hw2 * (RB / RG) * ((L.ci + CB - 1) / CB);
+  int ks = 1;
+  while (ks < 4 && items * ks * 2 <= THREADS) ks *= 2;
+  const int wco = k * k * wci;
+  for (int b0 = 0; b0 < items * ks; b0 += THREADS) {
+    const int id = b0 + threadIdx.x, it = id / ks, k0 = id % ks;
+    const bool act = it < items;
+    const int px = it % hw2, rg = it / hw2 % (RB / RG) * RG, grp = it / (hw2 * (RB / RG));
+    constexpr int R2 = RG == 4 ? 2 : 1;
+    float2 acc[CB][R2];
+#pragma unroll
+    for (int c = 0; c < CB; ++c)
+#pragma unroll
+      for (int r = 0; r < R2; ++r) acc[c][r] = make_float2(0.f, 0.f);
+    int yy = 0, xx = 0;
+    if (act) {
+      decode_phase(px, h2, w2, s, yy, xx);
+      for (int kh = yy % s, Y = yy / s; kh < k && Y >= 0; kh += s, --Y) {
+        if (Y >= h) continue;
+        for (int kw = xx % s, X = xx / s; kw < k && X >= 0; kw += s, --X) {
+          if (X >= w) continue;
+          const float* ap = A + (size_t)(k0 * hw + Y * w + X) * RB + rg;
+          const float* wp = Wt + (size_t)k0 * wco + (kh * k + kw) * wci + grp * CB;
+#pragma unroll 4
+          for (int o = k0; o < L.co; o += ks, ap += ks * hw * RB, wp += ks * wco) {
+            float2 v[R2];
+            if (RG == 4) {
+              const float4 v4 = *reinterpret_cast<const float4*>(ap);
+              v[0] = make_float2(v4.x, v4.y);
+              v[R2 - 1] = make_float2(v4.z, v4.w);
+            } else {
+              v[0] = make_float2(*ap, 0.f);
+            }
+            float wv[CB];
+            if (CB >= 4) {
+#pragma unroll
+              for (int c = 0; c < CB; c += 4) {
+                const float4* w4p = reinterpret_cast<const float4*>(wp + c);
+                const float4 w4 = SM ? *w4p : __ldg(w4p);
+                wv[c] = w4.x;
+                wv[c + 1 < CB ? c + 1 : c] = w4.y;
+                wv[c + 2 < CB ? c + 2 : c] = w4.z;
+                wv[c + 3 < CB ? c + 3 : c] = w4.w;
+              }
+            } else {
+              wv[0] = SM ? wp[0] : __ldg(wp);
+            }
+#pragma unroll
+            for (int c = 0; c < CB; ++c) {
+              if (RG == 4) {
+                const float2 ww = make_float2(wv[c], wv[c]);
+                acc[c][0] = fma2(v[0], ww, acc[c][0]);
+                acc[c][R2 - 1] = fma2(v[R2 - 1], ww, acc[c][R2 - 1]);
+              } else {
+                acc[c][0].x = fmaf(v[0].x, wv[c], acc[c][0].x);
+              }
+            }
+          }
+        }
+      }
+    }
+    for (int o = ks >> 1; o; o >>= 1)
+#pragma unroll
+      for (int c = 0; c < CB; ++c)
+#pragma unroll
+        for (int r = 0; r < R2; ++r) {
+          acc[c][r].x += __shfl_xor_sync(0xffffffffu, acc[c][r].x, o);
+          if (RG == 4) acc[c][r].y += __shfl_xor_sync(0xffffffffu, acc[c][r].y, o);
+        }
+    if (!act || k0) continue;
+    // positions outside the layer (padding) carry no coefficient
+    bool in[RG];
+#pragma unroll
+    for (int r = 0; r < RG; ++r) {
+      const int y = rows[rg + r].y0 * s - L.p + yy, x = rows[rg + r].x0 * s - L.p + xx;
+      in[r] = y >= 0 && y < L.hi && x >= 0 && x < L.wi;
+    }
+    float* bp = B + (size_t)(grp * CB * hw2 + yy * w2 + xx) * RB + rg;
+#pragma unroll
+    for (int c = 0; c < CB; ++c)
+      if (CB < 4 || grp * CB + c < L.ci) {
+        if constexpr (RG == 4)
+          *reinterpret_cast<float4*>(bp + (size_t)c * hw2 * RB) =
+              make_float4(in[0] ? acc[c][0].x : 0.f, in[1] ? acc[c][0].y : 0.f,
+                          in[2] ? acc[c][1].x : 0.f, in[3] ? acc[c][1].y : 0.f);
+        else
+          bp[c * hw2] = in[0] ? acc[c][0].x : 0.f;
+      }
+  }
+}
+
+// RB = 8, 4 or (windows beyond 56 KB a row) 1 rows per CTA, their windows in shared memory with the rows of a
+// position adjacent.  Bound by the latency of the weight and bound loads (FMA
+// pipe 34% busy) and FP32 FMAs: on the 3x32x32 network's layers 3 and 4 (32768
+// and 8192 rows, 31 GFLOP) 1.1 and 2.3 ms; a thread per output element of one
+// row took 16.3 ms together.  Four columns of one row per thread instead of four
+// rows took 1.2 and 2.4 ms, but 149 against 101 us for the 25600 rows of 16
+// 1x28x28 properties (112 us before): its columns are ragged in small windows.
+// WIDE: some layer of the chain has several input channels to a thread; without
+// one (a one-channel image below a single convolution) smaller CTAs of fewer
+// registers hide the latency of its short steps.
+template <bool WIDE, int RG>
+__global__ void __launch_bounds__(WIDE ? 512 : 256, WIDE ? 2 : 6)
+    k_win_rows(NetDev net, WinPlan wp, RowsDev rows, Epi e, float* __restrict__ lb) {
+  constexpr int THREADS = WIDE ? 512 : 256;
   extern __shared__ __align__(16) float wsm[];
-  float* A = wsm;
-  float* B = wsm + wp.maxw;
-  const int m = blockIdx.x;
-  const int t = wp.t;
-  const int j = rows.j[m];
-  const float sg = rows.sign ? rows.sign[m] : 1.f;
+  __shared__ WinRow s_row[WIN_RB_MAX];
+  __shared__ float s_sum[THREADS / 32][WIN_RB_MAX];
+  const int t = wp.t, RB = wp.rb, tpr = THREADS / RB;
   const LayerDev& Lt = net.aff[t];
+  // buffers of the layers t - 1, t - 3, ... and t - 2, t - 4, ...; then the
+  // padded weights of layers with 2 or 3 input channels
+  float* buf[2] = {wsm, wsm + RB * wp.plane[0]};
+  float* wpad = wsm + RB * (wp.plane[0] + wp.plane[1]);
+  if (WIDE) {
+    float* d = wpad;
+    for (int i = 1; i < t; ++i) {
+      const LayerDev& L = net.aff[i];
+      if (L.ci != 2 && L.ci != 3) continue;
+      const int n = L.co * L.k * L.k * 4;
+      for (int q = threadIdx.x; q < n; q += THREADS)
+        d[q] = (q & 3) < L.ci ? __ldg(L.Wb + (q >> 2) * L.ci + (q & 3)) : 0.f;
+      d += n;
+    }
+  }
+  const int q = threadIdx.x % RB, tl = threadIdx.x / RB;
+  const int m = min(blockIdx.x * RB + q, rows.M - 1);  // absent rows repeat the last (dropped)
+  const int j = rows.j[m], node = rows.node[m];
+  const float sg = rows.sign ? rows.sign[m] : 1.f;
   const int hwt = Lt.ho * Lt.wo;
   const int co = j / hwt, oh = (j % hwt) / Lt.wo, ow = j % Lt.wo;
   int y0 = oh * Lt.s - Lt.p, x0 = ow * Lt.s - Lt.p;
+  if (tl == 0) s_row[q] = WinRow{y0, x0};
   {
     const int n0 = Lt.ci * Lt.k * Lt.k;
-    for (int q = threadIdx.x; q < n0; q += blockDim.x) A[q] = sg * __ldg(Lt.W + (size_t)co * n0 + q);
+    for (int i = tl; i < n0; i += tpr) buf[0][i * RB + q] = sg * __ldg(Lt.W + (size_t)co * n0 + i);
   }
-  const float c0 = sg * (net.bfull[t] ? net.bfull[t][j] : Lt.b[co]);
+  const PropDev& P = e.props[e.pool.prop[node]];
   float part = 0.f;
   int h = Lt.k, w = Lt.k;
-  for (int i = t - 1; i >= 0; --i) {
+  for (int i = t - 1, side = 0; i >= 0; --i, side ^= 1) {
     const LayerDev& Ln = net.aff[i + 1];  // layer i is this edge's input
-    const int C = Ln.ci, H = Ln.hi, W = Ln.wi, hw = h * w;
+    const int C = Ln.ci, H = Ln.hi, W = Ln.wi, hw = h * w, n = C * hw;
+    const unsigned mhw = win_magic(hw), mw = win_magic(w);
+    float* A = buf[side] + q;
     __syncthreads();
     if (i == 0) {
       // concretisation over the input box
-      const PropDev& P = e.props[e.pool.prop[rows.node[m]]];
-      for (int q = threadIdx.x; q < C * hw; q += blockDim.x) {
-        const int c = q / hw, r = q % hw, y = y0 + r / w, x = x0 + r % w;
+      for (int r0 = tl; r0 < n; r0 += tpr) {
+        const int c = win_div(r0, mhw), r = r0 - c * hw, yr = win_div(r, mw);
+        const int y = y0 + yr, x = x0 + r - yr * w;
         if (y < 0 || y >= H || x < 0 || x >= W) continue;
         const int jx = (c * H + y) * W + x;
-        const float a = A[q];
+        const float a = A[r0 * RB];
         part += a * (a >= 0.f ? P.lo[jx] : P.hi[jx]);
       }
       break;
     }
-    // ReLU step of layer i (DeepPoly slopes, splits enforced)
-    Epi el = e;
-    el.kind = EPI_RELU;
-    el.off = net.off[i];
-    el.bias = net.bfull[i];
-    el.bias_div = 1;
-    for (int q = threadIdx.x; q < C * hw; q += blockDim.x) {
-      const int c = q / hw, r = q % hw, y = y0 + r / w, x = x0 + r % w;
-      if (y < 0 || y >= H || x < 0 || x >= W) {
-        A[q] = 0.f;
-        continue;
+    // ReLU step of layer i (DeepPoly slopes, splits enforced); the bounds of
+    // four elements are loaded before the first is used
+    const size_t nb = (size_t)node * e.SD + net.off[i];
+    const float* bias = net.bfull[i];
+    for (int r0 = tl; r0 < n; r0 += 4 * tpr) {
+      int jx[4];
+      float l[4], u[4], b[4];
+      int sp[4];
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int rr = r0 + v * tpr;
+        const int c = win_div(rr, mhw), r = rr - c * hw, yr = win_div(r, mw);
+        const int y = y0 + yr, x = x0 + r - yr * w;
+        jx[v] = rr < n && y >= 0 && y < H && x >= 0 && x < W ? (c * H + y) * W + x : -1;
+        l[v] = u[v] = b[v] = 0.f;
+        sp[v] = 0;
+        if (jx[v] >= 0) {
+          l[v] = e.pool.L[nb + jx[v]];
+          u[v] = e.pool.U[nb + jx[v]];
+          sp[v] = e.pool.S[nb + jx[v]];
+          b[v] = bias[jx[v]];
+        }
       }
-      A[q] = epi_relu(el, m, (c * H + y) * W + x, A[q], part);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int rr = r0 + v * tpr;
+        if (rr >= n) break;
+        if (jx[v] < 0) {
+          A[rr * RB] = 0.f;
+          continue;
+        }
+        const float a = A[rr * RB];
+        float D, bl = 0.f;
+        if (sp[v] == -1) D = 1.f;
+        else if (sp[v] == 1) D = 0.f;
+        else if (l[v] >= 0.f) D = 1.f;
+        else if (u[v] <= 0.f) D = 0.f;
+        else if (a >= 0.f) D = u[v] >= -l[v] ? 1.f : 0.f;
+        else {
+          const float den = u[v] - l[v];
+          D = u[v] / den;
+          bl = (-u[v] * l[v]) / den;
+        }
+        const float ah = a * D;
+        part += a * bl + ah * b[v];
+        A[rr * RB] = ah;
+      }
     }
     __syncthreads();
     // transposed convolution through layer i's edge
     const LayerDev& Li = net.aff[i];
-    const int s = Li.s, k = Li.k, kk = k * k;
-    const int h2 = (h - 1) * s + k, w2 = (w - 1) * s + k, hw2 = h2 * w2;
-    const int y2 = y0 * s - Li.p, x2 = x0 * s - Li.p;
-    const size_t wco = (size_t)Li.ci * kk;  // stride of W over output channels
-    for (int q = threadIdx.x; q < Li.ci * hw2; q += blockDim.x) {
-      const int c = q / hw2, r = q % hw2, yy = r / w2, xx = r % w2;
-      const int ya = y2 + yy, xa = x2 + xx;
-      float acc = 0.f;
-      if (ya >= 0 && ya < Li.hi && xa >= 0 && xa < Li.wi) {
-        for (int kh = yy % s; kh < k && kh <= yy; kh += s) {
-          const int Y = (yy - kh) / s;
-          if (Y >= h) continue;
-          for (int kw = xx % s; kw < k && kw <= xx; kw += s) {
-            const int X = (xx - kw) / s;
-            if (X >= w) continue;
-            const float* ap = A + Y * w + X;
-            const float* wp2 = Li.W + (size_t)c * kk + kh * k + kw;
-            for (int o = 0; o < Li.co; ++o) acc = fmaf(ap[o * hw], __ldg(wp2 + o * wco), acc);
-          }
-        }
-      }
-      B[q] = acc;
+    const float* in = buf[side];
+    float* out = buf[side ^ 1];
+    if (!WIDE) {
+      win_conv<THREADS, RG, 1, false>(Li, Li.Wb, Li.ci, in, out, RB, h, w, s_row);
+    } else if ((Li.ci & 7) == 0) {
+      win_conv<THREADS, RG, 8, false>(Li, Li.Wb, Li.ci, in, out, RB, h, w, s_row);
+    } else if ((Li.ci & 3) == 0) {
+      win_conv<THREADS, RG, 4, false>(Li, Li.Wb, Li.ci, in, out, RB, h, w, s_row);
+    } else if (Li.ci == 2 || Li.ci == 3) {
+      const float* wt = wpad;
+      for (int v = 1; v < i; ++v)
+        if (net.aff[v].ci == 2 || net.aff[v].ci == 3)
+          wt += net.aff[v].co * net.aff[v].k * net.aff[v].k * 4;
+      win_conv<THREADS, RG, 4, true>(Li, wt, 4, in, out, RB, h, w, s_row);
+    } else {
+      win_conv<THREADS, RG, 1, false>(Li, Li.Wb, Li.ci, in, out, RB, h, w, s_row);
     }
-    float* tmp = A;
-    A = B;
-    B = tmp;
-    h = h2;
-    w = w2;
-    y0 = y2;
-    x0 = x2;
-  }
-  const float tot = block_sum(part);
-  if (threadIdx.x == 0) e.part[(size_t)m * e.nslot + e.slot_base] = tot + c0;
-}
-
-// The same windowed rows, RB rows per CTA in lockstep (small windows): every
-// phase covers the RB rows' windows, so each barrier and index computation
-// serves RB rows; row q keeps its own window origin, node and partial sum.
-template <int RB>
-__global__ void k_win_rows_rb(NetDev net, WinPlan wp, RowsDev rows, Epi e) {
-  extern __shared__ __align__(16) float wsm[];
-  const int t = wp.t;
-  const LayerDev& Lt = net.aff[t];
-  const int m0 = blockIdx.x * RB;
-  float* A = wsm;                   // RB planes of wp.maxw
-  float* B = wsm + RB * wp.maxw;
-  int y0[RB], x0[RB], mq[RB];
-  float part[RB], c0[RB];
-  const int hwt = Lt.ho * Lt.wo;
-  const int n0 = Lt.ci * Lt.k * Lt.k;
-#pragma unroll
-  for (int q = 0; q < RB; ++q) {
-    const bool in = m0 + q < rows.M;
-    mq[q] = in ? m0 + q : m0;  // absent rows repeat the first (results dropped)
-    const int j = rows.j[mq[q]];
-    const float sg = rows.sign ? rows.sign[mq[q]] : 1.f;
-    const int co = j / hwt, oh = (j % hwt) / Lt.wo, ow = j % Lt.wo;
-    y0[q] = oh * Lt.s - Lt.p;
-    x0[q] = ow * Lt.s - Lt.p;
-    c0[q] = sg * (net.bfull[t] ? net.bfull[t][j] : Lt.b[co]);
-    part[q] = 0.f;
-    for (int i = threadIdx.x; i < n0; i += blockDim.x)
-      A[q * wp.maxw + i] = sg * __ldg(Lt.W + (size_t)co * n0 + i);
-  }
-  int h = Lt.k, w = Lt.k;
-  for (int i = t - 1; i >= 0; --i) {
-    const LayerDev& Ln = net.aff[i + 1];
-    const int C = Ln.ci, H = Ln.hi, W = Ln.wi, hw = h * w;
+    h = (h - 1) * Li.s + Li.k;
+    w = (w - 1) * Li.s + Li.k;
+    y0 = y0 * Li.s - Li.p;
+    x0 = x0 * Li.s - Li.p;
     __syncthreads();
-    if (i == 0) {
-#pragma unroll
-      for (int q = 0; q < RB; ++q) {
-        const PropDev& P = e.props[e.pool.prop[rows.node[mq[q]]]];
-        for (int r0 = threadIdx.x; r0 < C * hw; r0 += blockDim.x) {
-          const int c = r0 / hw, r = r0 % hw, y = y0[q] + r / w, x = x0[q] + r % w;
-          if (y < 0 || y >= H || x < 0 || x >= W) continue;
-          const int jx = (c * H + y) * W + x;
-          const float a = A[q * wp.maxw + r0];
-          part[q] += a * (a >= 0.f ? P.lo[jx] : P.hi[jx]);
-        }
-      }
-      break;
-    }
-    Epi el = e;
-    el.kind = EPI_RELU;
-    el.off = net.off[i];
-    el.bias = net.bfull[i];
-    el.bias_div = 1;
-#pragma unroll
-    for (int q = 0; q < RB; ++q)
-      for (int r0 = threadIdx.x; r0 < C * hw; r0 += blockDim.x) {
-        const int c = r0 / hw, r = r0 % hw, y = y0[q] + r / w, x = x0[q] + r % w;
-        float* a = A + q * wp.maxw + r0;
-        if (y < 0 || y >= H || x < 0 || x >= W) {
-          *a = 0.f;
-          continue;
-        }
-        *a = epi_relu(el, mq[q], (c * H + y) * W + x, *a, part[q]);
-      }
-    __syncthreads();
-    const LayerDev& Li = net.aff[i];
-    const int s = Li.s, k = Li.k, kk = k * k;
-    const int h2 = (h - 1) * s + k, w2 = (w - 1) * s + k, hw2 = h2 * w2;
-    const size_t wco = (size_t)Li.ci * kk;
-    for (int r0 = threadIdx.x; r0 < Li.ci * hw2; r0 += blockDim.x) {
-      const int c = r0 / hw2, r = r0 % hw2, yy = r / w2, xx = r % w2;
-      float acc[RB];
-#pragma unroll
-      for (int q = 0; q < RB; ++q) acc[q] = 0.f;
-      for (int kh = yy % s; kh < k && kh <= yy; kh += s) {
-        const int Y = (yy - kh) / s;
-        if (Y >= h) continue;
-        for (int kw = xx % s; kw < k && kw <= xx; kw += s) {
-          const int X = (xx - kw) / s;
-          if (X >= w) continue;
-          const float* ap = A + Y * w + X;
-          const float* wp2 = Li.W + (size_t)c * kk + kh * k + kw;
-          for (int o = 0; o < Li.co; ++o) {
-            const float wv = __ldg(wp2 + o * wco);
-#pragma unroll
-            for (int q = 0; q < RB; ++q) acc[q] = fmaf(ap[q * wp.maxw + o * hw], wv, acc[q]);
-          }
-        }
-      }
-      // positions outside the layer (padding) carry no coefficient
-#pragma unroll
-      for (int q = 0; q < RB; ++q) {
-        const int ya = y0[q] * s - Li.p + yy, xa = x0[q] * s - Li.p + xx;
-        B[q * wp.maxw + r0] = (ya >= 0 && ya < Li.hi && xa >= 0 && xa < Li.wi) ? acc[q] : 0.f;
-      }
-    }
-    float* tmp = A;
-    A = B;
-    B = tmp;
-    h = h2;
-    w = w2;
-#pragma unroll
-    for (int q = 0; q < RB; ++q) {
-      y0[q] = y0[q] * s - Li.p;
-      x0[q] = x0[q] * s - Li.p;
-    }
+    if (tl == 0) s_row[q] = WinRow{y0, x0};
   }
-#pragma unroll
-  for (int q = 0; q < RB; ++q) {
-    const float tot = block_sum(part[q]);
-    if (threadIdx.x == 0 && m0 + q < rows.M)
-      e.part[(size_t)(m0 + q) * e.nslot + e.slot_base] = tot + c0[q];
+  // a row's threads are RB lanes apart
+  for (int o = 16; o >= RB; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+  if ((threadIdx.x & 31) < RB) s_sum[threadIdx.x >> 5][q] = part;
+  __syncthreads();
+  if (tl == 0 && blockIdx.x * RB + q < rows.M) {
+    float tot = sg * (net.bfull[t] ? net.bfull[t][j] : Lt.b[co]);
+    for (int v = 0; v < THREADS / 32; ++v) tot += s_sum[v][q];
+    lb[m] = tot;
   }
 }
 
 void launch_win_rows(const NetDev& net, const WinPlan& wp, const RowsDev& rows, const Epi& e,
-                     cudaStream_t st) {
+                     float* lb, cudaStream_t st) {
   if (rows.M <= 0) return;
-  if (wp.maxw <= 1024) {
-    constexpr int RB = 4;
-    const int smem = 2 * RB * wp.maxw * (int)sizeof(float);
-    k_win_rows_rb<RB><<<(rows.M + RB - 1) / RB, 128, smem, st>>>(net, wp, rows, e);
-    return;
-  }
-  const int threads = wp.maxw >= 1024 ? 256 : 128;
-  const int smem = 2 * wp.maxw * (int)sizeof(float);
-  set_smem(k_win_rows, smem);
-  k_win_rows<<<rows.M, threads, smem, st>>>(net, wp, rows, e);
+  const int smem = (wp.rb * (wp.plane[0] + wp.plane[1]) + wp.wpad) * (int)sizeof(float);
+  const int grid = (rows.M + wp.rb - 1) / wp.rb;
+  bool wide = false;
+  for (int i = 1; i < wp.t; ++i)
+    wide = wide || (net.aff[i].ci & 3) == 0 || net.aff[i].ci == 2 || net.aff[i].ci == 3;
+  auto go = [&](auto kern, int threads) {
+    set_smem(kern, smem);
+    kern<<<grid, threads, smem, st>>>(net, wp, rows, e, lb);
+  };
+  if (wp.rb == 1) go(k_win_rows<true, 1>, 512);
+  else if (wide) go(k_win_rows<true, 4>, 512);
+  else go(k_win_rows<false, 4>, 256);
 }
 
 // ---------------------------------------------------------------------------
@@ -668,26 +779,6 @@ static int gemm_launch(int M, int N, int K, const float* A, int lda, const float
 // ---------------------------------------------------------------------------
 // convolution: transposed (back-substitution) and forward (adjoint / forward)
 // ---------------------------------------------------------------------------
-// Input positions are enumerated phase-major (ih mod s, iw mod s) so that the
-// threads of a warp share kernel taps and read the weights from shared memory
-// as broadcasts.
-__device__ __forceinline__ void decode_phase(int pidx, int hi, int wi, int s, int& ih, int& iw) {
-  for (int ph = 0; ph < s; ++ph) {
-    const int nh = (hi - ph + s - 1) / s;
-    for (int pw = 0; pw < s; ++pw) {
-      const int nw = (wi - pw + s - 1) / s;
-      const int cnt = nh * nw;
-      if (pidx < cnt) {
-        ih = ph + s * (pidx / nw);
-        iw = pw + s * (pidx % nw);
-        return;
-      }
-      pidx -= cnt;
-    }
-  }
-  ih = iw = -1;
-}
-
 template <int CB>
 __global__ void __launch_bounds__(128) k_convT(int M, const float* __restrict__ in, int ld_in,
                                                float* out, int ld_out, LayerDev L, Epi e) {

@@ -205,19 +205,21 @@ void launch_first_rows(const NetDev& net, const PoolDev& pool, const PropDev* pr
 // convolution neuron of zhat_t and meet only convolutions below it: after each
 // step the row is nonzero only within its receptive-field window, so one CTA
 // carries it to the input in shared memory.  h[i] x w[i] is the window at
-// layer i (all of the layer's channels); maxw the largest window in floats.
+// layer i (all of the layer's channels).
 struct WinPlan {
   int t;
   int h[MNBAB_MAXR + 2], w[MNBAB_MAXR + 2];
-  int maxw;
+  int plane[2];  // floats of a row's window buffers (layers t - 1, t - 3, ...; t - 2, t - 4, ...)
+  int wpad;      // floats of the staged weights of layers with 2 or 3 input channels
+  int rb;        // rows per CTA
 };
 // Plan for rows at zhat_t with the DeepPoly epilogue, or false where the layers
 // below t are not a single chain of convolutions or the windows do not fit.
 bool win_plan(const NetDev& net, int t, WinPlan& wp);
 // Bounds of rows.M rows through plan wp: the whole lower bound of row m (offset
-// terms, concretisation and sign * b_t[j]) goes to partial slot e.slot_base.
+// terms, concretisation and sign * b_t[j]) goes to lb[m].
 void launch_win_rows(const NetDev& net, const WinPlan& wp, const RowsDev& rows, const Epi& e,
-                     cudaStream_t st);
+                     float* lb, cudaStream_t st);
 // Fused optimisation loop for chain networks without multi-neuron constraints
 // (csrc/fused.cu): one CTA per objective row runs all sweeps, adjoints and Adam
 // steps.  bc1[s] / bc2[s] are Adam's bias corrections 1 - beta^(s+1).

@@ -577,15 +577,9 @@ void sweep(mnbab_net* n, int t, const RowsDev& rows, const SweepOpts& o) {
       macs += (double)L.ci * wp.h[i - 1] * wp.w[i - 1] * L.co * taps * taps;
       elems += (double)L.ci * wp.h[i - 1] * wp.w[i - 1];
     }
-    Epi e = base_epi(n, rows.node);
-    e.slot_base = 0;
-    {
-      Scope sc(c, C_WIN, 2.0 * rows.M * macs, 9.0 * rows.M * elems);
-      launch_win_rows(nd, wp, rows, e, c->st);
-    }
-    Scope sc(c, C_REDUCE, 0.0, 4.0 * rows.M);
-    launch_reduce_lb(rows.M, n->part, n->nslot, 1, nullptr, n->lb, false, rows.node, n->pool,
-                     n->X, n->d0, c->st);
+    const Epi e = base_epi(n, rows.node);
+    Scope sc(c, C_WIN, 2.0 * rows.M * macs, 9.0 * rows.M * elems);
+    launch_win_rows(nd, wp, rows, e, n->lb, c->st);
     return;
   }
   auto setup = [&](Epi& e, int layer) {

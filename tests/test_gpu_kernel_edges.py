@@ -95,3 +95,39 @@ def test_gamma_terms(Context, spec, k):
             top, *_ = core.optimize(net, on, dense, lo_t, hi_t, core.AdamHP(steps=1, eps_rel=1e-3))
             assert close(best[j], top).all()
 
+
+# windowed rows: stride classes of one to more than three taps (two passes over
+# the reduction), kernels smaller than the stride, 1, 2, 3, 4, 5 and 8 input
+# channels, windows cut by the padding, a row count that is not a multiple of
+# the rows per CTA, splits in the layers that the rows pass
+@pytest.mark.parametrize("layers,shape", [
+    ([("conv", 3, 3, 1, 1), ("relu",), ("conv", 5, 2, 2, 0), ("relu",), ("conv", 3, 3, 1, 1), ("relu",),
+      ("fc", 3)], (2, 7, 9)),
+    ([("conv", 4, 4, 3, 2), ("relu",), ("conv", 8, 5, 1, 2), ("relu",), ("conv", 7, 3, 2, 1), ("relu",),
+      ("fc", 3)], (1, 13, 11)),
+    ([("conv", 8, 1, 1, 0), ("relu",), ("conv", 12, 4, 1, 1), ("relu",), ("conv", 5, 1, 2, 0), ("relu",),
+      ("fc", 3)], (3, 6, 5)),
+    ([("conv", 2, 3, 4, 1), ("relu",), ("conv", 6, 3, 1, 2), ("relu",), ("fc", 3)], (5, 17, 14)),
+    # one row per CTA: the window at the input holds 54 x 54 values of 4 channels
+    ([("conv", 4, 4, 2, 1), ("relu",), ("conv", 4, 12, 2, 1), ("relu",), ("conv", 2, 8, 2, 0), ("relu",),
+      ("fc", 3)], (4, 72, 72)),
+])
+def test_window_rows(Context, layers, shape):
+    layers, C, d, lo, hi, prep = _case(dict(seed=41, in_shape=shape, layers=layers), 0.05)
+    net, lo_t, hi_t, l, u, S, _, _ = prep
+    rng = np.random.default_rng(2)
+    with Context(node_capacity=64) as ctx:
+        gnet = ctx.load_network(layers)
+        prop = ctx.set_property(gnet, lo, hi, C, d)
+        for i in l:
+            gl, gu = ctx.root_bounds(prop, i)
+            assert close(gl, l[i].numpy()).all() and close(gu, u[i].numpy()).all(), i
+        for j in range(3):
+            on = random_node(prep, rng, n_splits=j + 1, row=j % 2)
+            on.split_layer = 1
+            gid = ctx.node_root(prop, on.row)
+            ctx.import_params(gid, to_params(on, net.R))
+            ctx.bound_batch([gid])
+            core.rebound_node(net, on, lo_t, hi_t)
+            p = ctx.export_params(gid)
+            assert close(p.l, concat(on.l, net.R)).all() and close(p.u, concat(on.u, net.R)).all()
