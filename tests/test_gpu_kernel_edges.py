@@ -131,3 +131,31 @@ def test_window_rows(Context, layers, shape):
             core.rebound_node(net, on, lo_t, hi_t)
             p = ctx.export_params(gid)
             assert close(p.l, concat(on.l, net.R)).all() and close(p.u, concat(on.u, net.R)).all()
+
+
+def test_row_roots_are_created_by_the_first_step(Context):
+    """Started properties hold the slots of their row root nodes without
+    creating them: other nodes cannot take those slots, the queue counts them, and
+    the first step finds them."""
+    from paper_2205_00263_gb300.api import MnbabError
+    layers, C, d, lo, hi, _ = _case(dict(seed=43, in_shape=(1, 6, 6), layers=[
+        ("conv", 3, 3, 1, 1), ("relu",), ("fc", 4)]), 0.05)
+    rows = C.shape[0]
+    cap = 64  # the pad slot, two properties (root and rows), other nodes
+    with Context(node_capacity=cap) as ctx, Context(node_capacity=256) as big:
+        net = ctx.load_network(layers)
+        a, b = (ctx.set_property(net, lo, hi, C, d) for _ in range(2))
+        ctx.root_bounds(a, 1)
+        assert ctx.queue_size(a) == rows and ctx.queue_size(b) == rows
+        extra = [ctx.node_root(a, 0) for _ in range(cap - 1 - 2 * (rows + 1))]
+        with pytest.raises(MnbabError):
+            ctx.node_root(a, 0)
+        for n in extra:
+            ctx.node_free(n)
+        net2 = big.load_network(layers)
+        ref = big.set_property(net2, lo, hi, C, d)
+        assert big.bab_step([ref], max_nodes=rows, steps=2)["nodes_bounded"] == rows
+        assert ctx.bab_step([a, b], max_nodes=2 * rows, steps=2)["nodes_bounded"] == 2 * rows
+        for p in (a, b):
+            assert [(r["row"], r["seq"], r["lb"]) for r in ctx.trace(p)] == \
+                   [(r["row"], r["seq"], r["lb"]) for r in big.trace(ref)]
