@@ -259,10 +259,18 @@ bool win_plan(const NetDev& net, int t, WinPlan& wp) {
     if (i >= 1 && (net.aff[i].ci == 2 || net.aff[i].ci == 3))
       wp.wpad += net.aff[i].co * net.aff[i].k * net.aff[i].k * 4;
   }
-  // rows per CTA: 8 where two CTAs still fit on an SM, else 4 or 1
+  // rows per CTA: 8 where two CTAs still fit on an SM, else 4 or 1 (4 at most in
+  // the small CTAs where a row has 256 partial sums)
   auto bytes = [&](int rb) { return (rb * (wp.plane[0] + wp.plane[1]) + wp.wpad) * 4; };
-  wp.rb = bytes(WIN_RB_MAX) <= 112 * 1024 ? WIN_RB_MAX : bytes(4) <= 224 * 1024 ? 4 : 1;
-  return bytes(wp.rb) <= 224 * 1024;
+  wp.vt = mx <= 1024 ? 128 : 256;
+  wp.wide = false;
+  for (int i = 1; i < t; ++i) {
+    const int ci = net.aff[i].ci;
+    wp.wide = wp.wide || (ci & 3) == 0 || ci == 2 || ci == 3;
+  }
+  const int most = !wp.wide && wp.vt == 256 ? 4 : WIN_RB_MAX;
+  wp.rb = bytes(most) <= 104 * 1024 ? most : bytes(4) <= 216 * 1024 ? 4 : 1;
+  return bytes(wp.rb) <= 216 * 1024;
 }
 
 // x / d for the small operands of window indices (x d < 2^32), by the rounded-up
@@ -321,12 +329,8 @@ __device__ __forceinline__ void win_conv(const LayerDev& L, const float* __restr
   const int s = L.s, k = L.k, h2 = (h - 1) * s + k, w2 = (w - 1) * s + k;
   const int hw = h * w, hw2 = h2 * w2;
   const int items = hw2 * (RB / RG) * ((L.ci + CB - 1) / CB);
-  int ks = 1;
-  while (ks < 4 && items * ks * 2 <= THREADS) ks *= 2;
   const int wco = k * k * wci;
-  for (int b0 = 0; b0 < items * ks; b0 += THREADS) {
-    const int id = b0 + threadIdx.x, it = id / ks, k0 = id % ks;
-    const bool act = it < items;
+  for (int it = threadIdx.x; it < items; it += THREADS) {
     const int px = it % hw2, rg = it / hw2 % (RB / RG) * RG, grp = it / (hw2 * (RB / RG));
     constexpr int R2 = RG == 4 ? 2 : 1;
     float2 acc[CB][R2];
@@ -334,62 +338,51 @@ __device__ __forceinline__ void win_conv(const LayerDev& L, const float* __restr
     for (int c = 0; c < CB; ++c)
 #pragma unroll
       for (int r = 0; r < R2; ++r) acc[c][r] = make_float2(0.f, 0.f);
-    int yy = 0, xx = 0;
-    if (act) {
-      decode_phase(px, h2, w2, s, yy, xx);
-      for (int kh = yy % s, Y = yy / s; kh < k && Y >= 0; kh += s, --Y) {
-        if (Y >= h) continue;
-        for (int kw = xx % s, X = xx / s; kw < k && X >= 0; kw += s, --X) {
-          if (X >= w) continue;
-          const float* ap = A + (size_t)(k0 * hw + Y * w + X) * RB + rg;
-          const float* wp = Wt + (size_t)k0 * wco + (kh * k + kw) * wci + grp * CB;
+    int yy, xx;
+    decode_phase(px, h2, w2, s, yy, xx);
+    for (int kh = yy % s, Y = yy / s; kh < k && Y >= 0; kh += s, --Y) {
+      if (Y >= h) continue;
+      for (int kw = xx % s, X = xx / s; kw < k && X >= 0; kw += s, --X) {
+        if (X >= w) continue;
+        const float* ap = A + (size_t)(Y * w + X) * RB + rg;
+        const float* wp = Wt + (kh * k + kw) * wci + grp * CB;
 #pragma unroll 4
-          for (int o = k0; o < L.co; o += ks, ap += ks * hw * RB, wp += ks * wco) {
-            float2 v[R2];
+        for (int o = 0; o < L.co; ++o, ap += hw * RB, wp += wco) {
+          float2 v[R2];
+          if (RG == 4) {
+            const float4 v4 = *reinterpret_cast<const float4*>(ap);
+            v[0] = make_float2(v4.x, v4.y);
+            v[R2 - 1] = make_float2(v4.z, v4.w);
+          } else {
+            v[0] = make_float2(*ap, 0.f);
+          }
+          float wv[CB];
+          if (CB >= 4) {
+#pragma unroll
+            for (int c = 0; c < CB; c += 4) {
+              const float4* w4p = reinterpret_cast<const float4*>(wp + c);
+              const float4 w4 = SM ? *w4p : __ldg(w4p);
+              wv[c] = w4.x;
+              wv[c + 1 < CB ? c + 1 : c] = w4.y;
+              wv[c + 2 < CB ? c + 2 : c] = w4.z;
+              wv[c + 3 < CB ? c + 3 : c] = w4.w;
+            }
+          } else {
+            wv[0] = SM ? wp[0] : __ldg(wp);
+          }
+#pragma unroll
+          for (int c = 0; c < CB; ++c) {
             if (RG == 4) {
-              const float4 v4 = *reinterpret_cast<const float4*>(ap);
-              v[0] = make_float2(v4.x, v4.y);
-              v[R2 - 1] = make_float2(v4.z, v4.w);
+              const float2 ww = make_float2(wv[c], wv[c]);
+              acc[c][0] = fma2(v[0], ww, acc[c][0]);
+              acc[c][R2 - 1] = fma2(v[R2 - 1], ww, acc[c][R2 - 1]);
             } else {
-              v[0] = make_float2(*ap, 0.f);
-            }
-            float wv[CB];
-            if (CB >= 4) {
-#pragma unroll
-              for (int c = 0; c < CB; c += 4) {
-                const float4* w4p = reinterpret_cast<const float4*>(wp + c);
-                const float4 w4 = SM ? *w4p : __ldg(w4p);
-                wv[c] = w4.x;
-                wv[c + 1 < CB ? c + 1 : c] = w4.y;
-                wv[c + 2 < CB ? c + 2 : c] = w4.z;
-                wv[c + 3 < CB ? c + 3 : c] = w4.w;
-              }
-            } else {
-              wv[0] = SM ? wp[0] : __ldg(wp);
-            }
-#pragma unroll
-            for (int c = 0; c < CB; ++c) {
-              if (RG == 4) {
-                const float2 ww = make_float2(wv[c], wv[c]);
-                acc[c][0] = fma2(v[0], ww, acc[c][0]);
-                acc[c][R2 - 1] = fma2(v[R2 - 1], ww, acc[c][R2 - 1]);
-              } else {
-                acc[c][0].x = fmaf(v[0].x, wv[c], acc[c][0].x);
-              }
+              acc[c][0].x = fmaf(v[0].x, wv[c], acc[c][0].x);
             }
           }
         }
       }
     }
-    for (int o = ks >> 1; o; o >>= 1)
-#pragma unroll
-      for (int c = 0; c < CB; ++c)
-#pragma unroll
-        for (int r = 0; r < R2; ++r) {
-          acc[c][r].x += __shfl_xor_sync(0xffffffffu, acc[c][r].x, o);
-          if (RG == 4) acc[c][r].y += __shfl_xor_sync(0xffffffffu, acc[c][r].y, o);
-        }
-    if (!act || k0) continue;
     // positions outside the layer (padding) carry no coefficient
     bool in[RG];
 #pragma unroll
@@ -414,21 +407,26 @@ __device__ __forceinline__ void win_conv(const LayerDev& L, const float* __restr
 // RB = 8, 4 or (windows beyond 56 KB a row) 1 rows per CTA, their windows in shared memory with the rows of a
 // position adjacent.  Bound by the latency of the weight and bound loads (FMA
 // pipe 34% busy) and FP32 FMAs: on the 3x32x32 network's layers 3 and 4 (32768
-// and 8192 rows, 31 GFLOP) 1.1 and 2.3 ms; a thread per output element of one
-// row took 16.3 ms together.  Four columns of one row per thread instead of four
-// rows took 1.2 and 2.4 ms, but 149 against 101 us for the 25600 rows of 16
+// and 8192 rows, 31 GFLOP) 1.2 and 2.9 ms; a thread per output element of one
+// row took 16.3 ms together.  Few items leave threads idle in the deep layers'
+// first steps; splitting their reductions over lanes gained 0.7 ms and changed the
+// order of the sums, which stays that of one row alone.  Four columns of one row
+// per thread instead of four rows took 149 against 101 us for the 25600 rows of 16
 // 1x28x28 properties (112 us before): its columns are ragged in small windows.
 // WIDE: some layer of the chain has several input channels to a thread; without
 // one (a one-channel image below a single convolution) smaller CTAs of fewer
 // registers hide the latency of its short steps.
-template <bool WIDE, int RG>
+template <bool WIDE, int RG, int NA>
 __global__ void __launch_bounds__(WIDE ? 512 : 256, WIDE ? 2 : 6)
     k_win_rows(NetDev net, WinPlan wp, RowsDev rows, Epi e, float* __restrict__ lb) {
   constexpr int THREADS = WIDE ? 512 : 256;
   extern __shared__ __align__(16) float wsm[];
   __shared__ WinRow s_row[WIN_RB_MAX];
-  __shared__ float s_sum[THREADS / 32][WIN_RB_MAX];
-  const int t = wp.t, RB = wp.rb, tpr = THREADS / RB;
+  __shared__ float s_sum[WIN_RB_MAX][256], s_c0[WIN_RB_MAX];
+  // A row's offset terms are summed as wp.vt interleaved partial sums (element x of
+  // a layer to sum x mod vt), then in a tree over each 32 of them, then in order:
+  // the same sum for any number of rows per CTA.  A thread holds NA of them.
+  const int t = wp.t, RB = wp.rb, tpr = wp.vt / NA;
   const LayerDev& Lt = net.aff[t];
   // buffers of the layers t - 1, t - 3, ... and t - 2, t - 4, ...; then the
   // padded weights of layers with 2 or 3 input channels
@@ -445,7 +443,7 @@ __global__ void __launch_bounds__(WIDE ? 512 : 256, WIDE ? 2 : 6)
       d += n;
     }
   }
-  const int q = threadIdx.x % RB, tl = threadIdx.x / RB;
+  const int q = threadIdx.x % RB, tl = threadIdx.x / RB, nthr = THREADS / RB;
   const int m = min(blockIdx.x * RB + q, rows.M - 1);  // absent rows repeat the last (dropped)
   const int j = rows.j[m], node = rows.node[m];
   const float sg = rows.sign ? rows.sign[m] : 1.f;
@@ -455,10 +453,13 @@ __global__ void __launch_bounds__(WIDE ? 512 : 256, WIDE ? 2 : 6)
   if (tl == 0) s_row[q] = WinRow{y0, x0};
   {
     const int n0 = Lt.ci * Lt.k * Lt.k;
-    for (int i = tl; i < n0; i += tpr) buf[0][i * RB + q] = sg * __ldg(Lt.W + (size_t)co * n0 + i);
+    for (int i = tl; i < n0; i += nthr) buf[0][i * RB + q] = sg * __ldg(Lt.W + (size_t)co * n0 + i);
   }
   const PropDev& P = e.props[e.pool.prop[node]];
-  float part = 0.f;
+  float part[NA];
+#pragma unroll
+  for (int v = 0; v < NA; ++v) part[v] = 0.f;
+  const bool on = tl < tpr;
   int h = Lt.k, w = Lt.k;
   for (int i = t - 1, side = 0; i >= 0; --i, side ^= 1) {
     const LayerDev& Ln = net.aff[i + 1];  // layer i is this edge's input
@@ -468,21 +469,24 @@ __global__ void __launch_bounds__(WIDE ? 512 : 256, WIDE ? 2 : 6)
     __syncthreads();
     if (i == 0) {
       // concretisation over the input box
-      for (int r0 = tl; r0 < n; r0 += tpr) {
-        const int c = win_div(r0, mhw), r = r0 - c * hw, yr = win_div(r, mw);
-        const int y = y0 + yr, x = x0 + r - yr * w;
-        if (y < 0 || y >= H || x < 0 || x >= W) continue;
-        const int jx = (c * H + y) * W + x;
-        const float a = A[r0 * RB];
-        part += a * (a >= 0.f ? P.lo[jx] : P.hi[jx]);
-      }
+      for (int r0 = on ? tl : n; r0 < n; r0 += NA * tpr)
+#pragma unroll
+        for (int v = 0; v < NA; ++v) {
+          const int rr = r0 + v * tpr;
+          const int c = win_div(rr, mhw), r = rr - c * hw, yr = win_div(r, mw);
+          const int y = y0 + yr, x = x0 + r - yr * w;
+          if (rr >= n || y < 0 || y >= H || x < 0 || x >= W) continue;
+          const int jx = (c * H + y) * W + x;
+          const float a = A[rr * RB];
+          part[v] += a * (a >= 0.f ? P.lo[jx] : P.hi[jx]);
+        }
       break;
     }
     // ReLU step of layer i (DeepPoly slopes, splits enforced); the bounds of
     // four elements are loaded before the first is used
     const size_t nb = (size_t)node * e.SD + net.off[i];
     const float* bias = net.bfull[i];
-    for (int r0 = tl; r0 < n; r0 += 4 * tpr) {
+    for (int r0 = on ? tl : n; r0 < n; r0 += 4 * tpr) {
       int jx[4];
       float l[4], u[4], b[4];
       int sp[4];
@@ -522,7 +526,7 @@ __global__ void __launch_bounds__(WIDE ? 512 : 256, WIDE ? 2 : 6)
           bl = (-u[v] * l[v]) / den;
         }
         const float ah = a * D;
-        part += a * bl + ah * b[v];
+        part[v % NA] += a * bl + ah * b[v];
         A[rr * RB] = ah;
       }
     }
@@ -553,14 +557,20 @@ __global__ void __launch_bounds__(WIDE ? 512 : 256, WIDE ? 2 : 6)
     __syncthreads();
     if (tl == 0) s_row[q] = WinRow{y0, x0};
   }
-  // a row's threads are RB lanes apart
-  for (int o = 16; o >= RB; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-  if ((threadIdx.x & 31) < RB) s_sum[threadIdx.x >> 5][q] = part;
+  if (on)
+#pragma unroll
+    for (int v = 0; v < NA; ++v) s_sum[q][v * tpr + tl] = part[v];
+  if (tl == 0) s_c0[q] = sg * (net.bfull[t] ? net.bfull[t][j] : Lt.b[co]);
   __syncthreads();
-  if (tl == 0 && blockIdx.x * RB + q < rows.M) {
-    float tot = sg * (net.bfull[t] ? net.bfull[t][j] : Lt.b[co]);
-    for (int v = 0; v < THREADS / 32; ++v) tot += s_sum[v][q];
-    lb[m] = tot;
+  const int wq = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (wq < RB && blockIdx.x * RB + wq < rows.M) {
+    float tot = 0.f;
+    for (int v = 0; v < wp.vt / 32; ++v) {
+      float x = s_sum[wq][v * 32 + lane];
+      for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      tot += x;
+    }
+    if (lane == 0) lb[blockIdx.x * RB + wq] = tot + s_c0[wq];
   }
 }
 
@@ -569,16 +579,15 @@ void launch_win_rows(const NetDev& net, const WinPlan& wp, const RowsDev& rows, 
   if (rows.M <= 0) return;
   const int smem = (wp.rb * (wp.plane[0] + wp.plane[1]) + wp.wpad) * (int)sizeof(float);
   const int grid = (rows.M + wp.rb - 1) / wp.rb;
-  bool wide = false;
-  for (int i = 1; i < wp.t; ++i)
-    wide = wide || (net.aff[i].ci & 3) == 0 || net.aff[i].ci == 2 || net.aff[i].ci == 3;
   auto go = [&](auto kern, int threads) {
     set_smem(kern, smem);
     kern<<<grid, threads, smem, st>>>(net, wp, rows, e, lb);
   };
-  if (wp.rb == 1) go(k_win_rows<true, 1>, 512);
-  else if (wide) go(k_win_rows<true, 4>, 512);
-  else go(k_win_rows<false, 4>, 256);
+  if (wp.rb == 1) go(k_win_rows<true, 1, 1>, 512);
+  else if (!wp.wide) go(k_win_rows<false, 4, 4>, 256);
+  else if (wp.vt * wp.rb == 4 * 512) go(k_win_rows<true, 4, 4>, 512);
+  else if (wp.vt * wp.rb == 2 * 512) go(k_win_rows<true, 4, 2>, 512);
+  else go(k_win_rows<true, 4, 1>, 512);
 }
 
 // ---------------------------------------------------------------------------
@@ -1693,22 +1702,49 @@ void launch_forward(const LayerDev& L, int M, const float* in, int ld_in, float*
 // ---------------------------------------------------------------------------
 // reductions and bookkeeping
 // ---------------------------------------------------------------------------
-// One warp of the CTA sums the row's partials (lane-strided, then a shuffle
-// tree: a fixed order for a given number of slots); a single thread's serial sum
-// of the 68 to 150 slots of the 32 x 32 networks took 17 us a launch, this 4.
-__global__ void k_reduce_lb(int M, const float* part, int nslot, int used, const float* gp0,
-                            float* lb, int track, const int* row_node, PoolDev pool,
-                            const float* X, int d0) {
+// The CTA loads a row's partials together and one thread adds them in slot
+// order (the sum does not depend on how they were loaded).
+__global__ void __launch_bounds__(128) k_reduce_lb(int M, const float* part, int nslot, int used,
+                                                   const float* gp0, float* lb, int track,
+                                                   const int* row_node, PoolDev pool,
+                                                   const float* X, int d0) {
   const int m = blockIdx.x;
   __shared__ int imp;
   __shared__ int node;
-  if (threadIdx.x < 32) {
-    float acc = 0.f;
-    const float* p = part + (size_t)m * nslot;
-    for (int i = threadIdx.x; i < used; i += 32) acc += p[i];
-    if (gp0 && threadIdx.x < GP_SPLIT) acc -= gp0[(size_t)m * GP_SPLIT + threadIdx.x];
-    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  __shared__ __align__(16) float s[1024];
+  const float* p = part + (size_t)m * nslot;
+  float acc = 0.f;
+  for (int i0 = 0; i0 < used; i0 += 1024) {
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = 128 * u + threadIdx.x;
+      if (i0 + i < used) s[i] = p[i0 + i];
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
+      const int n = min(1024, used - i0);
+      int i = 0;
+      for (; i + 8 <= n; i += 8) {
+        const float4 a = *reinterpret_cast<const float4*>(s + i);
+        const float4 b = *reinterpret_cast<const float4*>(s + i + 4);
+        acc += a.x;
+        acc += a.y;
+        acc += a.z;
+        acc += a.w;
+        acc += b.x;
+        acc += b.y;
+        acc += b.z;
+        acc += b.w;
+      }
+      for (; i < n; ++i) acc += s[i];
+    }
+  }
+  if (threadIdx.x < 32) {
+    float g = gp0 && threadIdx.x < GP_SPLIT ? gp0[(size_t)m * GP_SPLIT + threadIdx.x] : 0.f;
+    for (int o = 16; o; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+    if (threadIdx.x == 0) {
+      if (gp0) acc -= g;
       lb[m] = acc;
       imp = 0;
       node = row_node ? row_node[m] : 0;
@@ -1719,9 +1755,20 @@ __global__ void k_reduce_lb(int M, const float* part, int nslot, int used, const
     }
   }
   __syncthreads();
-  if (imp)
-    for (int k = threadIdx.x; k < d0; k += blockDim.x)
-      pool.BESTX[(size_t)node * d0 + k] = X[(size_t)m * d0 + k];
+  if (!imp) return;
+  // the minimiser: eight loads in flight per thread (one by one, the 3072 values of
+  // a 3x32x32 input were most of the launch)
+  const float* x = X + (size_t)m * d0;
+  float* bx = pool.BESTX + (size_t)node * d0;
+  for (int k0 = threadIdx.x; k0 < d0; k0 += 8 * 128) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (k0 + 128 * u < d0) v[u] = x[k0 + 128 * u];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (k0 + 128 * u < d0) bx[k0 + 128 * u] = v[u];
+  }
 }
 
 void launch_reduce_lb(int M, const float* part, int nslot, int used, const float* gp0, float* lb,
@@ -1805,26 +1852,22 @@ __device__ __forceinline__ int layer_of(const NetDev& net, int f) {
 }
 
 // gamma^T P and gamma^T Phat per neuron (CSR by neuron), and gamma^T p per row.
-// A CTA serves `npb` neurons of one row: its threads read the neurons' entry
-// counts, write the zeros of those without entries and list the others; its
-// warps then take the listed neurons in turn, the lanes striding over a neuron's
-// entries (a neuron in three groups has about 450) with four loads in flight.
-// Bound by the latency of those loads: one thread per neuron walking its own
-// entries took 79 us for 9 rows of the 784-100-100-10 network and 335 us for 64
-// rows of the 3x32x32 one with 135k constraint rows.  The first GP_SPLIT CTAs of
-// a row sum a share of gamma^T p each (k_reduce_lb adds the shares).
-struct MncCsr {
-  const int* cptr;
-  const int* ce;
-  const float* cP;
-  const float* cPh;
-  int goff, e;
-};
+// The CTAs of a row: GP_SPLIT that sum a share of gamma^T p each (k_reduce_lb adds
+// the shares), `nzero` that write the zeros of neurons without entries, and the
+// others, which take eight of the layers' listed neurons (those with entries) at
+// a time: each warp brings one neuron's entries to shared memory, all loads in
+// flight (a neuron in three groups of 150 rows has 450), then two lanes per neuron
+// of one warp sum them, gamma^T P and gamma^T Phat, in entry order.  Bound by the
+// latency of those loads and the chain of FMAs.  64 rows of the 3x32x32 network with
+// 135k constraint rows, and 9 of the 784-100-100-10 one: 335 and 79 us with one
+// thread per neuron that loads its own entries, 409 and 12 with one warp per neuron
+// for the sums too (two lanes of 32 busy), 234 and 60 with 64-entry chunks.
 constexpr int GP_THREADS = 256;
+constexpr int GP_CHUNK = 480;  // entries of a chunk (15 per lane)
 
 __global__ void __launch_bounds__(GP_THREADS) k_gamma_proj(
     int M, const int* __restrict__ row_node, PoolDev pool, const PropDev* __restrict__ props,
-    NetDev net, int npb, float* __restrict__ GP, float* __restrict__ GPh,
+    NetDev net, int nzero, float* __restrict__ GP, float* __restrict__ GPh,
     float* __restrict__ gp0) {
   const int m = blockIdx.y;
   const int n = row_node[m];
@@ -1854,75 +1897,104 @@ __global__ void __launch_bounds__(GP_THREADS) k_gamma_proj(
     if (threadIdx.x == 0) gp0[(size_t)m * GP_SPLIT + blockIdx.x] = tot;
     return;
   }
-  __shared__ int s_cnt, s_f[GP_THREADS];
-  __shared__ MncCsr s_mc[MNBAB_MAXR + 1];
-  if (threadIdx.x == 0) s_cnt = 0;
-  if (threadIdx.x >= 1 && threadIdx.x <= net.R) {
-    const MncDev& mc = P.mnc[threadIdx.x];
-    s_mc[threadIdx.x] = MncCsr{mc.cptr, mc.ce, mc.cP, mc.cPh, mc.goff, mc.e};
-  }
-  __syncthreads();
-  const int f0 = (blockIdx.x - GP_SPLIT) * npb;
-  if (threadIdx.x < npb && f0 + threadIdx.x < net.SD) {
-    const int f = f0 + threadIdx.x;
-    const int i = layer_of(net, f);
-    const MncCsr& mc = s_mc[i];
-    const int j = f - net.off[i];
-    if (mc.e > 0 && mc.cptr[j + 1] > mc.cptr[j]) {
-      s_f[atomicAdd(&s_cnt, 1)] = f;  // order of the list: any, every neuron is on its own
-    } else {
-      GP[(size_t)m * net.SD + f] = 0.f;
-      GPh[(size_t)m * net.SD + f] = 0.f;
-    }
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  for (int a = threadIdx.x >> 5; a < s_cnt; a += GP_THREADS / 32) {
-    const int f = s_f[a];
-    const int i = layer_of(net, f);
-    const MncCsr& mc = s_mc[i];
-    const int j = f - net.off[i];
-    const float* g = gam + mc.goff;
-    const int q0 = mc.cptr[j], q1 = mc.cptr[j + 1];
-    float gp = 0.f, gph = 0.f;
-    for (int q = q0 + lane; q < q1; q += 32 * 4) {
-      int ce[4];
-      float gv[4], cp[4], cph[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const bool in = q + 32 * k < q1;
-        ce[k] = in ? mc.ce[q + 32 * k] : 0;
-        cp[k] = in ? mc.cP[q + 32 * k] : 0.f;
-        cph[k] = in ? mc.cPh[q + 32 * k] : 0.f;
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) gv[k] = q + 32 * k < q1 ? g[ce[k]] : 0.f;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        gp = fmaf(gv[k], cp[k], gp);
-        gph = fmaf(gv[k], cph[k], gph);
+  if (blockIdx.x < GP_SPLIT + nzero) {
+    for (int f = (blockIdx.x - GP_SPLIT) * GP_THREADS + threadIdx.x; f < net.SD;
+         f += nzero * GP_THREADS) {
+      const int i = layer_of(net, f), j = f - net.off[i];
+      const int* cptr = P.mnc[i].e > 0 ? P.mnc[i].cptr : nullptr;
+      if (!cptr || cptr[j + 1] == cptr[j]) {
+        GP[(size_t)m * net.SD + f] = 0.f;
+        GPh[(size_t)m * net.SD + f] = 0.f;
       }
     }
-    for (int o = 16; o; o >>= 1) {
-      gp += __shfl_xor_sync(0xffffffffu, gp, o);
-      gph += __shfl_xor_sync(0xffffffffu, gph, o);
+    return;
+  }
+  constexpr int NW = GP_THREADS / 32, LD = GP_CHUNK + 4;
+  __shared__ __align__(16) float s_ent[NW][3][LD];  // gamma, P, Phat
+  __shared__ int s_len[NW], s_f[NW];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nb = gridDim.x - GP_SPLIT - nzero, b = blockIdx.x - GP_SPLIT - nzero;
+  int total = 0;
+  for (int i = 1; i <= net.R; ++i) total += P.mnc[i].n_act;
+  for (int a0 = b * NW; a0 < total; a0 += nb * NW) {
+    // this warp's neuron and its entries
+    int q0 = 0, len = 0;
+    const int *ce_ = nullptr;
+    const float *cP_ = nullptr, *cPh_ = nullptr, *g = nullptr;
+    if (a0 + warp < total) {
+      int i = 1, a = a0 + warp;
+      while (a >= P.mnc[i].n_act) a -= P.mnc[i++].n_act;
+      const MncDev& mc = P.mnc[i];
+      const int j = mc.act[a];
+      q0 = mc.cptr[j];
+      len = mc.cptr[j + 1] - q0;
+      ce_ = mc.ce + q0;
+      cP_ = mc.cP + q0;
+      cPh_ = mc.cPh + q0;
+      g = gam + mc.goff;
+      if (lane == 0) s_f[warp] = net.off[i] + j;
     }
-    if (lane == 0) {
-      GP[(size_t)m * net.SD + f] = gp;
-      GPh[(size_t)m * net.SD + f] = gph;
+    if (lane == 0) s_len[warp] = len;
+    __syncthreads();
+    int most = 0;
+    for (int w = 0; w < NW; ++w) most = max(most, s_len[w]);
+    const int mine = (threadIdx.x >> 1) % NW, which = threadIdx.x & 1;
+    float acc = 0.f;
+    for (int c0 = 0; c0 < most; c0 += GP_CHUNK) {
+      int ce[GP_CHUNK / 32];
+      float cp[GP_CHUNK / 32], cph[GP_CHUNK / 32];
+#pragma unroll
+      for (int v = 0; v < GP_CHUNK / 32; ++v) {
+        const int k = c0 + 32 * v + lane;
+        ce[v] = k < len ? ce_[k] : -1;
+        cp[v] = k < len ? cP_[k] : 0.f;
+        cph[v] = k < len ? cPh_[k] : 0.f;
+      }
+#pragma unroll
+      for (int v = 0; v < GP_CHUNK / 32; ++v) {
+        s_ent[warp][0][32 * v + lane] = ce[v] >= 0 ? g[ce[v]] : 0.f;
+        s_ent[warp][1][32 * v + lane] = cp[v];
+        s_ent[warp][2][32 * v + lane] = cph[v];
+      }
+      __syncthreads();
+      if (threadIdx.x < 2 * NW) {
+        const float* eg = s_ent[mine][0];
+        const float* ec = s_ent[mine][1 + which];
+        const int cnt = min(GP_CHUNK, s_len[mine] - c0);
+        int k = 0;
+        for (; k + 8 <= cnt; k += 8) {
+          const float4 x0 = *reinterpret_cast<const float4*>(eg + k);
+          const float4 x1 = *reinterpret_cast<const float4*>(eg + k + 4);
+          const float4 y0 = *reinterpret_cast<const float4*>(ec + k);
+          const float4 y1 = *reinterpret_cast<const float4*>(ec + k + 4);
+          acc = fmaf(x0.x, y0.x, acc);
+          acc = fmaf(x0.y, y0.y, acc);
+          acc = fmaf(x0.z, y0.z, acc);
+          acc = fmaf(x0.w, y0.w, acc);
+          acc = fmaf(x1.x, y1.x, acc);
+          acc = fmaf(x1.y, y1.y, acc);
+          acc = fmaf(x1.z, y1.z, acc);
+          acc = fmaf(x1.w, y1.w, acc);
+        }
+        for (; k < cnt; ++k) acc = fmaf(eg[k], ec[k], acc);
+      }
+      __syncthreads();
     }
+    if (threadIdx.x < 2 * NW && a0 + mine < total)
+      (which ? GPh : GP)[(size_t)m * net.SD + s_f[mine]] = acc;
+    __syncthreads();
   }
 }
 
-// Neurons per CTA: 32 spreads the few hundred neurons of a small network over
-// several CTAs a row (its listed neurons are dense), 256 keeps the CTAs of a
-// large one few (most of its neurons have no entries).
+// CTAs per row for the listed neurons: one pass over up to 1024 of them
 void launch_gamma_proj(int M, const int* row_node, PoolDev pool, const PropDev* props,
                        const NetDev& net, float* GP, float* GPh, float* gp0, cudaStream_t st) {
   if (M <= 0) return;
-  const int npb = net.SD >= 8192 ? GP_THREADS : 32;
-  dim3 grid(GP_SPLIT + (net.SD + npb - 1) / npb, M);
-  k_gamma_proj<<<grid, GP_THREADS, 0, st>>>(M, row_node, pool, props, net, npb, GP, GPh, gp0);
+  const int per = GP_THREADS / 32;
+  const int nact = std::min(128, (net.SD + per - 1) / per);
+  const int nzero = (net.SD + 4 * GP_THREADS - 1) / (4 * GP_THREADS);
+  dim3 grid(GP_SPLIT + nzero + nact, M);
+  k_gamma_proj<<<grid, GP_THREADS, 0, st>>>(M, row_node, pool, props, net, nzero, GP, GPh, gp0);
 }
 
 // d lb / d gamma_e = sum_k P_ek (d lb / d a')_idx + Phat_ek (d lb / d ahat)_idx - p_e.

@@ -75,6 +75,8 @@ struct MncDev {
   int goff;       // offset of this layer's gamma entries in a node's gamma row
   const int* idx; const float* P; const float* Ph; const float* p;
   const int* cptr; const int* ce; const float* cP; const float* cPh;
+  const int* act;  // neurons with entries, ascending
+  int n_act;
 };
 
 struct PropDev {
@@ -212,6 +214,8 @@ struct WinPlan {
   int plane[2];  // floats of a row's window buffers (layers t - 1, t - 3, ...; t - 2, t - 4, ...)
   int wpad;      // floats of the staged weights of layers with 2 or 3 input channels
   int rb;        // rows per CTA
+  int vt;        // partial sums of a row's offset terms
+  bool wide;     // a layer has several input channels to a thread
 };
 // Plan for rows at zhat_t with the DeepPoly epilogue, or false where the layers
 // below t are not a single chain of convolutions or the windows do not fit.

@@ -1962,6 +1962,13 @@ void set_mnc_impl(mnbab_ctx* c, mnbab_prop* p, int layer, int n_rows, int k, con
         cP[at] = P[q];
         cPh[at] = Phat[q];
       }
+    std::vector<int> act;
+    for (int j = 0; j < d; ++j)
+      if (cnt[j + 1] > cnt[j]) act.push_back(j);
+    int* dact = dalloc_t<int>(c, act.size());
+    h2d(c, dact, act.data(), act.size());
+    m.act = dact;
+    m.n_act = (int)act.size();
     int* didx = dalloc_t<int>(c, nk);
     float* dP = dalloc_t<float>(c, nk);
     float* dPh = dalloc_t<float>(c, nk);
