@@ -247,6 +247,114 @@ __device__ __forceinline__ float epi_finish(const Epi& e, int m, int j, float v,
   }
 }
 
+// The two-phase form with the kind of epilogue as a template parameter, for
+// kernels that are instantiated per kind: a kernel that finishes many outputs per
+// thread and switches on the kind at each is several times as long, and its CTAs
+// wait for instructions more than for data.  The arithmetic is epi_finish's.
+enum EpiMode { EM_RELU, EM_RELU_FINAL, EM_RELU_GAMMA, EM_CONC, EM_ADJ, EM_ADJ_GAMMA, EM_FWD, EM_STORE };
+
+inline EpiMode epi_mode(const Epi& e) {
+  switch (e.kind) {
+    case EPI_RELU: return !e.final_mode ? EM_RELU : e.GP ? EM_RELU_GAMMA : EM_RELU_FINAL;
+    case EPI_CONC: return EM_CONC;
+    case EPI_ADJ: return e.Hz ? EM_ADJ_GAMMA : EM_ADJ;
+    case EPI_FWD_RELU: return EM_FWD;
+    default: return EM_STORE;
+  }
+}
+
+template <int EM>
+__device__ __forceinline__ void epi_load_m(const Epi& e, int n, const PropDev* P, int m, int j,
+                                           EpiIn& in) {
+  if (e.acc_in) in.acc = e.acc_in[(size_t)m * e.acc_ld + j];
+  const size_t q = (size_t)n * e.SD + e.off + j, qm = (size_t)m * e.SD + e.off + j;
+  if constexpr (EM <= EM_RELU_GAMMA) {
+    in.l = e.pool.L[q];
+    in.u = e.pool.U[q];
+    in.s = e.pool.S[q];
+    in.cb = e.bias[j];
+    if constexpr (EM >= EM_RELU_FINAL) {
+      in.al = e.pool.ALPHA[q];
+      in.be = e.pool.BETA[q];
+    }
+    if constexpr (EM == EM_RELU_GAMMA) {
+      in.gp = e.GP[qm];
+      in.gph = e.GPh[qm];
+    }
+  } else if constexpr (EM == EM_ADJ || EM == EM_ADJ_GAMMA) {
+    in.l = e.pool.L[q];
+    in.u = e.pool.U[q];
+    in.s = e.pool.S[q];
+    in.al = e.pool.ALPHA[q];
+    in.gp = e.AP[qm];
+  } else if constexpr (EM == EM_CONC) {
+    in.l = P->lo[j];
+    in.u = P->hi[j];
+  }
+}
+
+template <int EM>
+__device__ __forceinline__ float epi_finish_m(const Epi& e, int m, int j, float v, const EpiIn& in,
+                                              float& part) {
+  if (e.acc_in) v += in.acc;
+  const size_t qm = (size_t)m * e.SD + e.off + j;
+  if constexpr (EM <= EM_RELU_GAMMA) {
+    const float l = in.l, u = in.u;
+    const int s = in.s;
+    float ap = v;
+    if constexpr (EM == EM_RELU_GAMMA) ap += in.gp;
+    float D, bl = 0.f;
+    if (s == -1) D = 1.f;
+    else if (s == 1) D = 0.f;
+    else if (l >= 0.f) D = 1.f;
+    else if (u <= 0.f) D = 0.f;
+    else if (ap >= 0.f) D = EM >= EM_RELU_FINAL ? in.al : (u >= -l ? 1.f : 0.f);
+    else {
+      const float den = u - l;
+      D = u / den;
+      bl = (-u * l) / den;
+    }
+    float ah = ap * D;
+    if constexpr (EM >= EM_RELU_FINAL) ah += in.be * (float)s;
+    if constexpr (EM == EM_RELU_GAMMA) ah += in.gph;
+    if (e.AP) e.AP[qm] = ap;
+    part += ap * bl + ah * in.cb;
+    return ah;
+  } else if constexpr (EM == EM_CONC) {
+    const float x = v >= 0.f ? in.l : in.u;
+    part += v * x;
+    if (e.X) e.X[(size_t)m * e.d0 + j] = x;
+    return v;
+  } else if constexpr (EM == EM_ADJ || EM == EM_ADJ_GAMMA) {
+    const float l = in.l, u = in.u, ap = in.gp, h = v;
+    const int s = in.s;
+    float D, bl = 0.f;
+    bool abr = false;
+    if (s == -1) D = 1.f;
+    else if (s == 1) D = 0.f;
+    else if (l >= 0.f) D = 1.f;
+    else if (u <= 0.f) D = 0.f;
+    else if (ap >= 0.f) { D = in.al; abr = true; }
+    else {
+      const float den = u - l;
+      D = u / den;
+      bl = (-u * l) / den;
+    }
+    e.GA[qm] = abr ? h * ap : 0.f;
+    e.GB[qm] = h * (float)s;
+    const float g = h * D + bl;
+    if constexpr (EM == EM_ADJ_GAMMA) {
+      e.Hz[qm] = h;
+      e.Gz[qm] = g;
+    }
+    return g;
+  } else if constexpr (EM == EM_FWD) {
+    return fmaxf(v, 0.f);
+  } else {
+    return v;
+  }
+}
+
 __device__ __forceinline__ bool epi_has_part(const Epi& e) {
   return e.part != nullptr && (e.kind == EPI_RELU || e.kind == EPI_CONC);
 }

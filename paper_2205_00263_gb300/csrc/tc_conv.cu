@@ -25,7 +25,11 @@
 //    block k (3 MMAs of K = 8 per K step: hi.hi + hi.lo + lo.hi, FP32
 //    accumulation in tensor memory);
 //  - the epilogue reads each warp's 32 TMEM lanes (one objective row) with
-//    tcgen05.ld and applies the same epilogue functions as the SIMT kernels;
+//    tcgen05.ld and applies the same epilogue functions as the SIMT kernels, one
+//    instantiation per kind and a rolled loop over eight channels: unrolled with
+//    a switch on the kind at every output, the CTAs waited for instructions (64
+//    rows: conv_tc 10.0 ms of 20 Adam steps of the 3x32x32 network, now 6.6; 128
+//    rows of the residual one 10.2, now 6.3);
 //    a row's offset partial is a warp reduction in a fixed order, written to
 //    slot (class, position chunk), so it does not depend on the other rows.
 // Every wait is bounded; on timeout the kernel sets the device error flag,
@@ -123,26 +127,24 @@ __global__ void k_tc_conv_split(LayerDev L, int dir, int Kp, int NP, float* hi, 
 
 constexpr int TC_THREADS = 256;  // 8 warps: two threads per GEMM row gather a K block
 
-template <int NP>
-__global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ CUtensorMap tm_hi,
-                                                        const __grid_constant__ CUtensorMap tm_lo,
-                                                        LayerDev L, int dir, int M, int nchunk,
-                                                        const float* __restrict__ in, int ld_in,
-                                                        float* out, int ld_out, Epi e, int* err) {
+// one instantiation per kind of epilogue (EM); NP: channels padded to 16
+template <int EM>
+__global__ void __launch_bounds__(TC_THREADS, 2)
+    k_conv_tc(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant__ CUtensorMap tm_lo,
+              LayerDev L, int dir, int NP, int M, int nchunk, const float* __restrict__ in,
+              int ld_in, float* out, int ld_out, Epi e, int* err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   constexpr int A_BYTES = 128 * KC * 4;
-  constexpr int B_BYTES = NP * KC * 4;
-  constexpr int STAGE = 2 * A_BYTES + 2 * B_BYTES;
-  constexpr uint32_t NCOLS = NP <= 32 ? 32 : 64;
+  const int B_BYTES = NP * KC * 4;
+  const int STAGE = 2 * A_BYTES + 2 * B_BYTES;
+  const uint32_t NCOLS = NP <= 32 ? 32 : 64;
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bar = reinterpret_cast<uint64_t*>(base + 2 * STAGE);  // tma[2], mma[2]
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bar + 4);
-  // reduction table of the whole K range, computed once: source offset
-  // (channel plane + tap shift) and tap shifts for the bounds check
-  // (dy = dx = -1000: padding past K)
-  __shared__ int t_delta[TC_KMAX];
-  __shared__ short2 t_dd[TC_KMAX];
+  // reduction table of the whole K range, computed once: source offset (channel
+  // plane + tap shift) and tap, of which each thread knows which are in range
+  __shared__ __align__(16) int2 t_tab[TC_KMAX];
   __shared__ int s_fail;
   __shared__ float s_part[2][TROWS];
 
@@ -192,13 +194,13 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_holder;
-  constexpr uint32_t idesc = tc::idesc_tf32_m128(NP);
+  const uint32_t idesc = tc::idesc_tf32_m128(NP);
 
   const int nk = (c.K + KC - 1) / KC;
   for (int kidx = tid; kidx < nk * KC; kidx += TC_THREADS) {
-    int delta = 0, dy = -1000, dx = -1000;
+    int delta = 0, ta = 31, tb = 31;  // past K: a tap that is never in range
     if (kidx < c.K) {
-      int off;
+      int off, dy, dx;
       if (dir == 0) {
         const int kk2 = L.k * L.k;
         off = (kidx / kk2) * L.hi * L.wi;
@@ -211,21 +213,36 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
         dx = -(kidx % c.nb);
       }
       delta = off + dy * Wsrc + dx;
+      ta = abs(dy);
+      tb = abs(dx);
     }
-    t_delta[kidx] = delta;
-    t_dd[kidx] = make_short2((short)dy, (short)dx);
+    t_tab[kidx] = make_int2(delta, ta | tb << 8);
   }
+  // tap rows and columns whose source position lies in the plane, for this
+  // thread's position (a class has at most 32 of each: K <= TC_KMAX; all 32 x 32
+  // leave no padding past K)
+  unsigned vy = 0, vx = 0;
+  if (pv) {
+    for (int a = 0; a < c.na; ++a) {
+      const int yy = dir == 0 ? gy + a : gy - a;
+      if (yy >= 0 && yy < Hs) vy |= 1u << a;
+    }
+    for (int b = 0; b < c.nb; ++b) {
+      const int xx = dir == 0 ? gx + b : gx - b;
+      if (xx >= 0 && xx < Wsrc) vx |= 1u << b;
+    }
+  }
+  auto in_range = [&](int tap) { return (vy >> (tap & 31)) & (vx >> (tap >> 8)) & 1u; };
   __syncthreads();
   // implicit im2col: the 16 reduction values of this thread's GEMM row in K
   // block kb (half kh of the block)
   auto gather = [&](int kb, float (&v)[16]) {
+    const int4* tt = reinterpret_cast<const int4*>(t_tab + kb * KC + kh * 16);
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int kk = kb * KC + kh * 16 + u;
-      const short2 dd = t_dd[kk];
-      const int yy = gy + dd.x, xx = gx + dd.y;
-      const bool in_b = pv && yy >= 0 && yy < Hs && xx >= 0 && xx < Wsrc;
-      v[u] = in_b ? __ldg(src + t_delta[kk]) : 0.f;
+    for (int u = 0; u < 8; ++u) {
+      const int4 t2 = tt[u];  // two entries: source offset, tap
+      v[2 * u] = in_range(t2.y) ? __ldg(src + t2.x) : 0.f;
+      v[2 * u + 1] = in_range(t2.w) ? __ldg(src + t2.z) : 0.f;
     }
   };
   bool ok = true;
@@ -282,7 +299,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t ah = tc::smem_u32(a_hi), al = tc::smem_u32(a_lo);
         const uint32_t bh = tc::smem_u32(b_hi), bl = tc::smem_u32(b_lo);
-        constexpr uint32_t BLBO = NP * 16;  // B: core matrices along K
+        const uint32_t BLBO = (uint32_t)NP * 16u;  // B: core matrices along K
 #pragma unroll
         for (int ks = 0; ks < KC / 8; ++ks) {
           const uint32_t ao = ks * 256, bo = ks * 2 * BLBO;
@@ -316,8 +333,8 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
   }
   if (ok) {
     // epilogue: every warp reads its TMEM lane quarter (objective row rq); warp
-    // group kh takes the 16-column chunks 16 (2 i + kh).  The inputs of four
-    // outputs are loaded together before any of them is finished.
+    // group kh takes the 16-column chunks 16 (2 i + kh), eight columns at a time,
+    // whose inputs are loaded together before any of them is finished.
     float part = 0.f;
     const int y = dir == 0 ? iy : c.y0 + L.s * iy;
     const int x = dir == 0 ? ix : c.x0 + L.s * ix;
@@ -327,33 +344,33 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const __grid_constant__ 
     const uint32_t trow = tmem + ((uint32_t)(rq * 32) << 16);
     const int nrow = pv ? e.row_node[m] : 0;
     const PropDev* Pp = pv ? epi_prop(e, nrow) : nullptr;
-    for (int c0 = 16 * kh; c0 < NP; c0 += 32) {
-      float v[16];
+#pragma unroll 1
+    for (int it = 2 * kh; it < NP / 8; it += (it & 1) ? 3 : 1) {
+      const int c0 = 8 * it;
+      float v[8];
+      __syncwarp();
       if (nk > 0) {
-        tc::tmem_ld16(trow + (uint32_t)c0, v);
+        tc::tmem_ld8(trow + (uint32_t)c0, v);
       } else {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = 0.f;  // a class without taps
+        for (int i = 0; i < 8; ++i) v[i] = 0.f;  // a class without taps
       }
       if (pv) {
+        EpiIn ein[8];
 #pragma unroll
-        for (int g = 0; g < 16; g += 4) {
-          EpiIn in[4];
+        for (int i = 0; i < 8; ++i) {
+          const int n = c0 + i;
+          if (n < N) epi_load_m<EM>(e, nrow, Pp, m, n * plane + pj, ein[i]);
+        }
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int n = c0 + g + i;
-            if (n < N) epi_load(e, nrow, Pp, m, n * plane + pj, in[i]);
-          }
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int n = c0 + g + i;
-            if (n < N) {
-              const int j = n * plane + pj;
-              float val = v[g + i];
-              if (dir == 0) val += L.b[n];
-              const float o = epi_finish(e, m, j, val, in[i], part);
-              if (out) out[(size_t)m * ld_out + j] = o;
-            }
+        for (int i = 0; i < 8; ++i) {
+          const int n = c0 + i;
+          if (n < N) {
+            const int j = n * plane + pj;
+            float val = v[i];
+            if (dir == 0) val += L.b[n];
+            const float o = epi_finish_m<EM>(e, m, j, val, ein[i], part);
+            if (out) out[(size_t)m * ld_out + j] = o;
           }
         }
       }
@@ -389,10 +406,7 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-template <int NP>
-constexpr int conv_tc_smem() {
-  return 1024 + 2 * (2 * 128 * KC * 4 + 2 * NP * KC * 4) + 64;
-}
+int conv_tc_smem(int NP) { return 1024 + 2 * (2 * 128 * KC * 4 + 2 * NP * KC * 4) + 64; }
 
 }  // namespace
 
@@ -475,20 +489,21 @@ int launch_tc_conv(const LayerDev& L, int dir, int M, const float* in, int ld_in
                    int ld_out, const Epi& e, cudaStream_t st) {
   const TcConv* t = static_cast<const TcConv*>(L.tc);
   const dim3 grid(t->ncls[dir] * t->nchunk[dir], (M + TROWS - 1) / TROWS);
-  static bool attr[4] = {false, false, false, false};
-  auto go = [&](auto kern, int smem, int which) {
-    if (!attr[which]) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      attr[which] = true;
-    }
-    kern<<<grid, TC_THREADS, smem, st>>>(t->hi[dir], t->lo[dir], L, dir, M, t->nchunk[dir], in, ld_in,
-                                  out, ld_out, e, e.err);
+  const int NP = t->NP[dir], smem = conv_tc_smem(NP);
+  auto go = [&](auto kern) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    kern<<<grid, TC_THREADS, smem, st>>>(t->hi[dir], t->lo[dir], L, dir, NP, M, t->nchunk[dir], in,
+                                         ld_in, out, ld_out, e, e.err);
   };
-  switch (t->NP[dir]) {
-    case 16: go(k_conv_tc<16>, conv_tc_smem<16>(), 0); break;
-    case 32: go(k_conv_tc<32>, conv_tc_smem<32>(), 1); break;
-    case 48: go(k_conv_tc<48>, conv_tc_smem<48>(), 2); break;
-    default: go(k_conv_tc<64>, conv_tc_smem<64>(), 3); break;
+  switch (epi_mode(e)) {
+    case EM_RELU: go(k_conv_tc<EM_RELU>); break;
+    case EM_RELU_FINAL: go(k_conv_tc<EM_RELU_FINAL>); break;
+    case EM_RELU_GAMMA: go(k_conv_tc<EM_RELU_GAMMA>); break;
+    case EM_CONC: go(k_conv_tc<EM_CONC>); break;
+    case EM_ADJ: go(k_conv_tc<EM_ADJ>); break;
+    case EM_ADJ_GAMMA: go(k_conv_tc<EM_ADJ_GAMMA>); break;
+    case EM_FWD: go(k_conv_tc<EM_FWD>); break;
+    default: go(k_conv_tc<EM_STORE>); break;
   }
   return grid.x;
 }

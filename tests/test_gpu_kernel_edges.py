@@ -159,3 +159,43 @@ def test_row_roots_are_created_by_the_first_step(Context):
         for p in (a, b):
             assert [(r["row"], r["seq"], r["lb"]) for r in ctx.trace(p)] == \
                    [(r["row"], r["seq"], r["lb"]) for r in big.trace(ref)]
+
+
+# tensor-core convolutions in both directions (forced by gemm_path 2): strides
+# 1 to 4, kernels below and above the stride, padding beyond the kernel's reach, planes
+# smaller than a tile and rows across tiles, channel counts that are not multiples of 8 or 16,
+# several channel chunks and class groups; one row and enough rows for two tiles per CTA
+@pytest.mark.parametrize("layers,shape", [
+    ([("conv", 9, 5, 3, 2), ("relu",), ("conv", 17, 2, 4, 1), ("relu",), ("fc", 3)], (8, 22, 15)),
+    ([("conv", 24, 3, 1, 2), ("relu",), ("conv", 48, 5, 2, 2), ("relu",), ("fc", 3)], (10, 6, 9)),
+    ([("conv", 40, 1, 2, 0), ("relu",), ("conv", 64, 3, 1, 0), ("relu",), ("conv", 8, 1, 1, 0), ("relu",),
+      ("fc", 3)], (9, 9, 7)),
+    ([("conv", 16, 4, 2, 1), ("relu",), ("conv", 33, 4, 2, 1), ("relu",), ("fc", 3)], (12, 32, 20)),
+])
+def test_tensor_core_convolutions(Context, layers, shape):
+    layers, C, d, lo, hi, prep = _case(dict(seed=51, in_shape=shape, layers=layers), 0.01)
+    net, lo_t, hi_t, l, u, S, _, _ = prep
+    SD = sum(l[i].numel() for i in l)
+    rng = np.random.default_rng(4)
+    nodes = [random_node(prep, rng, n_splits=j, row=j % 2) for j in range(3)]
+    refs = []
+    for on in nodes:
+        on.split_layer = net.R
+        refs.append(core.bound_and_grad(net, on, on.alpha, on.beta, on.gamma, None, lo_t, hi_t))
+    with Context(node_capacity=2048, gemm_path=2) as ctx:
+        gnet = ctx.load_network(layers)
+        prop = ctx.set_property(gnet, lo, hi, C, d)
+        gids = []
+        for on in nodes:
+            gids.append(ctx.node_root(prop, on.row))
+            ctx.import_params(gids[-1], to_params(on, net.R))
+        for batch in ([0], [j % 3 for j in range(700)]):
+            lb, ga, gb, _ = ctx.bound_grad([gids[j] for j in batch], SD, 0)
+            for i in list(range(min(3, len(batch)))) + [len(batch) - 1]:
+                ref, _, oa, ob, _ = refs[batch[i]]
+                assert close(lb[i], float(ref)).all(), (batch[i], lb[i], float(ref))
+                o = np.concatenate([concat(oa, net.R), concat(ob, net.R)])
+                g = np.concatenate([ga[i], gb[i]])
+                assert np.abs(g - o).max() <= TOL * (1 + np.abs(o).max())
+            assert all((lb[j::3] == lb[j]).all() or np.abs(lb[j::3] - lb[j]).max() <= 1e-6 * (1 + abs(lb[j]))
+                       for j in range(min(3, len(batch))))
