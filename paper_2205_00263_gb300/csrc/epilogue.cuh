@@ -263,10 +263,10 @@ inline EpiMode epi_mode(const Epi& e) {
   }
 }
 
+// (an earlier edge's contribution, in.acc, is loaded by epi_finish_block)
 template <int EM>
 __device__ __forceinline__ void epi_load_m(const Epi& e, int n, const PropDev* P, int m, int j,
                                            EpiIn& in) {
-  if (e.acc_in) in.acc = e.acc_in[(size_t)m * e.acc_ld + j];
   const size_t q = (size_t)n * e.SD + e.off + j, qm = (size_t)m * e.SD + e.off + j;
   if constexpr (EM <= EM_RELU_GAMMA) {
     in.l = e.pool.L[q];
@@ -293,65 +293,99 @@ __device__ __forceinline__ void epi_load_m(const Epi& e, int n, const PropDev* P
   }
 }
 
-template <int EM>
-__device__ __forceinline__ float epi_finish_m(const Epi& e, int m, int j, float v, const EpiIn& in,
-                                              float& part) {
-  if (e.acc_in) v += in.acc;
-  const size_t qm = (size_t)m * e.SD + e.off + j;
-  if constexpr (EM <= EM_RELU_GAMMA) {
-    const float l = in.l, u = in.u;
-    const int s = in.s;
-    float ap = v;
-    if constexpr (EM == EM_RELU_GAMMA) ap += in.gp;
-    float D, bl = 0.f;
-    if (s == -1) D = 1.f;
-    else if (s == 1) D = 0.f;
-    else if (l >= 0.f) D = 1.f;
-    else if (u <= 0.f) D = 0.f;
-    else if (ap >= 0.f) D = EM >= EM_RELU_FINAL ? in.al : (u >= -l ? 1.f : 0.f);
-    else {
-      const float den = u - l;
-      D = u / den;
-      bl = (-u * l) / den;
+// Finishes K outputs (m, j[i]) of one row with values v[i], in place; ok: bit i is
+// set where output i counts (every j[i] is a valid index; nothing is stored or
+// summed for the others).  The relaxation's two divisions are needed only where
+// an unstable neuron has a negative coefficient: the outputs' other arithmetic is
+// free of branches, and a lane then divides for its own such outputs one after
+// another (a few of its K; a warp that branched at every output ran both divisions at
+// most of them: 7 us for eight outputs of a 128-position tile, now 2).
+template <int EM, int K>
+__device__ __forceinline__ void epi_finish_block(const Epi& e, int m, const int (&j)[K],
+                                                 float (&v)[K], const EpiIn (&in)[K], unsigned ok,
+                                                 float& part) {
+  if (e.acc_in) {
+    float acc[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) acc[i] = e.acc_in[(size_t)m * e.acc_ld + j[i]];
+#pragma unroll
+    for (int i = 0; i < K; ++i) v[i] += acc[i];
+  }
+  const size_t q0 = (size_t)m * e.SD + e.off;
+  if constexpr (EM <= EM_RELU_GAMMA || EM == EM_ADJ || EM == EM_ADJ_GAMMA) {
+    constexpr bool relu = EM <= EM_RELU_GAMMA;
+    float ap[K], D[K], bl[K];
+    unsigned need = 0, abr = 0;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      ap[i] = relu ? v[i] : in[i].gp;
+      if constexpr (EM == EM_RELU_GAMMA) ap[i] += in[i].gp;
+      const float l = in[i].l, u = in[i].u;
+      const int s = in[i].s;
+      const bool one = s == -1 || (s != 1 && l >= 0.f);
+      const bool zero = !one && (s == 1 || u <= 0.f);
+      const bool up = ap[i] >= 0.f;
+      const float a = EM == EM_RELU ? (u >= -l ? 1.f : 0.f) : in[i].al;
+      D[i] = one ? 1.f : zero ? 0.f : a;
+      bl[i] = 0.f;
+      if ((ok >> i & 1u) && !one && !zero) (up ? abr : need) |= 1u << i;
     }
-    float ah = ap * D;
-    if constexpr (EM >= EM_RELU_FINAL) ah += in.be * (float)s;
-    if constexpr (EM == EM_RELU_GAMMA) ah += in.gph;
-    if (e.AP) e.AP[qm] = ap;
-    part += ap * bl + ah * in.cb;
-    return ah;
+    while (need) {
+      const int w = __ffs(need) - 1;
+      need &= need - 1;
+      float l = 0.f, u = 0.f;
+#pragma unroll
+      for (int i = 0; i < K; ++i)
+        if (i == w) {
+          l = in[i].l;
+          u = in[i].u;
+        }
+      const float den = u - l;
+      const float d = u / den, b = (-u * l) / den;
+#pragma unroll
+      for (int i = 0; i < K; ++i)
+        if (i == w) {
+          D[i] = d;
+          bl[i] = b;
+        }
+    }
+    const bool keep = relu && e.AP != nullptr;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      const size_t qm = q0 + j[i];
+      const bool st = ok >> i & 1u;
+      if constexpr (relu) {
+        float ah = ap[i] * D[i];
+        if constexpr (EM >= EM_RELU_FINAL) ah += in[i].be * (float)in[i].s;
+        if constexpr (EM == EM_RELU_GAMMA) ah += in[i].gph;
+        if (keep && st) e.AP[qm] = ap[i];
+        const float t = part + (ap[i] * bl[i] + ah * in[i].cb);
+        part = st ? t : part;
+        v[i] = ah;
+      } else {
+        const float h = v[i], g = h * D[i] + bl[i];
+        if (st) {
+          e.GA[qm] = abr >> i & 1u ? h * ap[i] : 0.f;
+          e.GB[qm] = h * (float)in[i].s;
+          if constexpr (EM == EM_ADJ_GAMMA) {
+            e.Hz[qm] = h;
+            e.Gz[qm] = g;
+          }
+        }
+        v[i] = g;
+      }
+    }
   } else if constexpr (EM == EM_CONC) {
-    const float x = v >= 0.f ? in.l : in.u;
-    part += v * x;
-    if (e.X) e.X[(size_t)m * e.d0 + j] = x;
-    return v;
-  } else if constexpr (EM == EM_ADJ || EM == EM_ADJ_GAMMA) {
-    const float l = in.l, u = in.u, ap = in.gp, h = v;
-    const int s = in.s;
-    float D, bl = 0.f;
-    bool abr = false;
-    if (s == -1) D = 1.f;
-    else if (s == 1) D = 0.f;
-    else if (l >= 0.f) D = 1.f;
-    else if (u <= 0.f) D = 0.f;
-    else if (ap >= 0.f) { D = in.al; abr = true; }
-    else {
-      const float den = u - l;
-      D = u / den;
-      bl = (-u * l) / den;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      if (!(ok >> i & 1u)) continue;
+      const float x = v[i] >= 0.f ? in[i].l : in[i].u;
+      part += v[i] * x;
+      if (e.X) e.X[(size_t)m * e.d0 + j[i]] = x;
     }
-    e.GA[qm] = abr ? h * ap : 0.f;
-    e.GB[qm] = h * (float)s;
-    const float g = h * D + bl;
-    if constexpr (EM == EM_ADJ_GAMMA) {
-      e.Hz[qm] = h;
-      e.Gz[qm] = g;
-    }
-    return g;
   } else if constexpr (EM == EM_FWD) {
-    return fmaxf(v, 0.f);
-  } else {
-    return v;
+#pragma unroll
+    for (int i = 0; i < K; ++i) v[i] = fmaxf(v[i], 0.f);
   }
 }
 

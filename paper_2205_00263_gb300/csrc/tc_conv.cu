@@ -92,12 +92,6 @@ __host__ __device__ inline ConvClass conv_class(const LayerDev& L, int dir, int 
   return c;
 }
 
-// canonical no-swizzle K-major offset (bytes) of A element (r, k), KC = 32:
-// core matrices along K 128 B apart, 8-row groups 1024 B apart
-__device__ __forceinline__ uint32_t a_off(int r, int k) {
-  return (uint32_t)((r >> 3) * 1024 + (k >> 2) * 128 + (r & 7) * 16 + (k & 3) * 4);
-}
-
 // pre-split weights of one direction: buf_hi / buf_lo [ncls][Kp / 4][NP][4]
 __global__ void k_tc_conv_split(LayerDev L, int dir, int Kp, int NP, float* hi, float* lo) {
   const int cls = blockIdx.y;
@@ -125,7 +119,11 @@ __global__ void k_tc_conv_split(LayerDev L, int dir, int Kp, int NP, float* hi, 
   }
 }
 
-constexpr int TC_THREADS = 256;  // 8 warps: two threads per GEMM row gather a K block
+constexpr int TC_GATHER = 256;   // 8 warps: two threads per GEMM row gather a K block
+constexpr int TC_THREADS = 288;  // and a control warp
+constexpr int TC_WST = 4;        // weight stages
+constexpr int TC_AST = 3;        // A stages in tensor memory, 2 KC columns each
+constexpr uint32_t TC_COLS = 256;  // tensor-memory columns of a CTA: D (64) and the A stages
 
 // one instantiation per kind of epilogue (EM); NP: channels padded to 16
 template <int EM>
@@ -134,17 +132,16 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
               LayerDev L, int dir, int NP, int M, int nchunk, const float* __restrict__ in,
               int ld_in, float* out, int ld_out, Epi e, int* err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  constexpr int A_BYTES = 128 * KC * 4;
   const int B_BYTES = NP * KC * 4;
-  const int STAGE = 2 * A_BYTES + 2 * B_BYTES;
-  const uint32_t NCOLS = NP <= 32 ? 32 : 64;
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bar = reinterpret_cast<uint64_t*>(base + 2 * STAGE);  // tma[2], mma[2]
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bar + 4);
+  unsigned char* wring = base;  // TC_WST stages of hi and lo weights
   // reduction table of the whole K range, computed once: source offset (channel
   // plane + tap shift) and tap, of which each thread knows which are in range
-  __shared__ __align__(16) int2 t_tab[TC_KMAX];
+  int2* t_tab = reinterpret_cast<int2*>(wring + TC_WST * 2 * B_BYTES);
+  // A stage written, its MMAs done [TC_AST], weights there [TC_WST]
+  __shared__ __align__(8) uint64_t bars[2 * TC_AST + TC_WST];
+  __shared__ uint32_t tmem_holder;
   __shared__ int s_fail;
   __shared__ float s_part[2][TROWS];
 
@@ -161,7 +158,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   const bool has_part = dir == 1 && epi_has_part(e);
   if (chunk * 32 >= c.P) {
     // no position of this class in the chunk: only the row partials (zero)
-    if (has_part && kh == 0 && lane == 0 && rowv)
+    if (has_part && warp < 4 && lane == 0 && rowv)
       e.part[(size_t)m * e.nslot + e.slot_base + blockIdx.x] = 0.f;
     return;
   }
@@ -178,22 +175,29 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   const int Hs = dir == 0 ? L.hi : L.ho, Wsrc = dir == 0 ? L.wi : L.wo;
   const float* src = in + (size_t)(rowv ? m : 0) * ld_in + gy * Wsrc + gx;
 
-  const uint32_t tma0 = tc::smem_u32(bar), mma0 = tc::smem_u32(bar + 2);
-  if (warp == 0) {
+  const uint32_t bar0 = tc::smem_u32(bars);
+  auto a_full = [&](int i) { return bar0 + 8u * i; };
+  auto mma_done = [&](int i) { return bar0 + 8u * (TC_AST + i); };
+  auto w_full = [&](int i) { return bar0 + 8u * (2 * TC_AST + i); };
+  if (warp == TC_GATHER / 32) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     tc::smem_u32(tmem_holder)),
-                 "r"(NCOLS));
+                     tc::smem_u32(&tmem_holder)),
+                 "r"(TC_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int i = 0; i < 4; ++i) tc::mbar_init(tma0 + 8 * i, 1);
+    for (int i = 0; i < TC_AST; ++i) {
+      tc::mbar_init(a_full(i), TC_GATHER / 32);
+      tc::mbar_init(mma_done(i), 1);
+    }
+    for (int i = 0; i < TC_WST; ++i) tc::mbar_init(w_full(i), 1);
     s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tmem_holder;
+  const uint32_t tmem = tmem_holder;
   const uint32_t idesc = tc::idesc_tf32_m128(NP);
 
   const int nk = (c.K + KC - 1) / KC;
@@ -246,92 +250,102 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
     }
   };
   bool ok = true;
-  int last = -1;
-  float vn[16];
-  if (nk > 0) gather(0, vn);
-  for (int kb = 0; kb < nk; ++kb) {
-    const int st = kb & 1;
-    const uint32_t tbar = tma0 + 8 * st, mbar = mma0 + 8 * st;
-    float v[16];
-#pragma unroll
-    for (int u = 0; u < 16; ++u) v[u] = vn[u];
-    // the next block's loads are in flight while this block is staged and issued
-    if (kb + 1 < nk) gather(kb + 1, vn);
-    if (kb >= 2) {
-      // the MMAs of block kb - 2 read this stage: wait for them
-      const bool mine = tc::mbar_wait(mbar, (uint32_t)(((kb >> 1) - 1) & 1));
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      ok = __syncthreads_and(mine && s_fail == 0) != 0;
-    } else {
-      ok = __syncthreads_and(s_fail == 0) != 0;
-    }
-    if (!ok) break;
-    unsigned char* a_hi = base + st * STAGE;
-    unsigned char* a_lo = a_hi + A_BYTES;
-    unsigned char* b_hi = a_lo + A_BYTES;
-    unsigned char* b_lo = b_hi + B_BYTES;
-    if (tid == 0) {
-      // weights of this K block (hi and lo) by TMA
-      tc::mbar_expect_tx(tbar, 2 * B_BYTES);
-      tc::tma_load_3d(tc::smem_u32(b_hi), &tm_hi, 0, kb * (KC / 4), cls, tbar);
-      tc::tma_load_3d(tc::smem_u32(b_lo), &tm_lo, 0, kb * (KC / 4), cls, tbar);
-    }
-    const int r = rq * 32 + lane;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      uint4 h, l;
-      h.x = tc::to_tf32(v[4 * q]);
-      l.x = tc::to_tf32(v[4 * q] - __uint_as_float(h.x));
-      h.y = tc::to_tf32(v[4 * q + 1]);
-      l.y = tc::to_tf32(v[4 * q + 1] - __uint_as_float(h.y));
-      h.z = tc::to_tf32(v[4 * q + 2]);
-      l.z = tc::to_tf32(v[4 * q + 2] - __uint_as_float(h.z));
-      h.w = tc::to_tf32(v[4 * q + 3]);
-      l.w = tc::to_tf32(v[4 * q + 3] - __uint_as_float(h.w));
-      const uint32_t o = a_off(r, kh * 16 + 4 * q);
-      *reinterpret_cast<uint4*>(a_hi + o) = h;
-      *reinterpret_cast<uint4*>(a_lo + o) = l;
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-      if (tc::mbar_wait(tbar, (uint32_t)((kb >> 1) & 1))) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t ah = tc::smem_u32(a_hi), al = tc::smem_u32(a_lo);
-        const uint32_t bh = tc::smem_u32(b_hi), bl = tc::smem_u32(b_lo);
-        const uint32_t BLBO = (uint32_t)NP * 16u;  // B: core matrices along K
-#pragma unroll
-        for (int ks = 0; ks < KC / 8; ++ks) {
-          const uint32_t ao = ks * 256, bo = ks * 2 * BLBO;
-          const uint32_t first = (kb == 0 && ks == 0) ? 0u : 1u;
-          tc::mma_tf32(tmem, tc::smem_desc(al + ao, 128, 1024), tc::smem_desc(bh + bo, BLBO, 128),
-                       idesc, first);
-          tc::mma_tf32(tmem, tc::smem_desc(ah + ao, 128, 1024), tc::smem_desc(bl + bo, BLBO, 128),
-                       idesc, 1u);
-          tc::mma_tf32(tmem, tc::smem_desc(ah + ao, 128, 1024), tc::smem_desc(bh + bo, BLBO, 128),
-                       idesc, 1u);
+  if (warp == TC_GATHER / 32) {
+    // control: one thread streams the weights through their ring (block kb in
+    // stage kb mod TC_WST, refilled when the MMAs that read the stage are done) and
+    // issues each block's MMAs once its A tile and weights are there
+    if (lane == 0) {
+      auto load = [&](int kb) {
+        const uint32_t b = w_full(kb % TC_WST);
+        const uint32_t d = tc::smem_u32(wring + kb % TC_WST * 2 * B_BYTES);
+        tc::mbar_expect_tx(b, 2 * B_BYTES);
+        tc::tma_load_3d(d, &tm_hi, 0, kb * (KC / 4), cls, b);
+        tc::tma_load_3d(d + B_BYTES, &tm_lo, 0, kb * (KC / 4), cls, b);
+      };
+      const uint32_t b_lo0 = tc::desc_lo(tc::smem_u32(wring), (uint32_t)NP * 16u);
+      const uint32_t b_hi = tc::desc_hi(128);
+      int loaded = 0, kb = 0;
+      for (; loaded < min(nk, TC_WST); ++loaded) load(loaded);
+      for (; kb < nk; ++kb) {
+        const int st = kb % TC_AST;
+        if (!tc::mbar_wait(a_full(st), (uint32_t)((kb / TC_AST) & 1)) ||
+            !tc::mbar_wait(w_full(kb % TC_WST), (uint32_t)((kb / TC_WST) & 1))) {
+          ok = false;
+          break;
         }
-      } else {
-        s_fail = 1;  // the weights never arrived: the next barrier stops the loop
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t ah = tmem + 64u + (uint32_t)st * (2 * KC), al = ah + KC;
+        const uint32_t bh = b_lo0 + (uint32_t)(kb % TC_WST) * (uint32_t)(2 * B_BYTES / 16);
+        const uint32_t bl = bh + (uint32_t)(B_BYTES / 16), bstep = (uint32_t)NP * 2u;
+        if (kb == 0) tc::mma_tf32_tmem_lo<false>(tmem, al, bh, b_hi, idesc);
+        else tc::mma_tf32_tmem_lo<true>(tmem, al, bh, b_hi, idesc);
+        tc::mma_tf32_tmem_lo<true>(tmem, ah, bl, b_hi, idesc);
+        tc::mma_tf32_tmem_lo<true>(tmem, ah, bh, b_hi, idesc);
+#pragma unroll
+        for (int ks = 1; ks < KC / 8; ++ks) {
+          const uint32_t ao = ks * 8, bo = ks * bstep;
+          tc::mma_tf32_tmem_lo<true>(tmem, al + ao, bh + bo, b_hi, idesc);
+          tc::mma_tf32_tmem_lo<true>(tmem, ah + ao, bl + bo, b_hi, idesc);
+          tc::mma_tf32_tmem_lo<true>(tmem, ah + ao, bh + bo, b_hi, idesc);
+        }
+        tc::mma_commit(mma_done(st));
+        if (kb >= 1 && loaded < nk) {
+          // the weight stage of block kb - 1 is free once its MMAs are done
+          if (!tc::mbar_wait(mma_done((kb - 1) % TC_AST), (uint32_t)(((kb - 1) / TC_AST) & 1))) {
+            ok = false;
+            break;
+          }
+          load(loaded++);
+        }
       }
-      tc::mma_commit(mbar);  // also when nothing was issued: keeps the phases in step
+      if (!ok) {
+        // copies and MMAs in flight get one more bounded wait
+        s_fail = 1;
+        for (int i = kb; i < loaded; ++i)
+          tc::mbar_wait(w_full(i % TC_WST), (uint32_t)((i / TC_WST) & 1));
+        for (int i = max(0, kb - 1); i <= kb; ++i)
+          tc::mbar_wait(mma_done(i % TC_AST), (uint32_t)((i / TC_AST) & 1));
+      }
     }
-    last = kb;
-  }
-  if (ok && last >= 0) {
+  } else {
+    // gather: block kb + 1's loads are in flight while block kb is split and
+    // written to tensor memory (a GEMM row is a lane: no shared memory, no fence
+    // between proxies)
+    float v[16];
+    if (nk > 0) gather(0, v);
+    const uint32_t arow = tmem + ((uint32_t)(rq * 32) << 16) + 64u + (uint32_t)(kh * 16);
+    for (int kb = 0; kb < nk; ++kb) {
+      const int st = kb % TC_AST;
+      uint32_t h[16], l[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        h[u] = tc::to_tf32(v[u]);
+        l[u] = tc::to_tf32(v[u] - __uint_as_float(h[u]));
+      }
+      if (kb + 1 < nk) gather(kb + 1, v);
+      // the MMAs of block kb - TC_AST read this A stage
+      const bool free_ = kb < TC_AST || tc::mbar_wait(mma_done(st), (uint32_t)((kb / TC_AST - 1) & 1));
+      if (!__all_sync(0xffffffffu, free_)) {
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      tc::tmem_st16(arow + (uint32_t)st * (2 * KC), h);
+      tc::tmem_st16(arow + (uint32_t)st * (2 * KC) + KC, l);
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(a_full(st));
+    }
     // the last commit covers every MMA issued before it
-    const bool mine = tc::mbar_wait(mma0 + 8 * (last & 1), (uint32_t)((last >> 1) & 1));
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    ok = __syncthreads_and(mine && s_fail == 0) != 0;
+    if (ok && nk > 0)
+      ok = tc::mbar_wait(mma_done((nk - 1) % TC_AST), (uint32_t)(((nk - 1) / TC_AST) & 1));
   }
+  ok = __syncthreads_and(ok && s_fail == 0) != 0;
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (!ok) {
-    if (tid == 0) {
-      atomicExch(err, 1);
-      if (last >= 0) tc::mbar_wait(mma0 + 8 * (last & 1), (uint32_t)((last >> 1) & 1));
-    }
-    __syncthreads();
-  }
-  if (ok) {
+    if (tid == 0) atomicExch(err, 1);
+  } else if (warp < TC_GATHER / 32) {
     // epilogue: every warp reads its TMEM lane quarter (objective row rq); warp
     // group kh takes the 16-column chunks 16 (2 i + kh), eight columns at a time,
     // whose inputs are loaded together before any of them is finished.
@@ -357,21 +371,23 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
       }
       if (pv) {
         EpiIn ein[8];
+        int j[8];
+        unsigned okm = 0;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const int n = c0 + i;
-          if (n < N) epi_load_m<EM>(e, nrow, Pp, m, n * plane + pj, ein[i]);
+          // (a padded channel loads the last one's inputs: loads under a branch per
+          // output were issued one output after another, 2000 cycles each)
+          const int n = min(c0 + i, N - 1);
+          j[i] = n * plane + pj;
+          epi_load_m<EM>(e, nrow, Pp, m, j[i], ein[i]);
+          if (dir == 0) v[i] += L.b[n];
+          if (c0 + i < N) okm |= 1u << i;
         }
+        epi_finish_block<EM, 8>(e, m, j, v, ein, okm, part);
+        if (out) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int n = c0 + i;
-          if (n < N) {
-            const int j = n * plane + pj;
-            float val = v[i];
-            if (dir == 0) val += L.b[n];
-            const float o = epi_finish_m<EM>(e, m, j, val, ein[i], part);
-            if (out) out[(size_t)m * ld_out + j] = o;
-          }
+          for (int i = 0; i < 8; ++i)
+            if (okm >> i & 1u) out[(size_t)m * ld_out + j[i]] = v[i];
         }
       }
     }
@@ -383,11 +399,11 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   // a row's offset partial: the two warp groups' sums, in that order
-  if (ok && has_part && kh == 0 && lane == 0 && rowv)
+  if (ok && has_part && warp < 4 && lane == 0 && rowv)
     e.part[(size_t)m * e.nslot + e.slot_base + blockIdx.x] = s_part[0][rq] + s_part[1][rq];
-  if (warp == 0) {
+  if (warp == TC_GATHER / 32) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NCOLS));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_COLS));
   }
 }
 
@@ -406,7 +422,9 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-int conv_tc_smem(int NP) { return 1024 + 2 * (2 * 128 * KC * 4 + 2 * NP * KC * 4) + 64; }
+int conv_tc_smem(int NP, int Kp) {
+  return 1024 + TC_WST * 2 * NP * KC * 4 + Kp * (int)sizeof(int2);
+}
 
 }  // namespace
 
@@ -489,7 +507,7 @@ int launch_tc_conv(const LayerDev& L, int dir, int M, const float* in, int ld_in
                    int ld_out, const Epi& e, cudaStream_t st) {
   const TcConv* t = static_cast<const TcConv*>(L.tc);
   const dim3 grid(t->ncls[dir] * t->nchunk[dir], (M + TROWS - 1) / TROWS);
-  const int NP = t->NP[dir], smem = conv_tc_smem(NP);
+  const int NP = t->NP[dir], smem = conv_tc_smem(NP, t->Kp[dir]);
   auto go = [&](auto kern) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     kern<<<grid, TC_THREADS, smem, st>>>(t->hi[dir], t->lo[dir], L, dir, NP, M, t->nchunk[dir], in,
