@@ -21,6 +21,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "epilogue.cuh"
 #include "mnbab.h"
@@ -72,6 +73,40 @@ __device__ __forceinline__ int f_split(int items) {
   return ks;
 }
 
+// x / d by the rounded-up reciprocal m = ceil(2^32 / d), exact for x d < 2^32 (the
+// fused kernels' indices stay below 2^16, their layers fit in shared memory); a
+// convolution step decodes its item with ten divisions by layer sizes, which took
+// a third of its instructions.
+struct FDiv {
+  unsigned d, m;
+};
+__host__ __device__ inline FDiv f_div_of(int d) {
+  return FDiv{(unsigned)d, d <= 1 ? 0u : 0xffffffffu / (unsigned)d + 1u};
+}
+__device__ __forceinline__ int f_div(int x, FDiv v) {
+  return v.m ? (int)__umulhi((unsigned)x, v.m) : x;
+}
+__device__ __forceinline__ int f_mod(int x, FDiv v) { return x - f_div(x, v) * (int)v.d; }
+
+struct FusedIdx {
+  struct Layer {
+    FDiv pp, w2, s;   // transposed step: first positions, those of a row, stride
+    FDiv p, wo;       // forward step: output positions, their columns
+  } l[MNBAB_MAXR + 2];
+};
+
+static FusedIdx fused_idx(const NetDev& net) {
+  FusedIdx x{};
+  for (int t = 1; t <= net.R; ++t) {
+    const LayerDev& L = net.aff[t];
+    if (L.kind != MNBAB_CONV2D) continue;
+    const int w2 = (L.wi + 2 * L.s - 1) / (2 * L.s) * L.s;
+    x.l[t] = {f_div_of(L.hi * w2), f_div_of(w2), f_div_of(L.s), f_div_of(L.ho * L.wo),
+              f_div_of(L.wo)};
+  }
+  return x;
+}
+
 __device__ __forceinline__ float f_group_sum(float v, int ks) {
   for (int o = ks >> 1; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
@@ -82,12 +117,12 @@ __device__ void f_fc_back(const LayerDev& L, const float* cur, float* nxt) {
   const int din = L.d_in, dout = L.d_out;
   const bool vec = (din & 3) == 0 && (reinterpret_cast<uintptr_t>(L.W) & 15) == 0;
   const int CB = vec ? 4 : 1;
-  const int items = din / CB;
-  const int ks = f_split(items);
+  const int items = vec ? din >> 2 : din;
+  const int ks = f_split(items), lg = __ffs(ks) - 1;
   const int rounds = (items * ks + FT - 1) / FT;
   for (int rr = 0; rr < rounds; ++rr) {
     const int b = rr * FT + threadIdx.x;
-    const int it = b / ks, k0 = b % ks;
+    const int it = b >> lg, k0 = b & (ks - 1);
     const bool act = it < items;
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
     if (act) {
@@ -102,10 +137,13 @@ __device__ void f_fc_back(const LayerDev& L, const float* cur, float* nxt) {
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
             const float a = cur[j + u * ks];
-            a0 = fmaf(a, w[u].x, a0);
-            a1 = fmaf(a, w[u].y, a1);
-            a2 = fmaf(a, w[u].z, a2);
-            a3 = fmaf(a, w[u].w, a3);
+            const float2 aa = make_float2(a, a);
+            const float2 x = fma2(aa, make_float2(w[u].x, w[u].y), make_float2(a0, a1));
+            const float2 y = fma2(aa, make_float2(w[u].z, w[u].w), make_float2(a2, a3));
+            a0 = x.x;
+            a1 = x.y;
+            a2 = y.x;
+            a3 = y.y;
           }
         }
         for (; j < dout; j += ks) {
@@ -133,53 +171,69 @@ __device__ void f_fc_back(const LayerDev& L, const float* cur, float* nxt) {
   }
 }
 
-// Forward through FC layer L: g (d_in) -> h (d_out) = W g + b; one warp per
-// pair of outputs (each load of g serves both rows).
+// NO outputs of a warp (i0, i0 + FT / 32, ...): each load of g serves all of them,
+// and their weight loads are in flight together.  A lane's terms of an output
+// add up in ascending order, then a tree over the lanes.
+template <int NO>
+__device__ __forceinline__ void f_fc_fwd_rows(const LayerDev& L, const float* g, float* h, int i0) {
+  constexpr int NW = FT / 32;
+  const int lane = threadIdx.x & 31, n4 = L.d_in >> 2;
+  const float4* g4 = reinterpret_cast<const float4*>(g);
+  const float4* w[NO];
+  float acc[NO];
+#pragma unroll
+  for (int q = 0; q < NO; ++q) {
+    w[q] = reinterpret_cast<const float4*>(L.W + (size_t)min(i0 + NW * q, L.d_out - 1) * L.d_in);
+    acc[q] = 0.f;
+  }
+  for (int c = lane; c < n4; c += 32) {
+    float4 v[NO];
+#pragma unroll
+    for (int q = 0; q < NO; ++q)
+      v[q] = i0 + NW * q < L.d_out ? __ldg(w[q] + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 x = g4[c];
+#pragma unroll
+    for (int q = 0; q < NO; ++q) {
+      acc[q] = fmaf(v[q].x, x.x, acc[q]);
+      acc[q] = fmaf(v[q].y, x.y, acc[q]);
+      acc[q] = fmaf(v[q].z, x.z, acc[q]);
+      acc[q] = fmaf(v[q].w, x.w, acc[q]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < NO; ++q) {
+    for (int o = 16; o; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+    if (lane == 0 && i0 + NW * q < L.d_out) h[i0 + NW * q] = acc[q] + L.b[i0 + NW * q];
+  }
+}
+
+// Forward through FC layer L: g (d_in) -> h (d_out) = W g + b.  A warp takes up to
+// seven outputs at once (100 outputs of 800 inputs: one round of 44 KB of weight
+// loads in flight; two outputs a warp took four rounds, the last of two warps).
 __device__ void f_fc_fwd(const LayerDev& L, const float* g, float* h) {
   const int din = L.d_in, dout = L.d_out;
+  constexpr int NW = FT / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool vec = (din & 3) == 0 && (reinterpret_cast<uintptr_t>(L.W) & 15) == 0 &&
                    (reinterpret_cast<uintptr_t>(g) & 15) == 0;
-  for (int i = 2 * warp; i < dout; i += FT / 16) {
+  if (vec) {
+    for (int i0 = warp; i0 < dout; i0 += 7 * NW) {
+      const int left = (dout - i0 + warp + NW - 1) / NW;  // outputs of warp 0 from here on
+      if (left <= 1) f_fc_fwd_rows<1>(L, g, h, i0);
+      else if (left <= 2) f_fc_fwd_rows<2>(L, g, h, i0);
+      else if (left <= 4) f_fc_fwd_rows<4>(L, g, h, i0);
+      else f_fc_fwd_rows<7>(L, g, h, i0);
+    }
+    return;
+  }
+  for (int i = 2 * warp; i < dout; i += 2 * NW) {
     const bool two = i + 1 < dout;
     const int i1 = two ? i + 1 : i;
     float acc0 = 0.f, acc1 = 0.f;
-    if (vec) {
-      const float4* w0 = reinterpret_cast<const float4*>(L.W + (size_t)i * din);
-      const float4* w1 = reinterpret_cast<const float4*>(L.W + (size_t)i1 * din);
-      const float4* g4 = reinterpret_cast<const float4*>(g);
-      const int n4 = din >> 2;
-      for (int c0 = lane; c0 < n4; c0 += 32 * 2) {
-        float4 a[2], b[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int c = c0 + 32 * u;
-          const bool in = c < n4;
-          a[u] = in ? __ldg(w0 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-          b[u] = in ? __ldg(w1 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int c = c0 + 32 * u;
-          if (c < n4) {
-            const float4 x = g4[c];
-            acc0 = fmaf(a[u].x, x.x, acc0);
-            acc0 = fmaf(a[u].y, x.y, acc0);
-            acc0 = fmaf(a[u].z, x.z, acc0);
-            acc0 = fmaf(a[u].w, x.w, acc0);
-            acc1 = fmaf(b[u].x, x.x, acc1);
-            acc1 = fmaf(b[u].y, x.y, acc1);
-            acc1 = fmaf(b[u].z, x.z, acc1);
-            acc1 = fmaf(b[u].w, x.w, acc1);
-          }
-        }
-      }
-    } else {
-      for (int j = lane; j < din; j += 32) {
-        const float x = g[j];
-        acc0 = fmaf(__ldg(L.W + (size_t)i * din + j), x, acc0);
-        acc1 = fmaf(__ldg(L.W + (size_t)i1 * din + j), x, acc1);
-      }
+    for (int j = lane; j < din; j += 32) {
+      const float x = g[j];
+      acc0 = fmaf(__ldg(L.W + (size_t)i * din + j), x, acc0);
+      acc1 = fmaf(__ldg(L.W + (size_t)i1 * din + j), x, acc1);
     }
     for (int o = 16; o; o >>= 1) {
       acc0 += __shfl_xor_sync(0xffffffffu, acc0, o);
@@ -228,35 +282,38 @@ __device__ inline void f_stage(float* dst, const float* src, int rows, int w, in
 // one row, s columns apart: both have the taps kh = (ih + p) mod s (+ s, ...),
 // kw = (iw + p) mod s (+ s, ...), the second at ow + 1, so every staged
 // weight load serves both positions.
-__device__ void f_conv_back(const LayerDev& L, const float* cur, float* nxt, const float* Wb) {
+__device__ void f_conv_back(const LayerDev& L, const FusedIdx::Layer& X, const float* cur, float* nxt,
+                            const float* Wb) {
   const int CB = (L.ci & 3) == 0 ? 4 : 1;
   const int S = L.s;
-  const int W2 = (L.wi + 2 * S - 1) / (2 * S) * S;  // first positions per row (a few past the edge)
-  const int ngr = L.ci / CB, P = L.hi * L.wi, hwo = L.ho * L.wo, PP = L.hi * W2;
+  const int W2 = (int)X.w2.d;  // first positions per row (a few past the edge)
+  const int ngr = CB == 4 ? L.ci >> 2 : L.ci, P = L.hi * L.wi, hwo = L.ho * L.wo;
+  const int PP = (int)X.pp.d;
   const int items = PP * ngr;
-  const int ks = f_split(items);
+  const int ks = f_split(items), lg = __ffs(ks) - 1;
   const int rounds = (items * ks + FT - 1) / FT;
   const size_t wco = (size_t)f_wb_stride(L);
   for (int rr = 0; rr < rounds; ++rr) {
     const int b = rr * FT + threadIdx.x;
-    const int it = b / ks, k0 = b % ks;
+    const int it = b >> lg, k0 = b & (ks - 1);
     bool act = it < items;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-    float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f;
+    const float2 z2 = make_float2(0.f, 0.f);
+    float2 a01 = z2, a23 = z2, c01 = z2, c23 = z2;
     int grp = 0, ih = 0, iw = 0;
     bool two = false;
     if (act) {
-      grp = it / PP;
-      const int q = it % PP;
-      ih = q / W2;
-      const int qw = q % W2;
-      iw = (qw / S) * 2 * S + qw % S;
+      grp = f_div(it, X.pp);
+      const int q = it - grp * PP;
+      ih = f_div(q, X.w2);
+      const int qw = q - ih * W2, qs = f_div(qw, X.s);
+      iw = qs * S + qw;
       act = iw < L.wi;
       two = iw + S < L.wi;
     }
     if (act) {
-      const int kh0 = (ih + L.p) % S, kw0 = (iw + L.p) % S;
-      const int oh0 = (ih + L.p - kh0) / S, ow0 = (iw + L.p - kw0) / S;
+      const int oh0 = f_div(ih + L.p, X.s), ow0 = f_div(iw + L.p, X.s);
+      const int kh0 = ih + L.p - oh0 * S, kw0 = iw + L.p - ow0 * S;
+      const int da = ks * hwo, dw = ks * (int)wco, n = (L.co - k0 + ks - 1) >> lg;
       for (int kh = kh0, oh = oh0; kh < L.k && oh >= 0; kh += S, --oh) {
         if (oh >= L.ho) continue;
         // the second position's ow is ow + 1, valid down to ow = -1
@@ -264,34 +321,41 @@ __device__ void f_conv_back(const LayerDev& L, const float* cur, float* nxt, con
           const bool ok0 = ow >= 0 && ow < L.wo;
           const bool ok1 = two && ow + 1 < L.wo;
           if (!ok0 && !ok1) continue;
-          const float* ap = cur + oh * L.wo + ow;
-          const float* wp = Wb + (size_t)(kh * L.k + kw) * L.ci + grp * CB;
-          if (CB == 4) {
-#pragma unroll 2
-            for (int co = k0; co < L.co; co += ks) {
-              const float v0 = ok0 ? ap[co * hwo] : 0.f;
-              const float v1 = ok1 ? ap[co * hwo + 1] : 0.f;
-              const float4 w = *reinterpret_cast<const float4*>(wp + co * wco);
-              a0 = fmaf(v0, w.x, a0);
-              a1 = fmaf(v0, w.y, a1);
-              a2 = fmaf(v0, w.z, a2);
-              a3 = fmaf(v0, w.w, a3);
-              c0 = fmaf(v1, w.x, c0);
-              c1 = fmaf(v1, w.y, c1);
-              c2 = fmaf(v1, w.z, c2);
-              c3 = fmaf(v1, w.w, c3);
+          // a position without this tap reads the other's coefficient as zero
+          const float* p0 = cur + oh * L.wo + ow + (ok0 ? 0 : 1) + k0 * hwo;
+          const float* p1 = p0 + (ok0 && ok1 ? 1 : 0);
+          const float* wp = Wb + (size_t)(kh * L.k + kw) * L.ci + grp * CB + k0 * wco;
+          auto run = [&](auto all_) {
+            constexpr bool all = decltype(all_)::value;
+            if (CB == 4) {
+#pragma unroll 4
+              for (int i = 0; i < n; ++i, p0 += da, p1 += da, wp += dw) {
+                const float v0 = all || ok0 ? *p0 : 0.f;
+                const float v1 = all || ok1 ? *p1 : 0.f;
+                const float4 w = *reinterpret_cast<const float4*>(wp);
+                a01 = fma2(make_float2(v0, v0), make_float2(w.x, w.y), a01);
+                a23 = fma2(make_float2(v0, v0), make_float2(w.z, w.w), a23);
+                c01 = fma2(make_float2(v1, v1), make_float2(w.x, w.y), c01);
+                c23 = fma2(make_float2(v1, v1), make_float2(w.z, w.w), c23);
+              }
+            } else {
+#pragma unroll 8
+              for (int i = 0; i < n; ++i, p0 += da, p1 += da, wp += dw) {
+                const float v0 = all || ok0 ? *p0 : 0.f;
+                const float v1 = all || ok1 ? *p1 : 0.f;
+                const float w = *wp;
+                a01.x = fmaf(v0, w, a01.x);
+                c01.x = fmaf(v1, w, c01.x);
+              }
             }
-          } else {
-#pragma unroll 2
-            for (int co = k0; co < L.co; co += ks) {
-              const float w = wp[co * wco];
-              a0 = fmaf(ok0 ? ap[co * hwo] : 0.f, w, a0);
-              c0 = fmaf(ok1 ? ap[co * hwo + 1] : 0.f, w, c0);
-            }
-          }
+          };
+          if (ok0 && ok1) run(std::true_type());
+          else run(std::false_type());
         }
       }
     }
+    float a0 = a01.x, a1 = a01.y, a2 = a23.x, a3 = a23.y;
+    float c0 = c01.x, c1 = c01.y, c2 = c23.x, c3 = c23.y;
     a0 = f_group_sum(a0, ks);
     c0 = f_group_sum(c0, ks);
     if (CB == 4) {
@@ -327,49 +391,55 @@ __device__ void f_conv_back(const LayerDev& L, const float* cur, float* nxt, con
 // CB output channels of one position: each input load serves CB channels (the
 // weight loads of a warp are mostly broadcasts, the input loads are not).
 template <int CB>
-__device__ void f_conv_fwd_cb(const LayerDev& L, const float* g, float* h, const float* Wf) {
-  const int ngr = L.co / CB, P = L.ho * L.wo, hwi = L.hi * L.wi;
+__device__ void f_conv_fwd_cb(const LayerDev& L, const FusedIdx::Layer& X, const float* g, float* h,
+                              const float* Wf) {
+  const int ngr = L.co / CB, P = (int)X.p.d, hwi = L.hi * L.wi;
   const int items = P * ngr;
-  const int ks = f_split(items);
+  const int ks = f_split(items), lg = __ffs(ks) - 1;
   const int rounds = (items * ks + FT - 1) / FT;
   for (int rr = 0; rr < rounds; ++rr) {
     const int b = rr * FT + threadIdx.x;
-    const int it = b / ks, k0 = b % ks;
+    const int it = b >> lg, k0 = b & (ks - 1);
     const bool act = it < items;
-    float a[CB];
+    constexpr int C2 = CB >= 4 ? CB / 2 : 1;
+    float2 acc[C2];
 #pragma unroll
-    for (int u = 0; u < CB; ++u) a[u] = 0.f;
+    for (int u = 0; u < C2; ++u) acc[u] = make_float2(0.f, 0.f);
     int grp = 0, pos = 0;
     if (act) {
-      grp = it / P;
-      pos = it % P;
-      const int oh = pos / L.wo, ow = pos % L.wo;
+      grp = f_div(it, X.p);
+      pos = it - grp * P;
+      const int oh = f_div(pos, X.wo), ow = pos - oh * L.wo;
       const int ih0 = oh * L.s - L.p, iw0 = ow * L.s - L.p;
       const int kh_lo = max(0, -ih0), kh_hi = min(L.k, L.hi - ih0);
       const int kw_lo = max(0, -iw0), kw_hi = min(L.k, L.wi - iw0);
+      const int ws = f_wf_stride(L), nkw = kw_hi - kw_lo;
       for (int ci = k0; ci < L.ci; ci += ks) {
-        const float* gp = g + ci * hwi;
-        const float* wc = Wf + (size_t)ci * f_wf_stride(L) + grp * CB;
-        for (int kh = kh_lo; kh < kh_hi; ++kh)
+        const float* gr = g + ci * hwi + (ih0 + kh_lo) * L.wi + iw0 + kw_lo;
+        const float* wr = Wf + ci * ws + (kh_lo * L.k + kw_lo) * L.co + grp * CB;
+        for (int kh = kh_lo; kh < kh_hi; ++kh, gr += L.wi, wr += L.k * L.co) {
+          const float* wp = wr;
 #pragma unroll 4
-          for (int kw = kw_lo; kw < kw_hi; ++kw) {
-            const float v = gp[(ih0 + kh) * L.wi + iw0 + kw];
-            const float* wp = wc + (size_t)(kh * L.k + kw) * L.co;
+          for (int i = 0; i < nkw; ++i, wp += L.co) {
+            const float v = gr[i];
             if (CB >= 4) {
 #pragma unroll
               for (int q = 0; q < CB / 4; ++q) {
                 const float4 w = *reinterpret_cast<const float4*>(wp + 4 * q);
-                a[4 * q] = fmaf(v, w.x, a[4 * q]);
-                a[4 * q + 1] = fmaf(v, w.y, a[4 * q + 1]);
-                a[4 * q + 2] = fmaf(v, w.z, a[4 * q + 2]);
-                a[4 * q + 3] = fmaf(v, w.w, a[4 * q + 3]);
+                acc[(2 * q) % C2] = fma2(make_float2(v, v), make_float2(w.x, w.y), acc[(2 * q) % C2]);
+                acc[(2 * q + 1) % C2] =
+                    fma2(make_float2(v, v), make_float2(w.z, w.w), acc[(2 * q + 1) % C2]);
               }
             } else {
-              a[0] = fmaf(v, wp[0], a[0]);
+              acc[0].x = fmaf(v, wp[0], acc[0].x);
             }
           }
+        }
       }
     }
+    float a[CB];
+#pragma unroll
+    for (int u = 0; u < CB; ++u) a[u] = u & 1 ? acc[u / 2].y : acc[u / 2].x;
 #pragma unroll
     for (int u = 0; u < CB; ++u) a[u] = f_group_sum(a[u], ks);
     if (act && k0 == 0) {
@@ -380,10 +450,11 @@ __device__ void f_conv_fwd_cb(const LayerDev& L, const float* g, float* h, const
   }
 }
 
-__device__ void f_conv_fwd(const LayerDev& L, const float* g, float* h, const float* Wf) {
-  if ((L.co & 7) == 0) f_conv_fwd_cb<8>(L, g, h, Wf);
-  else if ((L.co & 3) == 0) f_conv_fwd_cb<4>(L, g, h, Wf);
-  else f_conv_fwd_cb<1>(L, g, h, Wf);
+__device__ void f_conv_fwd(const LayerDev& L, const FusedIdx::Layer& X, const float* g, float* h,
+                           const float* Wf) {
+  if ((L.co & 7) == 0) f_conv_fwd_cb<8>(L, X, g, h, Wf);
+  else if ((L.co & 3) == 0) f_conv_fwd_cb<4>(L, X, g, h, Wf);
+  else f_conv_fwd_cb<1>(L, X, g, h, Wf);
 }
 
 
@@ -415,11 +486,9 @@ struct FusedTc {
 // shared-memory floats of layer t's first weight region: the staged Wb, or
 // for the tensor-core layer its B tile (hi and lo) and later its Z
 __host__ __device__ inline int ftc_wb_region(const LayerDev& L, int t, const FusedTc& ft) {
-  const int wb = f_wb_floats(L);
-  if (t != ft.t) return wb;
+  if (t != ft.t) return f_wb_floats(L);
   const int z = (ft.RK * ft.zs + 3) / 4 * 4, b = 2 * ft.Np * ft.Kp;
-  const int m = z > b ? z : b;
-  return wb > m ? wb : m;
+  return z > b ? z : b;
 }
 
 // A (hi and lo) into tensor memory: warp w writes lanes 32 (w mod 4) .. + 31
@@ -443,6 +512,53 @@ __device__ void ftc_load_a(const FusedTc& ft, const LayerDev& L, uint32_t tmem) 
                  v);
   }
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+// nxt from Z, at most TAPS taps per dimension and stride class.  One item per
+// (channel, input row, column residue mod s); its columns share the row taps (kh, oy)
+// and the column taps kw with ox = base + i for the i-th column of the residue
+// class.  Taps are summed in (kh, kw) order.
+template <int TAPS>
+__device__ __forceinline__ void ftc_gather(const FusedTc& ft, const LayerDev& L, float* nxt,
+                                           const float* Z) {
+  const int S = L.s, HW = L.hi * L.wi, kk = L.k * L.k;
+  const int items = L.ci * L.hi * S;
+  for (int it = threadIdx.x; it < items; it += FT) {
+    const int rx = it % S, y = (it / S) % L.hi, c = it / (S * L.hi);
+    // row taps kh = kh0 + a s (valid: inside the kernel, oy in range) and
+    // column taps kw = kw0 + b s
+    const int kh0 = (y + L.p) % S, kw0 = (rx + L.p) % S;
+    const float* z[TAPS][TAPS];
+    int base[TAPS];
+    bool rv[TAPS], cv[TAPS];
+#pragma unroll
+    for (int b = 0; b < TAPS; ++b) {
+      const int kw = kw0 + b * S;
+      cv[b] = kw < L.k;
+      base[b] = (rx + L.p - kw) / S;  // exact: rx + p - kw is a multiple of s
+    }
+#pragma unroll
+    for (int a = 0; a < TAPS; ++a) {
+      const int kh = kh0 + a * S, ty = y + L.p - kh;
+      rv[a] = kh < L.k && ty >= 0 && ty / S < L.ho;
+      const int zrow = (c * kk + kh * L.k) * ft.zs + (rv[a] ? (ty / S) * L.wo : 0);
+#pragma unroll
+      for (int b = 0; b < TAPS; ++b) z[a][b] = Z + zrow + (kw0 + b * S) * ft.zs + base[b];
+    }
+    float* out = nxt + c * HW + y * L.wi;
+    for (int x = rx, i = 0; x < L.wi; x += S, ++i) {
+      float acc = 0.f;
+#pragma unroll
+      for (int a = 0; a < TAPS; ++a) {
+#pragma unroll
+        for (int b = 0; b < TAPS; ++b) {
+          const int ox = base[b] + i;
+          if (rv[a] && cv[b] && ox >= 0 && ox < L.wo) acc += z[a][b][i];
+        }
+      }
+      out[x] = acc;
+    }
+  }
 }
 
 // cur [co][ho][wo] -> nxt [ci][hi][wi]; the B tile and then Z in the region
@@ -472,16 +588,18 @@ __device__ bool ftc_back(const FusedTc& ft, const LayerDev& L, const float* cur,
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t idesc = tc::idesc_tf32_m128(ft.Np);
     const uint32_t bh = tc::smem_u32(bhi), bl = tc::smem_u32(blo);
-    for (int i = 0; i < ft.Mt; ++i) {
-      const uint32_t d = tmem + (uint32_t)(ft.dcol + i * ft.Np);
-      for (int ks = 0; ks < ft.Kp / 8; ++ks) {
-        const uint32_t ah = tmem + (uint32_t)(i * 2 * ft.Kp + ks * 8);
-        const uint32_t bo = (uint32_t)ks * 256u;
-        tc::mma_tf32_tmem_a(d, ah + (uint32_t)ft.Kp, tc::smem_desc(bh + bo, 128, sbo), idesc,
+    // the tiles' products alternate: each accumulates on its own predecessor
+    for (int ks = 0; ks < ft.Kp / 8; ++ks) {
+      const uint32_t bo = (uint32_t)ks * 256u;
+      const uint64_t dh = tc::smem_desc(bh + bo, 128, sbo), dl = tc::smem_desc(bl + bo, 128, sbo);
+      const uint32_t a = tmem + (uint32_t)(ks * 8), d = tmem + (uint32_t)ft.dcol;
+      for (int i = 0; i < ft.Mt; ++i)
+        tc::mma_tf32_tmem_a(d + (uint32_t)(i * ft.Np), a + (uint32_t)((2 * i + 1) * ft.Kp), dh, idesc,
                             ks > 0 ? 1u : 0u);
-        tc::mma_tf32_tmem_a(d, ah, tc::smem_desc(bl + bo, 128, sbo), idesc, 1u);
-        tc::mma_tf32_tmem_a(d, ah, tc::smem_desc(bh + bo, 128, sbo), idesc, 1u);
-      }
+      for (int i = 0; i < ft.Mt; ++i)
+        tc::mma_tf32_tmem_a(d + (uint32_t)(i * ft.Np), a + (uint32_t)(2 * i * ft.Kp), dl, idesc, 1u);
+      for (int i = 0; i < ft.Mt; ++i)
+        tc::mma_tf32_tmem_a(d + (uint32_t)(i * ft.Np), a + (uint32_t)(2 * i * ft.Kp), dh, idesc, 1u);
     }
     tc::mma_commit(bar);
   }
@@ -512,42 +630,10 @@ __device__ bool ftc_back(const FusedTc& ft, const LayerDev& L, const float* cur,
     return false;
   }
   phase ^= 1u;
-  // gather: one item per (channel, input row, column residue mod s); its
-  // columns share the row taps (kh, oy) and the column taps kw with ox = base + i
-  // for the i-th column of the residue class.  Taps are summed in (kh, kw) order.
-  const int S = L.s, HW = L.hi * L.wi, kk = L.k * L.k;
-  const int items = L.ci * L.hi * S;
-  for (int it = threadIdx.x; it < items; it += FT) {
-    const int rx = it % S, y = (it / S) % L.hi, c = it / (S * L.hi);
-    // row taps kh = kh0 + a s (valid: inside the kernel, oy in range) and
-    // column taps kw = kw0 + b s
-    const int kh0 = (y + L.p) % S, kw0 = (rx + L.p) % S;
-    int zrow[FTC_TAPS], kwz[FTC_TAPS], base[FTC_TAPS];
-    bool rv[FTC_TAPS], cv[FTC_TAPS];
-#pragma unroll
-    for (int a = 0; a < FTC_TAPS; ++a) {
-      const int kh = kh0 + a * S, ty = y + L.p - kh;
-      rv[a] = kh < L.k && ty >= 0 && ty / S < L.ho;
-      zrow[a] = (c * kk + kh * L.k) * ft.zs + (rv[a] ? (ty / S) * L.wo : 0);
-      const int kw = kw0 + a * S;
-      cv[a] = kw < L.k;
-      kwz[a] = kw * ft.zs;
-      base[a] = (rx + L.p - kw) / S;  // exact: rx + p - kw is a multiple of s
-    }
-    float* out = nxt + c * HW + y * L.wi;
-    for (int x = rx, i = 0; x < L.wi; x += S, ++i) {
-      float acc = 0.f;
-#pragma unroll
-      for (int a = 0; a < FTC_TAPS; ++a) {
-#pragma unroll
-        for (int b = 0; b < FTC_TAPS; ++b) {
-          const int ox = base[b] + i;
-          if (rv[a] && cv[b] && ox >= 0 && ox < L.wo) acc += Z[zrow[a] + kwz[b] + ox];
-        }
-      }
-      out[x] = acc;
-    }
-  }
+  const int taps = (L.k + L.s - 1) / L.s;
+  if (taps <= 1) ftc_gather<1>(ft, L, nxt, Z);
+  else if (taps == 2) ftc_gather<2>(ft, L, nxt, Z);
+  else ftc_gather<FTC_TAPS>(ft, L, nxt, Z);
   return true;
 }
 
@@ -556,8 +642,9 @@ __device__ bool ftc_back(const FusedTc& ft, const LayerDev& L, const float* cur,
 // two CTAs per SM: at most 64 registers a thread
 __global__ void __launch_bounds__(FT, 2) k_opt_chain(NetDev net, PoolDev pool, const PropDev* props,
                                                   const int* row_node, const int* row_j,
-                                                  FusedHP hp, float* AP_out, float* GB_out,
-                                                  int maxw, FusedTc ft, int* err,
+                                                  FusedHP hp, float* AP_out, float* GA_out,
+                                                  float* GB_out, int maxw, FusedTc ft, FusedIdx X,
+                                                  int use_list, int* err,
                                                   const float* __restrict__ skip_lb) {
   extern __shared__ __align__(16) float fsm[];
   __shared__ float red[32];
@@ -609,6 +696,10 @@ __global__ void __launch_bounds__(FT, 2) k_opt_chain(NetDev net, PoolDev pool, c
   // change): 0 inactive, 1 active, 2 unstable and unsplit, 3 split with S = -1
   // (zhat >= 0), 4 split with S = +1 (zhat <= 0)
   unsigned char* code = reinterpret_cast<unsigned char*>(Xs + ((d0 + 3) & ~3));
+  // neurons with a parameter to step (code >= 2), in any order; a tenth of them
+  // all in the small convolution network
+  unsigned short* list = reinterpret_cast<unsigned short*>(code + SDp);
+  __shared__ int n_list;
   auto wsm = [&](int t) {  // staged weights of conv layer t
     int o = 0;
     for (int u = 1; u < t; ++u)
@@ -621,6 +712,12 @@ __global__ void __launch_bounds__(FT, 2) k_opt_chain(NetDev net, PoolDev pool, c
   const PropDev& P = props[pool.prop[n]];
   const size_t nb = (size_t)n * SD;
   float* GBs = GB_out + (size_t)m * SD;  // d lb / d beta
+  // the upper line of each unstable neuron, zhat slope + intercept, fixed like its
+  // code (a' goes to AP_out only after the last sweep)
+  float* SLs = AP_out + (size_t)m * SD;
+  float* ICs = GA_out + (size_t)m * SD;
+  if (threadIdx.x == 0) n_list = 0;
+  __syncthreads();
   // Adam moments restart per node
   for (int i = threadIdx.x; i < SD; i += FT) {
     pool.MA[nb + i] = 0.f;
@@ -628,7 +725,15 @@ __global__ void __launch_bounds__(FT, 2) k_opt_chain(NetDev net, PoolDev pool, c
     pool.MB[nb + i] = 0.f;
     pool.VB[nb + i] = 0.f;
     const int sv = pool.S[nb + i];
-    code[i] = sv == -1 ? 3 : sv == 1 ? 4 : pool.L[nb + i] >= 0.f ? 1 : pool.U[nb + i] <= 0.f ? 0 : 2;
+    const float l = pool.L[nb + i], u = pool.U[nb + i];
+    const int cd = sv == -1 ? 3 : sv == 1 ? 4 : l >= 0.f ? 1 : u <= 0.f ? 0 : 2;
+    code[i] = (unsigned char)cd;
+    if (cd == 2) {
+      const float den = u - l;
+      SLs[i] = u / den;
+      ICs[i] = (-u * l) / den;
+    }
+    if (use_list && cd >= 2) list[atomicAdd(&n_list, 1)] = (unsigned short)i;
   }
   const int dR = net.d[R];
   for (int step = 0; step <= hp.steps; ++step) {
@@ -654,31 +759,18 @@ __global__ void __launch_bounds__(FT, 2) k_opt_chain(NetDev net, PoolDev pool, c
           ap[k] = j < dt ? cur[j] : 0.f;
           v0[k] = v1[k] = 0.f;
           const size_t q = nb + off + j;
-          if (cd[k] == 2) {
-            v0[k] = ap[k] >= 0.f ? pool.ALPHA[q] : pool.L[q];
-            if (ap[k] < 0.f) v1[k] = pool.U[q];
-          } else if (cd[k] >= 3) {
-            v0[k] = pool.BETA[q];
-          }
+          // slope and intercept of the line taken, or beta
+          const bool lower = cd[k] == 2 && !(ap[k] >= 0.f);
+          const float* src = cd[k] >= 3 ? pool.BETA + q : lower ? SLs + off + j : pool.ALPHA + q;
+          if (cd[k] >= 2) v0[k] = *src;
+          if (lower) v1[k] = ICs[off + j];
         }
 #pragma unroll
         for (int k = 0; k < FU; ++k) {
           const int j = j0 + k * FT;
           if (j >= dt) break;
-          float D, bl = 0.f, bt = 0.f;
-          if (cd[k] == 2) {
-            if (ap[k] >= 0.f) {
-              D = v0[k];
-            } else {
-              const float l = v0[k], u = v1[k];
-              const float den = u - l;
-              D = u / den;
-              bl = (-u * l) / den;
-            }
-          } else {
-            D = (cd[k] == 1 || cd[k] == 3) ? 1.f : 0.f;
-            if (cd[k] >= 3) bt = v0[k] * (cd[k] == 3 ? -1.f : 1.f);
-          }
+          const float D = cd[k] == 2 ? v0[k] : (cd[k] & 1) ? 1.f : 0.f, bl = v1[k];
+          const float bt = cd[k] >= 3 ? v0[k] * (cd[k] == 3 ? -1.f : 1.f) : 0.f;
           const float ah = ap[k] * D + bt;
           APs[off + j] = ap[k];
           part += ap[k] * bl + ah * bias[j];
@@ -695,7 +787,7 @@ __global__ void __launch_bounds__(FT, 2) k_opt_chain(NetDev net, PoolDev pool, c
           break;
         }
       } else {
-        f_conv_back(L, cur, nxt, wsm(t));
+        f_conv_back(L, X.l[t], cur, nxt, wsm(t));
       }
       __syncthreads();
       float* tmp = cur;
@@ -731,7 +823,7 @@ __global__ void __launch_bounds__(FT, 2) k_opt_chain(NetDev net, PoolDev pool, c
       __syncthreads();
       const LayerDev& L = net.aff[t];
       if (L.kind == MNBAB_FC) f_fc_fwd(L, g, h);
-      else f_conv_fwd(L, g, h, wsm(t) + ftc_wb_region(L, t, ft));
+      else f_conv_fwd(L, X.l[t], g, h, wsm(t) + ftc_wb_region(L, t, ft));
       __syncthreads();
       const int dt = net.d[t], off = net.off[t];
       for (int j0 = threadIdx.x; j0 < dt; j0 += FU * FT) {
@@ -743,11 +835,9 @@ __global__ void __launch_bounds__(FT, 2) k_opt_chain(NetDev net, PoolDev pool, c
           cdk[k] = j < dt ? code[off + j] : 0;
           apk[k] = j < dt ? APs[off + j] : 0.f;
           v0[k] = v1[k] = 0.f;
-          if (cdk[k] == 2) {
-            const size_t q = nb + off + j;
-            v0[k] = apk[k] >= 0.f ? pool.ALPHA[q] : pool.L[q];
-            if (apk[k] < 0.f) v1[k] = pool.U[q];
-          }
+          const bool lower = cdk[k] == 2 && !(apk[k] >= 0.f);
+          if (cdk[k] == 2) v0[k] = *(lower ? SLs + off + j : pool.ALPHA + nb + off + j);
+          if (lower) v1[k] = ICs[off + j];
         }
 #pragma unroll
         for (int k = 0; k < FU; ++k) {
@@ -756,23 +846,12 @@ __global__ void __launch_bounds__(FT, 2) k_opt_chain(NetDev net, PoolDev pool, c
           const int cd = cdk[k];
           const float ap = apk[k];
           const float hv = h[j];
-          float D, bl = 0.f, ga = 0.f, gb = 0.f;
-          if (cd == 2) {
-            if (ap >= 0.f) {
-              D = v0[k];
-              ga = hv * ap;
-            } else {
-              const float l = v0[k], u = v1[k];
-              const float den = u - l;
-              D = u / den;
-              bl = (-u * l) / den;
-            }
-          } else {
-            D = (cd == 1 || cd == 3) ? 1.f : 0.f;
-            if (cd >= 3) {
-              gb = hv * (cd == 3 ? -1.f : 1.f);
-              GBs[off + j] = gb;  // row scratch in global memory (L2-resident)
-            }
+          const float D = cd == 2 ? v0[k] : (cd & 1) ? 1.f : 0.f, bl = v1[k];
+          const float ga = cd == 2 && ap >= 0.f ? hv * ap : 0.f;
+          float gb = 0.f;
+          if (cd >= 3) {
+            gb = hv * (cd == 3 ? -1.f : 1.f);
+            GBs[off + j] = gb;  // row scratch in global memory (L2-resident)
           }
           APs[off + j] = ga;
           gm = fmaxf(gm, fmaxf(fabsf(ga), fabsf(gb)));
@@ -790,13 +869,16 @@ __global__ void __launch_bounds__(FT, 2) k_opt_chain(NetDev net, PoolDev pool, c
     // zero gradient at every step, so their (zero-moment) updates are identities
     // FA parameters per thread at a time: all their loads (parameter, both
     // moments, gradient) are issued before the first update
-    for (int i0 = threadIdx.x; i0 < SD; i0 += FA * FT) {
-      int cd[FA];
+    const int np = use_list ? n_list : SD;
+    for (int i0 = threadIdx.x; i0 < np; i0 += FA * FT) {
+      int cd[FA], at[FA];
       float th[FA], mo[FA], ve[FA], gr[FA];
 #pragma unroll
       for (int k = 0; k < FA; ++k) {
-        const int i = i0 + k * FT;
-        cd[k] = i < SD ? code[i] : 0;
+        const int e = i0 + k * FT;
+        const int i = e >= np ? 0 : use_list ? list[e] : e;
+        at[k] = i;
+        cd[k] = e < np ? code[i] : 0;
         th[k] = mo[k] = ve[k] = gr[k] = 0.f;
         const size_t q = nb + i;
         if (cd[k] == 2) {
@@ -814,7 +896,7 @@ __global__ void __launch_bounds__(FT, 2) k_opt_chain(NetDev net, PoolDev pool, c
 #pragma unroll
       for (int k = 0; k < FA; ++k) {
         if (cd[k] < 2) continue;
-        const size_t q = nb + i0 + k * FT;
+        const size_t q = nb + at[k];
         float g = gr[k];
         if (fabsf(g) <= thr) g = 0.f;
         if (cd[k] == 2) {
@@ -1073,7 +1155,7 @@ static int sweep_wfloats(const NetDev& net, int t0) {
 __global__ void __launch_bounds__(FT) k_attack_chain(NetDev net, const PropDev* props, int prop,
                                                      const float* starts, int n_starts,
                                                      int steps, float* best_out,
-                                                     float* bx_out, int maxw) {
+                                                     float* bx_out, int maxw, FusedIdx IX) {
   extern __shared__ __align__(16) float fsm[];
   __shared__ float red[32];
   __shared__ int improved;
@@ -1114,7 +1196,7 @@ __global__ void __launch_bounds__(FT) k_attack_chain(NetDev net, const PropDev* 
       float* h = (t & 1) ? B0 : B1;
       const LayerDev& L = net.aff[t];
       if (L.kind == MNBAB_FC) f_fc_fwd(L, g, h);
-      else f_conv_fwd(L, g, h, wsm(t) + f_wb_floats(L));
+      else f_conv_fwd(L, IX.l[t], g, h, wsm(t) + f_wb_floats(L));
       __syncthreads();
       const int off = net.off[t];
       for (int j = threadIdx.x; j < net.d[t]; j += FT) {
@@ -1144,7 +1226,7 @@ __global__ void __launch_bounds__(FT) k_attack_chain(NetDev net, const PropDev* 
     for (int t = R; t >= 1; --t) {
       const LayerDev& L = net.aff[t];
       if (L.kind == MNBAB_FC) f_fc_back(L, cur, nxt);
-      else f_conv_back(L, cur, nxt, wsm(t));
+      else f_conv_back(L, IX.l[t], cur, nxt, wsm(t));
       __syncthreads();
       if (t > 1) {
         const int off = net.off[t - 1];
@@ -1166,6 +1248,8 @@ __global__ void __launch_bounds__(FT) k_attack_chain(NetDev net, const PropDev* 
   }
   if (threadIdx.x == 0) best_out[blockIdx.x] = best;
 }
+
+constexpr int kTwoPerSm = 112 * 1024;  // dynamic shared memory of two CTAs per SM
 
 static int fused_maxw(const NetDev& net, int d0) {
   int maxw = d0;
@@ -1198,7 +1282,6 @@ bool fused_supported(const NetDev& net, int SD, int d0, int steps) {
 // tensor-memory columns, the whole shared-memory layout with B and Z within the
 // fused kernel's limit); t = 0 when none fits.
 static FusedTc fused_tc_plan(const NetDev& net, int SD, int d0) {
-  constexpr int kTwoPerSm = 112 * 1024;  // dynamic shared memory of two CTAs per SM
   const int simt = fused_smem_floats(net, SD, d0) * (int)sizeof(float);
   FusedTc best;
   double best_macs = 0.0;
@@ -1215,8 +1298,10 @@ static FusedTc fused_tc_plan(const NetDev& net, int SD, int d0) {
     f.zs = f.P | 1;
     f.dcol = f.Mt * 2 * f.Kp;
     const int cols = f.dcol + f.Mt * f.Np;
-    // a larger Z region must not cost the second CTA per SM
-    const int bytes = fused_smem_floats(net, SD, d0, f) * (int)sizeof(float);
+    // a larger Z region must not cost the second CTA per SM (counted beside the
+    // weights it replaces: the layers that keep their FP32 step stay the same)
+    const int over = std::max(0, f_wb_floats(L) - ftc_wb_region(L, t, f));
+    const int bytes = (fused_smem_floats(net, SD, d0, f) + over) * (int)sizeof(float);
     if (f.Np > 256 || cols > 256 || bytes > 200 * 1024 ||
         (simt <= kTwoPerSm && bytes > kTwoPerSm))
       continue;
@@ -1235,16 +1320,21 @@ int fused_tc_layer(const NetDev& net, int SD, int d0) { return fused_tc_plan(net
 
 void launch_opt_chain(int M, const NetDev& net, const PoolDev& pool, const PropDev* props,
                       const int* row_node, const int* row_j, const FusedHP& hp, float* AP_out,
-                      float* GB_out, bool allow_tc, int* err, cudaStream_t st,
+                      float* GA_out, float* GB_out, bool allow_tc, int* err, cudaStream_t st,
                       const float* skip_lb) {
   if (M <= 0) return;
   const FusedTc ft = allow_tc && err ? fused_tc_plan(net, pool.SD, pool.d0) : FusedTc();
-  const int smem = fused_smem_floats(net, pool.SD, pool.d0, ft) * (int)sizeof(float);
+  int smem = fused_smem_floats(net, pool.SD, pool.d0, ft) * (int)sizeof(float);
+  // the list of neurons with a parameter, where it neither costs the second CTA
+  // per SM nor exceeds the SM
+  const int lsm = (pool.SD + 1) / 2 * 4;
+  const int use_list = smem + lsm <= (smem <= kTwoPerSm ? kTwoPerSm : 220 * 1024) ? 1 : 0;
+  if (use_list) smem += lsm;
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(k_opt_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   const int maxw = fused_maxw(net, pool.d0);
-  k_opt_chain<<<M, FT, smem, st>>>(net, pool, props, row_node, row_j, hp, AP_out, GB_out, maxw, ft,
-                                  err, skip_lb);
+  k_opt_chain<<<M, FT, smem, st>>>(net, pool, props, row_node, row_j, hp, AP_out, GA_out, GB_out, maxw,
+                                   ft, fused_idx(net), use_list, err, skip_lb);
 }
 
 bool sweep_chain_supported(const NetDev& net, int t0) {
@@ -1312,7 +1402,7 @@ void launch_attack_chain(const NetDev& net, const PropDev* props, int prop, int 
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(k_attack_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   k_attack_chain<<<n_rows * n_starts, FT, smem, st>>>(net, props, prop, starts, n_starts, steps,
-                                                      best_out, bx_out, fused_maxw(net, net.d[0]));
+                                                      best_out, bx_out, fused_maxw(net, net.d[0]), fused_idx(net));
 }
 
 }  // namespace mnbab

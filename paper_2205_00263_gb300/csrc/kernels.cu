@@ -282,17 +282,6 @@ __device__ __forceinline__ int win_div(int x, unsigned magic) {
   return magic ? (int)__umulhi((unsigned)x, magic) : x;
 }
 
-// two FP32 FMAs in one instruction, each rounded as fmaf
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;"
-      : "=l"(r)
-      : "l"(*reinterpret_cast<unsigned long long*>(&a)),
-        "l"(*reinterpret_cast<unsigned long long*>(&b)),
-        "l"(*reinterpret_cast<unsigned long long*>(&c)));
-  return *reinterpret_cast<float2*>(&r);
-}
-
 struct WinRow {
   int y0, x0;  // window origin at the current layer
 };

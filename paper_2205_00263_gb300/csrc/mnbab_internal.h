@@ -235,7 +235,8 @@ struct FusedHP {
 };
 bool fused_supported(const NetDev& net, int SD, int d0, int steps);
 // rows m < M: node row_node[m], objective row row_j[m]; a' of the final sweep
-// goes to AP_out [M][SD]; GB_out [M][SD] is row scratch for d lb / d beta;
+// goes to AP_out [M][SD]; GA_out and GB_out [M][SD] are row scratch (upper lines of
+// the relaxation, d lb / d beta);
 // BEST / BESTX of the node track the best iterate.
 // allow_tc: the largest conv layer whose operands fit takes its transposed
 // convolution on the tensor cores (3xTF32); err is the device error flag of
@@ -243,7 +244,7 @@ bool fused_supported(const NetDev& net, int SD, int d0, int steps);
 // value is positive (verified by the DeepPoly pass) are not optimised.
 void launch_opt_chain(int M, const NetDev& net, const PoolDev& pool, const PropDev* props,
                       const int* row_node, const int* row_j, const FusedHP& hp, float* AP_out,
-                      float* GB_out, bool allow_tc, int* err, cudaStream_t st,
+                      float* GA_out, float* GB_out, bool allow_tc, int* err, cudaStream_t st,
                       const float* skip_lb = nullptr);
 // the layer launch_opt_chain(allow_tc = true) runs on the tensor cores (0: none)
 int fused_tc_layer(const NetDev& net, int SD, int d0);

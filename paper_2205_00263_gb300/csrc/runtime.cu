@@ -895,7 +895,7 @@ void run_optimize_body(mnbab_net* n, int M, bool has_gamma, const mnbab_adam& a,
     n->fused_row_flops = 2.0 * ((a.steps + 1.0) * (macs + n->nd.d[n->R]) + a.steps * macs);
     n->fused_row_bytes = (a.steps + 1.0) * n->SD * 66.0;
     Scope sc(c, n->fused_cat, M * n->fused_row_flops, M * n->fused_row_bytes);
-    launch_opt_chain(M, n->nd, n->pool, c->d_props, n->bslots, n->brows, hp, n->AP, n->GB, tc,
+    launch_opt_chain(M, n->nd, n->pool, c->d_props, n->bslots, n->brows, hp, n->AP, n->GA, n->GB, tc,
                      c->d_err, c->st, skip_lb);
     return;
   }
