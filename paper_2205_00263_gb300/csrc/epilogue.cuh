@@ -2,6 +2,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "mnbab_internal.h"
 
 namespace mnbab {
@@ -16,6 +18,21 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
         "l"(*reinterpret_cast<unsigned long long*>(&c)));
   return *reinterpret_cast<float2*>(&r);
 }
+
+// x / d for 0 <= x < 2^31 by the rounded-down reciprocal m = floor((2^32 - 1) / d):
+// the high product is the quotient or one less.  A convolution kernel decodes each
+// of its items with several divisions by layer sizes.
+struct FDiv {
+  unsigned d, m;
+};
+__host__ __device__ inline FDiv f_div_of(int d) {
+  return FDiv{(unsigned)d, 0xffffffffu / (unsigned)d};
+}
+__device__ __forceinline__ int f_div(int x, FDiv v) {
+  const unsigned q = __umulhi((unsigned)x, v.m);
+  return (int)(q + ((unsigned)x - q * v.d >= v.d ? 1u : 0u));
+}
+__device__ __forceinline__ int f_mod(int x, FDiv v) { return x - f_div(x, v) * (int)v.d; }
 
 // ---------------------------------------------------------------------------
 // epilogues
@@ -272,6 +289,35 @@ inline EpiMode epi_mode(const Epi& e) {
     case EPI_FWD_RELU: return EM_FWD;
     default: return EM_STORE;
   }
+}
+
+// calls go(mode as a constant) for an epilogue of the back-substitution / of the
+// forward pass
+template <typename F>
+inline void epi_dispatch_back(const Epi& e, F&& go) {
+  switch (epi_mode(e)) {
+    case EM_RELU: go(std::integral_constant<int, EM_RELU>{}); break;
+    case EM_RELU_FINAL: go(std::integral_constant<int, EM_RELU_FINAL>{}); break;
+    case EM_RELU_GAMMA: go(std::integral_constant<int, EM_RELU_GAMMA>{}); break;
+    case EM_CONC: go(std::integral_constant<int, EM_CONC>{}); break;
+    default: go(std::integral_constant<int, EM_STORE>{}); break;
+  }
+}
+template <typename F>
+inline void epi_dispatch_fwd(const Epi& e, F&& go) {
+  switch (epi_mode(e)) {
+    case EM_ADJ: go(std::integral_constant<int, EM_ADJ>{}); break;
+    case EM_ADJ_GAMMA: go(std::integral_constant<int, EM_ADJ_GAMMA>{}); break;
+    case EM_FWD: go(std::integral_constant<int, EM_FWD>{}); break;
+    default: go(std::integral_constant<int, EM_STORE>{}); break;
+  }
+}
+
+// whether a zero coefficient passes the epilogue as a zero that adds nothing to
+// the row's offset
+template <int EM>
+__device__ __forceinline__ bool epi_zero_passes(const Epi& e) {
+  return !e.acc_in && ((EM == EM_RELU && !e.AP) || (EM == EM_CONC && !e.X) || EM == EM_STORE);
 }
 
 // (an earlier edge's contribution, in.acc, is loaded by epi_finish_block)

@@ -73,21 +73,6 @@ __device__ __forceinline__ int f_split(int items) {
   return ks;
 }
 
-// x / d by the rounded-up reciprocal m = ceil(2^32 / d), exact for x d < 2^32 (the
-// fused kernels' indices stay below 2^16, their layers fit in shared memory); a
-// convolution step decodes its item with ten divisions by layer sizes, which took
-// a third of its instructions.
-struct FDiv {
-  unsigned d, m;
-};
-__host__ __device__ inline FDiv f_div_of(int d) {
-  return FDiv{(unsigned)d, d <= 1 ? 0u : 0xffffffffu / (unsigned)d + 1u};
-}
-__device__ __forceinline__ int f_div(int x, FDiv v) {
-  return v.m ? (int)__umulhi((unsigned)x, v.m) : x;
-}
-__device__ __forceinline__ int f_mod(int x, FDiv v) { return x - f_div(x, v) * (int)v.d; }
-
 struct FusedIdx {
   struct Layer {
     FDiv pp, w2, s;   // transposed step: first positions, those of a row, stride
