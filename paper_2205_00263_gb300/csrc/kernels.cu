@@ -334,6 +334,37 @@ __device__ __forceinline__ void decode_phase(int pidx, int hi, int wi, int s, in
   ih = iw = -1;
 }
 
+// the same with the divisions prepared once per thread
+struct PhaseIdx {
+  int s, wi, hq, hr, wq, wr;  // rows / columns of a phase: hq (+ 1 for the first hr phases)
+  FDiv w0, w1;                // columns of a phase: wq + 1, wq
+  __device__ __forceinline__ PhaseIdx(int hi, int wi_, int s_) : s(s_), wi(wi_) {
+    hq = hi / s;
+    hr = hi - hq * s;
+    wq = wi / s;
+    wr = wi - wq * s;
+    w0 = f_div_of(wq + 1);
+    w1 = f_div_of(max(wq, 1));
+  }
+  __device__ __forceinline__ void decode(int pidx, int& ih, int& iw) const {
+    int ph = 0, nh = hq + (hr > 0);
+    while (pidx >= nh * wi) {
+      pidx -= nh * wi;
+      ++ph;
+      nh = hq + (ph < hr);
+    }
+    int pw = 0, nw = wq + (wr > 0);
+    while (pidx >= nh * nw) {
+      pidx -= nh * nw;
+      ++pw;
+      nw = wq + (pw < wr);
+    }
+    const int r = f_div(pidx, pw < wr ? w0 : w1);
+    ih = ph + s * r;
+    iw = pw + s * (pidx - r * nw);
+  }
+};
+
 // Transposed convolution of the CTA's row windows, A (h x w) to B (h2 x w2),
 // both [channel][position][RB rows].  An item is one output position x CB
 // channels x four rows: a 16-byte load brings a coefficient of the four rows,
@@ -930,52 +961,70 @@ __device__ __forceinline__ void stage_rows(float* __restrict__ dst, const float*
                    (width & 3) == 0 && (valid & 3) == 0;
   if (vec) {
     const int w4 = width >> 2, n4 = nrows * w4;
+    const FDiv dw = f_div_of(w4);
     float4* d4 = reinterpret_cast<float4*>(dst);
-    int i = threadIdx.x;
     const int bd = blockDim.x;
-    for (; i + 3 * bd < n4; i += 4 * bd) {
+    for (int i = threadIdx.x; i < n4; i += 4 * bd) {
       float4 v[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int ii = i + u * bd, r = ii / w4, c = (ii % w4) * 4;
+        const int ii = min(i + u * bd, n4 - 1), r = f_div(ii, dw), c = (ii - r * w4) * 4;
         v[u] = c < valid ? __ldg(reinterpret_cast<const float4*>(src + r * stride + c))
                          : make_float4(0.f, 0.f, 0.f, 0.f);
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) d4[i + u * bd] = v[u];
-    }
-    for (; i < n4; i += bd) {
-      const int r = i / w4, c = (i % w4) * 4;
-      d4[i] = c < valid ? __ldg(reinterpret_cast<const float4*>(src + r * stride + c))
-                        : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int u = 0; u < 4; ++u)
+        if (i + u * bd < n4) d4[i + u * bd] = v[u];
     }
     return;
   }
   const int n = nrows * width;
-  int i = threadIdx.x;
+  const FDiv dw = f_div_of(width);
   const int bd = blockDim.x;
-  for (; i + 3 * bd < n; i += 4 * bd) {
+  for (int i = threadIdx.x; i < n; i += 4 * bd) {
     float v[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int ii = i + u * bd, r = ii / width, c = ii % width;
+      const int ii = min(i + u * bd, n - 1), r = f_div(ii, dw), c = ii - r * width;
       v[u] = c < valid ? __ldg(src + r * stride + c) : 0.f;
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) dst[i + u * bd] = v[u];
-  }
-  for (; i < n; i += bd) {
-    const int r = i / width, c = i % width;
-    dst[i] = c < valid ? __ldg(src + r * stride + c) : 0.f;
+    for (int u = 0; u < 4; ++u)
+      if (i + u * bd < n) dst[i + u * bd] = v[u];
   }
 }
 
+// one row of n floats
+__device__ __forceinline__ void stage_row(float* __restrict__ dst, const float* __restrict__ src,
+                                          int n) {
+  const int bd = blockDim.x;
+  if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
+    const int n4 = n >> 2;
+    const float4* s4 = reinterpret_cast<const float4*>(src);
+    float4* d4 = reinterpret_cast<float4*>(dst);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n4; i += bd) d4[i] = __ldg(s4 + i);
+    for (int i = n4 * 4 + threadIdx.x; i < n; i += bd) dst[i] = __ldg(src + i);
+    return;
+  }
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += bd) dst[i] = __ldg(src + i);
+}
+
 // Row-resident convolution kernels.  A CTA takes one row, one chunk of output
-// positions and one group of channel blocks.  It stages the row's input and
+// positions and one group of channel blocks.  It stages the input rows it reads and
 // its slice of the weights (pre-arranged in global memory so that a channel
 // block is contiguous, float4 loads) in shared memory; each thread computes
 // CB channels of one output position.  Few rows are spread over more CTAs
 // (position chunks x channel groups) so that a launch fills the GPU.
+// What bounds them is latency and instructions, not bandwidth: the epilogue's
+// inputs of an item are loaded together (they were issued one output after another,
+// each behind its branches), indices are decoded by reciprocal, and registers are
+// kept to 5 to 7 CTAs per SM.  Measured before and now: transposed, 594 rows of
+// conv_small_28's second layer 77 and 37 us, its first layer 29 and 21 (dense rows),
+// 65 and 29 (1462 rows that start at a neuron); resnet_32's first layer, 128 rows,
+// 42 and 19.  Forward: 1462 rows of the first layer 50 and 26, 594 of the second 45
+// and 22; resnet_32's layers, 128 rows, 36 and 22 on average.
 struct ConvSplit {
   int ppc;   // positions per chunk
   int npc;   // position chunks
@@ -1005,118 +1054,163 @@ static int convT_row_smem(const LayerDev& L, int cwidth) {
   return L.co * L.ho * L.wo + L.co * L.k * L.k * cwidth;
 }
 
+// acc += v w over CB adjacent channels
 template <int CB>
-__global__ void __launch_bounds__(128) k_convT_row(int M, const float* __restrict__ in, int ld_in,
+__device__ __forceinline__ void row_fma(float v, const float* w, float2 (&acc)[(CB + 1) / 2]) {
+  if constexpr (CB % 4 == 0) {
+    const float2 vv = make_float2(v, v);
+#pragma unroll
+    for (int c = 0; c < CB; c += 4) {
+      const float4 w4 = *reinterpret_cast<const float4*>(w + c);
+      acc[c / 2] = fma2(vv, make_float2(w4.x, w4.y), acc[c / 2]);
+      acc[c / 2 + 1] = fma2(vv, make_float2(w4.z, w4.w), acc[c / 2 + 1]);
+    }
+  } else {
+    acc[0].x = fmaf(v, w[0], acc[0].x);
+  }
+}
+
+// CTAs per SM that the registers allow: as many as leave the epilogue's inputs of
+// CB outputs in registers
+constexpr int convT_row_ctas(int CB, int EM) {
+  return CB == 1 ? 6 : EM > EM_RELU_GAMMA ? 7 : CB == 8 ? 4 : 5;
+}
+
+template <int CB, int EM>
+__global__ void __launch_bounds__(128, convT_row_ctas(CB, EM)) k_convT_row(int M, const float* __restrict__ in, int ld_in,
                                                    float* out, int ld_out, LayerDev L, Epi e,
                                                    ConvSplit cs) {
   extern __shared__ __align__(16) float sm[];
   const int kk = L.k * L.k;
-  const int nIn = L.co * L.ho * L.wo;
   const int chunk = blockIdx.x % cs.npc, grp = blockIdx.x / cs.npc;
   const int nblk = (L.ci + CB - 1) / CB;
   const int b0 = grp * cs.bpg, b1 = min(nblk, b0 + cs.bpg);
   const int c0 = b0 * CB, c1 = min(L.ci, b1 * CB);
   const int cw = cs.bpg * CB;       // stride of the staged channel slice
   float* Ws = sm;                   // [co][kh][kw][cw]
-  float* Ls = sm + L.co * kk * cw;  // input row
+  float* Ls = sm + L.co * kk * cw;  // input rows r_lo .. r_hi of every channel
   const int m = blockIdx.y;
-  // weight slice: rows (co, kh, kw) of Wb [co][kh][kw][ci], channels c0 .. c0 + cw
-  stage_rows(Ws, L.Wb + c0, L.co * kk, cw, (size_t)L.ci, c1 - c0);
-  const float* lam = in + (size_t)m * ld_in;
-  // bounding box (over all channels) of the row's nonzero coefficients: rows
-  // that start at a convolution neuron are nonzero only in its receptive field
-  __shared__ int box[4];
-  if (threadIdx.x == 0) { box[0] = L.ho; box[1] = -1; box[2] = L.wo; box[3] = -1; }
-  __syncthreads();
-  int bh0 = L.ho, bh1 = -1, bw0 = L.wo, bw1 = -1;
-  stage_rows(Ls, lam, 1, nIn, 0, nIn);
-  __syncthreads();
-  // (dense rows: the whole plane)
-  if (!e.sparse_rows) {
-    bh0 = bw0 = 0;
-    bh1 = L.ho - 1;
-    bw1 = L.wo - 1;
-  }
-  for (int i = threadIdx.x; e.sparse_rows && i < nIn; i += blockDim.x) {
-    if (Ls[i] != 0.f) {
-      const int r = i % (L.ho * L.wo), oh = r / L.wo, ow = r % L.wo;
-      bh0 = min(bh0, oh); bh1 = max(bh1, oh); bw0 = min(bw0, ow); bw1 = max(bw1, ow);
-    }
-  }
-  atomicMin(&box[0], bh0); atomicMax(&box[1], bh1); atomicMin(&box[2], bw0); atomicMax(&box[3], bw1);
-  __syncthreads();
-  // output positions that can be nonzero: ih in [oh0*s - p, oh1*s - p + k - 1]
-  const int ih_lo = box[0] * L.s - L.p, ih_hi = box[1] * L.s - L.p + L.k - 1;
-  const int iw_lo = box[2] * L.s - L.p, iw_hi = box[3] * L.s - L.p + L.k - 1;
-  // a zero coefficient maps to 0 with no offset contribution through these
-  // epilogues, so positions outside the window are written as 0 directly
-  const bool zero_passes = !e.acc_in &&
-                           ((e.kind == EPI_RELU && !e.final_mode && !e.GP && !e.GPh && !e.AP) ||
-                            (e.kind == EPI_CONC && !e.X) || e.kind == EPI_STORE);
   const int Pin = L.hi * L.wi;
   const int p0 = chunk * cs.ppc;
   const int np = min(cs.ppc, Pin - p0);
-  const int hwo = L.ho * L.wo;
+  // the input rows that the chunk's positions read (stride 1: its positions are
+  // consecutive rows; the phase-major order of a larger stride reaches all of them)
+  const int r_lo = L.s == 1 ? max(0, p0 / L.wi + L.p - L.k + 1) : 0;
+  const int r_hi = L.s == 1 ? min(L.ho - 1, (p0 + np - 1) / L.wi + L.p) : L.ho - 1;
+  const int plane = max(0, r_hi - r_lo + 1) * L.wo, nIn = L.co * plane;
+  // weight slice: rows (co, kh, kw) of Wb [co][kh][kw][ci], channels c0 .. c0 + cw
+  stage_rows(Ws, L.Wb + c0, L.co * kk, cw, (size_t)L.ci, c1 - c0);
+  const float* lam = in + (size_t)m * ld_in;
+  if (plane == L.ho * L.wo) stage_row(Ls, lam, nIn);
+  else if (plane > 0) stage_rows(Ls, lam + r_lo * L.wo, L.co, plane, (size_t)L.ho * L.wo, plane);
+  // bounding box (over all channels) of the row's nonzero coefficients: rows
+  // that start at a convolution neuron are nonzero only in its receptive field
+  // (and at split neurons), and only taps inside the box are summed
+  __shared__ int box[4];
+  if (threadIdx.x == 0) {
+    const bool s = e.sparse_rows != 0;
+    box[0] = s ? L.ho : r_lo;
+    box[1] = s ? -1 : r_hi;
+    box[2] = s ? L.wo : 0;
+    box[3] = s ? -1 : L.wo - 1;
+  }
+  __syncthreads();
+  if (e.sparse_rows && plane > 0) {
+    const FDiv dhw = f_div_of(plane), dwo = f_div_of(L.wo);
+    int bh0 = L.ho, bh1 = -1, bw0 = L.wo, bw1 = -1;
+    for (int i = threadIdx.x; i < nIn; i += blockDim.x) {
+      if (Ls[i] != 0.f) {
+        const int r = f_mod(i, dhw), orow = f_div(r, dwo), ow = r - orow * L.wo, oh = r_lo + orow;
+        bh0 = min(bh0, oh); bh1 = max(bh1, oh); bw0 = min(bw0, ow); bw1 = max(bw1, ow);
+      }
+    }
+    bh0 = __reduce_min_sync(0xffffffffu, bh0);
+    bh1 = __reduce_max_sync(0xffffffffu, bh1);
+    bw0 = __reduce_min_sync(0xffffffffu, bw0);
+    bw1 = __reduce_max_sync(0xffffffffu, bw1);
+    if ((threadIdx.x & 31) == 0) {
+      atomicMin(&box[0], bh0);
+      atomicMax(&box[1], bh1);
+      atomicMin(&box[2], bw0);
+      atomicMax(&box[3], bw1);
+    }
+    __syncthreads();
+  }
+  const int oh_lo = box[0], oh_hi = box[1], ow_lo = box[2], ow_hi = box[3];
+  // a zero coefficient maps to 0 with no offset contribution through these
+  // epilogues, so positions that no tap reaches are written as 0 directly
+  const bool zero_passes = e.sparse_rows && epi_zero_passes<EM>(e);
+  const FDiv dnp = f_div_of(np), ds = f_div_of(L.s);
+  const PhaseIdx phases(L.hi, L.wi, L.s);
   const int rn = e.row_node[m];
   const PropDev* rp = epi_prop(e, rn);
   float part = 0.f;
-  for (int item = threadIdx.x; item < np * (b1 - b0); item += blockDim.x) {
-    const int cb = b0 + item / np, pidx = p0 + item % np;
-    int ih, iw;
-    decode_phase(pidx, L.hi, L.wi, L.s, ih, iw);
-    if (zero_passes && (ih < ih_lo || ih > ih_hi || iw < iw_lo || iw > iw_hi)) {
-      if (out)
-        for (int c = 0; c < CB && cb * CB + c < L.ci; ++c)
-          out[(size_t)m * ld_out + (cb * CB + c) * Pin + ih * L.wi + iw] = 0.f;
-      continue;
-    }
-    float acc[CB];
+  // U items of a thread together; their epilogue inputs, where they are few, are in
+  // flight during the taps
+  constexpr int U = CB == 1 ? 4 : 1;
+  constexpr bool EARLY = CB == 1 || (CB == 4 && EM == EM_CONC);
+  const int items = np * (b1 - b0), bd = blockDim.x;
+  for (int i0 = threadIdx.x; i0 < items; i0 += U * bd) {
+    float v[U * CB];
+    int j[U * CB];
+    unsigned ok = 0, have = 0;
+    EpiIn pin[U * CB];
+    int ihs[U], iws[U], cbs[U];
 #pragma unroll
-    for (int c = 0; c < CB; ++c) acc[c] = 0.f;
-    const int kh0 = (ih + L.p) % L.s, kw0 = (iw + L.p) % L.s;
-    const int coff = (cb - b0) * CB;
-    for (int kh = kh0; kh < L.k; kh += L.s) {
-      const int th = ih + L.p - kh;
-      if (th < 0) break;
-      const int oh = th / L.s;
-      if (oh >= L.ho) continue;
-      for (int kw = kw0; kw < L.k; kw += L.s) {
-        const int tw = iw + L.p - kw;
-        if (tw < 0) break;
-        const int ow = tw / L.s;
-        if (ow >= L.wo) continue;
-        const float* lp = Ls + oh * L.wo + ow;
-        const float* wp = Ws + (size_t)(kh * L.k + kw) * cw + coff;
-        for (int co = 0; co < L.co; ++co) {
-          const float v = lp[co * hwo];
-          const float* w = wp + (size_t)co * kk * cw;
-          if (CB % 4 == 0) {
+    for (int u = 0; u < U; ++u) {
+      const int it = min(i0 + u * bd, items - 1), b = f_div(it, dnp), cb = b0 + b;
+      int ih, iw;
+      if (CB == 1) phases.decode(p0 + it - b * np, ih, iw);
+      else decode_phase(p0 + it - b * np, L.hi, L.wi, L.s, ih, iw);
+      ihs[u] = ih;
+      iws[u] = iw;
+      cbs[u] = cb;
 #pragma unroll
-            for (int c = 0; c < CB; c += 4) {
-              const float4 w4 = *reinterpret_cast<const float4*>(w + c);
-              acc[c] = fmaf(v, w4.x, acc[c]);
-              acc[c + 1] = fmaf(v, w4.y, acc[c + 1]);
-              acc[c + 2] = fmaf(v, w4.z, acc[c + 2]);
-              acc[c + 3] = fmaf(v, w4.w, acc[c + 3]);
-            }
-          } else {
-#pragma unroll
-            for (int c = 0; c < CB; ++c) acc[c] = fmaf(v, w[c], acc[c]);
-          }
-        }
+      for (int c = 0; c < CB; ++c) {
+        j[u * CB + c] = min(cb * CB + c, L.ci - 1) * Pin + ih * L.wi + iw;
+        if (i0 + u * bd < items && cb * CB + c < L.ci) have |= 1u << (u * CB + c);
+        if (EARLY) epi_load_m<EM>(e, rn, rp, m, j[u * CB + c], pin[u * CB + c]);
       }
     }
-    EpiIn pin[CB];
 #pragma unroll
-    for (int c = 0; c < CB; ++c)
-      if (cb * CB + c < L.ci) epi_load(e, rn, rp, m, (cb * CB + c) * Pin + ih * L.wi + iw, pin[c]);
+    for (int u = 0; u < U; ++u) {
+      if (u > 0 && i0 + u * bd >= items) {
 #pragma unroll
-    for (int c = 0; c < CB; ++c) {
-      const int ci = cb * CB + c;
-      if (ci >= L.ci) break;
-      const int j = ci * Pin + ih * L.wi + iw;
-      const float o = epi_finish(e, m, j, acc[c], pin[c], part);
-      if (out) out[(size_t)m * ld_out + j] = o;
+        for (int c = 0; c < CB; ++c) v[u * CB + c] = 0.f;
+        continue;
+      }
+      // taps kh = kh0 + a s meet input row oh0 - a; columns alike
+      const int oh0 = f_div(ihs[u] + L.p, ds), ow0 = f_div(iws[u] + L.p, ds);
+      const int kh0 = ihs[u] + L.p - oh0 * L.s, kw0 = iws[u] + L.p - ow0 * L.s;
+      const int a0 = max(0, oh0 - oh_hi), a1 = min(f_div(L.k - 1 - kh0 + L.s, ds) - 1, oh0 - oh_lo);
+      const int e0 = max(0, ow0 - ow_hi), e1 = min(f_div(L.k - 1 - kw0 + L.s, ds) - 1, ow0 - ow_lo);
+      const int coff = (cbs[u] - b0) * CB;
+      float2 acc[(CB + 1) / 2];
+#pragma unroll
+      for (int c = 0; c < (CB + 1) / 2; ++c) acc[c] = make_float2(0.f, 0.f);
+      if (!zero_passes || (a0 <= a1 && e0 <= e1)) ok |= ((1u << CB) - 1u) << (u * CB);
+      for (int a = a0; a <= a1; ++a)
+        for (int q = e0; q <= e1; ++q) {
+          const float* lp = Ls + (oh0 - a - r_lo) * L.wo + ow0 - q;
+          const float* wp = Ws + ((kh0 + a * L.s) * L.k + kw0 + q * L.s) * cw + coff;
+#pragma unroll 4
+          for (int co = 0; co < L.co; ++co, lp += plane, wp += kk * cw) row_fma<CB>(*lp, wp, acc);
+        }
+#pragma unroll
+      for (int c = 0; c < CB; ++c) v[u * CB + c] = c & 1 ? acc[c / 2].y : acc[c / 2].x;
+    }
+    ok &= have;
+    if (ok) {
+      if (!EARLY) {
+#pragma unroll
+        for (int c = 0; c < U * CB; ++c) epi_load_m<EM>(e, rn, rp, m, j[c], pin[c]);
+      }
+      epi_finish_block<EM, U * CB>(e, m, j, v, pin, ok, part);
+    }
+    if (out) {
+#pragma unroll
+      for (int c = 0; c < U * CB; ++c)
+        if (have >> c & 1u) out[(size_t)m * ld_out + j[c]] = (ok >> c & 1u) ? v[c] : 0.f;
     }
   }
   if (epi_has_part(e)) {
@@ -1129,80 +1223,177 @@ static int conv_fwd_row_smem(const LayerDev& L, int cwidth) {
   return L.ci * L.hi * L.wi + L.ci * L.k * L.k * cwidth;
 }
 
+// acc += v w where `on` (a tap outside the plane is left out, not multiplied by 0)
 template <int CB>
-__global__ void __launch_bounds__(128) k_conv_fwd_row(int M, const float* __restrict__ in,
+__device__ __forceinline__ void row_fma_if(unsigned on, float v, const float (&w)[CB],
+                                           float2 (&acc)[CB / 2]) {
+  const float2 vv = make_float2(v, v);
+  const unsigned long long x = *reinterpret_cast<const unsigned long long*>(&vv);
+#pragma unroll
+  for (int c = 0; c < CB / 2; ++c) {
+    const float2 ww = make_float2(w[2 * c], w[2 * c + 1]);
+    unsigned long long r = *reinterpret_cast<unsigned long long*>(&acc[c]);
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p fma.rn.f32x2 %0, %1, %2, %0;\n\t}"
+        : "+l"(r)
+        : "l"(x), "l"(*reinterpret_cast<const unsigned long long*>(&ww)), "r"(on));
+    acc[c] = *reinterpret_cast<float2*>(&r);
+  }
+}
+
+// The taps of one output position, in (ci, kh, kw) order, CB channels.  xp: its
+// input at tap (0, 0), channels `plane` apart; [y0, y1), [x0, x1): the tap rows / columns that lie in the
+// plane.  K: the kernel size where it is a constant (the taps are unrolled then).
+template <int CB, int K>
+__device__ __forceinline__ void fwd_taps(const LayerDev& L, const float* xp, int plane,
+                                         const float* wp, int cw, int y0, int y1, int x0, int x1,
+                                         float2 (&acc)[CB / 2]) {
+  const int k = K ? K : L.k;
+  auto weights = [&](const float* w, float (&wv)[CB]) {
+#pragma unroll
+    for (int c = 0; c < CB; c += 4) {
+      const float4 w4 = *reinterpret_cast<const float4*>(w + c);
+      wv[c] = w4.x;
+      wv[c + 1] = w4.y;
+      wv[c + 2] = w4.z;
+      wv[c + 3] = w4.w;
+    }
+  };
+  if (K > 0 && L.p == 0) {  // every tap of every position lies in the plane
+    for (int ci = 0; ci < L.ci; ++ci, xp += plane, wp += k * k * cw) {
+      constexpr int KK = K ? K * K : 1;
+      float v[KK];
+#pragma unroll
+      for (int t = 0; t < KK; ++t) v[t] = xp[t / (K ? K : 1) * L.wi + t % (K ? K : 1)];
+#pragma unroll
+      for (int t = 0; t < KK; ++t) row_fma<CB>(v[t], wp + t * cw, acc);
+    }
+  } else if constexpr (K > 0) {
+    const unsigned vy = (1u << y1) - (1u << y0), vx = (1u << x1) - (1u << x0);
+    unsigned on[K];  // bit kw of on[kh]: the tap lies in the plane
+#pragma unroll
+    for (int kh = 0; kh < K; ++kh) on[kh] = vy >> kh & 1u ? vx : 0u;
+    for (int ci = 0; ci < L.ci; ++ci, xp += plane, wp += K * K * cw) {
+      float v[K * K];
+#pragma unroll
+      for (int t = 0; t < K * K; ++t)
+        v[t] = on[t / K] >> t % K & 1u ? xp[t / K * L.wi + t % K] : 0.f;
+#pragma unroll
+      for (int t = 0; t < K * K; ++t) {
+        float wv[CB];
+        weights(wp + t * cw, wv);
+        row_fma_if<CB>(on[t / K] >> t % K & 1u, v[t], wv, acc);
+      }
+    }
+  } else {
+    for (int ci = 0; ci < L.ci; ++ci, xp += plane, wp += k * k * cw)
+      for (int kh = y0; kh < y1; ++kh)
+#pragma unroll 4
+        for (int kw = x0; kw < x1; ++kw) {
+          float wv[CB];
+          weights(wp + (kh * k + kw) * cw, wv);
+          row_fma_if<CB>(1u, xp[kh * L.wi + kw], wv, acc);
+        }
+  }
+}
+
+// The position chunks and channel groups of a row: about 4 x 152 CTAs over all rows,
+// and of the ways to split a row that many times the one whose CTAs stage the least
+// (a chunk stages only the input rows it reads, a group only its channels' weights).
+constexpr int FWD_CTAS = 4;  // (8: 594 rows 30 us instead of 25 on average)
+static ConvSplit fwd_split(const LayerDev& L, int M, int CB, int* smem_floats) {
+  const int per_row = std::max(1, std::min(32, (FWD_CTAS * 152 + M - 1) / M));
+  const int P = L.ho * L.wo, nblk = (L.co + CB - 1) / CB;
+  ConvSplit best{};
+  long bs = 0;
+  for (int g = 1; g <= nblk; ++g) {
+    ConvSplit cs;
+    cs.bpg = (nblk + g - 1) / g;
+    cs.ngrp = (nblk + cs.bpg - 1) / cs.bpg;
+    cs.npc = std::max((P + 1023) / 1024,
+                      std::max(1, std::min((per_row + cs.ngrp - 1) / cs.ngrp, (P + 31) / 32)));
+    cs.ppc = (P + cs.npc - 1) / cs.npc;
+    cs.npc = (P + cs.ppc - 1) / cs.ppc;
+    const int orows = std::min(L.ho, (cs.ppc + L.wo - 2) / L.wo + 1);  // output rows of a chunk
+    const int irows = std::min(L.hi, (orows - 1) * L.s + L.k);
+    const long fl = (long)L.ci * (irows * L.wi + (long)L.k * L.k * cs.bpg * CB);
+    if (g == 1 || fl < bs) {
+      best = cs;
+      bs = fl;
+    }
+    if (g >= per_row && bs <= 40 * 1024) break;
+  }
+  *smem_floats = (int)std::min<long>(bs, 1 << 28);
+  return best;
+}
+
+// CB = 4: with eight channels per thread the epilogue's inputs took 118 registers,
+// and four CTAs per SM left the loads' latency uncovered (1462 rows: 52 us, now 26;
+// two or four positions per thread, which share the weights' loads, 60 and more).
+template <int CB, int EM>
+__global__ void __launch_bounds__(128, 6) k_conv_fwd_row(int M, const float* __restrict__ in,
                                                       int ld_in, float* out, int ld_out,
                                                       LayerDev L, Epi e, ConvSplit cs) {
   extern __shared__ __align__(16) float sm[];
   const int kk = L.k * L.k;
-  const int nIn = L.ci * L.hi * L.wi;
   const int chunk = blockIdx.x % cs.npc, grp = blockIdx.x / cs.npc;
   const int nblk = (L.co + CB - 1) / CB;
   const int b0 = grp * cs.bpg, b1 = min(nblk, b0 + cs.bpg);
   const int c0 = b0 * CB, c1 = min(L.co, b1 * CB);
   const int cw = cs.bpg * CB;
   float* Ws = sm;                   // [ci][kh][kw][cw]
-  float* Xs = sm + L.ci * kk * cw;  // input row
+  float* Xs = sm + L.ci * kk * cw;  // input rows r_lo .. r_hi of every channel
   const int m = blockIdx.y;
-  // weight slice: rows (ci, kh, kw) of Wf [ci][kh][kw][co], channels c0 .. c0 + cw
-  stage_rows(Ws, L.Wf + c0, L.ci * kk, cw, (size_t)L.co, c1 - c0);
-  stage_rows(Xs, in + (size_t)m * ld_in, 1, nIn, 0, nIn);
-  __syncthreads();
   const int P = L.ho * L.wo;
   const int p0 = chunk * cs.ppc;
   const int np = min(cs.ppc, P - p0);
-  const int hwi = L.hi * L.wi;
-  const int rn = (e.kind == EPI_RELU || e.kind == EPI_ADJ) ? e.row_node[m] : 0;
-  float part = 0.f;
+  const int r_lo = max(0, p0 / L.wo * L.s - L.p);
+  const int r_hi = min(L.hi - 1, (p0 + np - 1) / L.wo * L.s - L.p + L.k - 1);
+  const int plane = max(0, r_hi - r_lo + 1) * L.wi;
+  // weight slice: rows (ci, kh, kw) of Wf [ci][kh][kw][co], channels c0 .. c0 + cw
+  stage_rows(Ws, L.Wf + c0, L.ci * kk, cw, (size_t)L.co, c1 - c0);
+  if (plane > 0)
+    stage_rows(Xs, in + (size_t)m * ld_in + r_lo * L.wi, L.ci, plane, (size_t)L.hi * L.wi, plane);
+  __syncthreads();
+  const FDiv dnp = f_div_of(np), dwo = f_div_of(L.wo);
+  const int rn = (EM == EM_ADJ || EM == EM_ADJ_GAMMA) ? e.row_node[m] : 0;
+  float part = 0.f;  // forward epilogues (adjoint, ReLU) produce no offset partials
   for (int item = threadIdx.x; item < np * (b1 - b0); item += blockDim.x) {
-    const int cb = b0 + item / np, pos = p0 + item % np;
-    const int oh = pos / L.wo, ow = pos % L.wo;
-    const int coff = (cb - b0) * CB;
-    float acc[CB];
-#pragma unroll
-    for (int c = 0; c < CB; ++c) acc[c] = 0.f;
-    for (int ci = 0; ci < L.ci; ++ci) {
-      for (int kh = 0; kh < L.k; ++kh) {
-        const int ih = oh * L.s - L.p + kh;
-        if (ih < 0 || ih >= L.hi) continue;
-        for (int kw = 0; kw < L.k; ++kw) {
-          const int iw = ow * L.s - L.p + kw;
-          if (iw < 0 || iw >= L.wi) continue;
-          const float v = Xs[ci * hwi + ih * L.wi + iw];
-          const float* w = Ws + (size_t)((ci * L.k + kh) * L.k + kw) * cw + coff;
-          if (CB % 4 == 0) {
-#pragma unroll
-            for (int c = 0; c < CB; c += 4) {
-              const float4 w4 = *reinterpret_cast<const float4*>(w + c);
-              acc[c] = fmaf(v, w4.x, acc[c]);
-              acc[c + 1] = fmaf(v, w4.y, acc[c + 1]);
-              acc[c + 2] = fmaf(v, w4.z, acc[c + 2]);
-              acc[c + 3] = fmaf(v, w4.w, acc[c + 3]);
-            }
-          } else {
-#pragma unroll
-            for (int c = 0; c < CB; ++c) acc[c] = fmaf(v, w[c], acc[c]);
-          }
-        }
-      }
-    }
+    const int b = f_div(item, dnp), cb = b0 + b, pos = p0 + item - b * np;
+    const int oh = f_div(pos, dwo), ow = pos - oh * L.wo;
+    const int ih0 = oh * L.s - L.p, iw0 = ow * L.s - L.p;
+    // the item's epilogue inputs are in flight during its taps
+    float v[CB];
+    int j[CB];
+    unsigned ok = 0;
     EpiIn pin[CB];
 #pragma unroll
-    for (int c = 0; c < CB; ++c)
-      if (cb * CB + c < L.co) epi_load(e, rn, nullptr, m, (cb * CB + c) * P + pos, pin[c]);
-#pragma unroll
     for (int c = 0; c < CB; ++c) {
-      const int co = cb * CB + c;
-      if (co >= L.co) break;
-      const int j = co * P + pos;
-      const float o = epi_finish(e, m, j, acc[c] + L.b[co], pin[c], part);
-      if (out) out[(size_t)m * ld_out + j] = o;
+      const int co = min(cb * CB + c, L.co - 1);
+      if (cb * CB + c < L.co) ok |= 1u << c;
+      j[c] = co * P + pos;
+      epi_load_m<EM>(e, rn, nullptr, m, j[c], pin[c]);
+    }
+    const int y0 = max(0, -ih0), y1 = max(y0, min(L.k, L.hi - ih0));
+    const int x0 = max(0, -iw0), x1 = max(x0, min(L.k, L.wi - iw0));
+    const float* xp = Xs + (ih0 - r_lo) * L.wi + iw0;
+    const float* wp = Ws + b * CB;
+    float2 acc[CB / 2];
+#pragma unroll
+    for (int c = 0; c < CB / 2; ++c) acc[c] = make_float2(0.f, 0.f);
+    if (L.k == 3) fwd_taps<CB, 3>(L, xp, plane, wp, cw, min(y0, 3), y1, min(x0, 3), x1, acc);
+    else if (L.k == 4) fwd_taps<CB, 4>(L, xp, plane, wp, cw, min(y0, 4), y1, min(x0, 4), x1, acc);
+    else fwd_taps<CB, 0>(L, xp, plane, wp, cw, y0, y1, x0, x1, acc);
+#pragma unroll
+    for (int c = 0; c < CB; ++c)
+      v[c] = (c & 1 ? acc[c / 2].y : acc[c / 2].x) + L.b[min(cb * CB + c, L.co - 1)];
+    epi_finish_block<EM, CB>(e, m, j, v, pin, ok, part);
+    if (out) {
+#pragma unroll
+      for (int c = 0; c < CB; ++c)
+        if (ok >> c & 1u) out[(size_t)m * ld_out + j[c]] = v[c];
     }
   }
-  (void)part;  // forward epilogues (adjoint, ReLU) produce no offset partials
 }
-
-
 
 // ---------------------------------------------------------------------------
 // implicit-GEMM convolutions for dense rows
@@ -1569,35 +1760,35 @@ static int conv_variant(int v, int dir, const LayerDev& L, int M, const float* i
     const int CBv = L.ci <= 1 ? 1 : (L.ci <= 4 ? 4 : 8);
     const ConvSplit cs = conv_split(M, L.hi * L.wi, (L.ci + CBv - 1) / CBv, CBv,
                                     [&](int cw) { return convT_row_smem(L, cw); }, 40 * 1024);
-    const int rsm = convT_row_smem(L, cs.bpg * CBv) * 4;
+    // (stride 1: a chunk's input rows only)
+    const int irows = std::min(L.ho, L.s == 1 ? (cs.ppc + L.wi - 2) / L.wi + L.k : L.ho);
+    const int rsm = (convT_row_smem(L, cs.bpg * CBv) - L.co * (L.ho - irows) * L.wo) * 4;
     if (rsm > 160 * 1024 || !L.Wb || cs.npc * cs.ngrp > backsub_slots(L)) return -1;
     dim3 grid(cs.npc * cs.ngrp, M);
-    if (CBv == 1) {
-      set_smem(k_convT_row<1>, rsm);
-      k_convT_row<1><<<grid, 128, rsm, st>>>(M, in, ld_in, out, ld_out, L, e, cs);
-    } else if (CBv == 4) {
-      set_smem(k_convT_row<4>, rsm);
-      k_convT_row<4><<<grid, 128, rsm, st>>>(M, in, ld_in, out, ld_out, L, e, cs);
-    } else {
-      set_smem(k_convT_row<8>, rsm);
-      k_convT_row<8><<<grid, 128, rsm, st>>>(M, in, ld_in, out, ld_out, L, e, cs);
-    }
+    epi_dispatch_back(e, [&](auto em) {
+      auto go = [&](auto kern) {
+        set_smem(kern, rsm);
+        kern<<<grid, 128, rsm, st>>>(M, in, ld_in, out, ld_out, L, e, cs);
+      };
+      constexpr int EM = decltype(em)::value;
+      if (CBv == 1) go(k_convT_row<1, EM>);
+      else if (CBv == 4) go(k_convT_row<4, EM>);
+      else go(k_convT_row<8, EM>);
+    });
     return grid.x;
   }
   if (v == V_ROW && dir == 0) {
-    const int CBv = (L.co % 8 == 0 && L.ho * L.wo >= 64) ? 8 : 4;
-    const ConvSplit cs = conv_split(M, L.ho * L.wo, (L.co + CBv - 1) / CBv, CBv,
-                                    [&](int cw) { return conv_fwd_row_smem(L, cw); }, 40 * 1024);
-    const int rsm = conv_fwd_row_smem(L, cs.bpg * CBv) * 4;
+    constexpr int CB = 4;
+    int fl;
+    const ConvSplit cs = fwd_split(L, M, CB, &fl);
+    const int rsm = fl * 4;
     if (rsm > 160 * 1024 || !L.Wf) return -1;
     dim3 grid(cs.npc * cs.ngrp, M);
-    if (CBv == 8) {
-      set_smem(k_conv_fwd_row<8>, rsm);
-      k_conv_fwd_row<8><<<grid, 128, rsm, st>>>(M, in, ld_in, out, ld_out, L, e, cs);
-    } else {
-      set_smem(k_conv_fwd_row<4>, rsm);
-      k_conv_fwd_row<4><<<grid, 128, rsm, st>>>(M, in, ld_in, out, ld_out, L, e, cs);
-    }
+    epi_dispatch_fwd(e, [&](auto em) {
+      auto kern = k_conv_fwd_row<CB, decltype(em)::value>;
+      set_smem(kern, rsm);
+      kern<<<grid, 128, rsm, st>>>(M, in, ld_in, out, ld_out, L, e, cs);
+    });
     return 0;
   }
   if (v == V_PLAIN) {

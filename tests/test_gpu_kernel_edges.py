@@ -199,3 +199,46 @@ def test_tensor_core_convolutions(Context, layers, shape):
                 assert np.abs(g - o).max() <= TOL * (1 + np.abs(o).max())
             assert all((lb[j::3] == lb[j]).all() or np.abs(lb[j::3] - lb[j]).max() <= 1e-6 * (1 + abs(lb[j]))
                        for j in range(min(3, len(batch))))
+
+
+# row-resident convolutions in both directions and starting rows (gemm_path 1, layers
+# too small for the implicit GEMM): kernels of 3 and 4 with and without padding, and
+# others; strides 1 to 3; channel counts that are no multiple of a block; one input
+# channel (several items per thread) with a last round that is not full; planes split
+# into chunks whose first and last input rows are cut off; one row and several
+@pytest.mark.parametrize("layers,shape", [
+    ([("conv", 5, 3, 1, 1), ("relu",), ("conv", 6, 2, 2, 0), ("relu",), ("fc", 7), ("relu",), ("fc", 3)], (3, 9, 7)),
+    ([("conv", 8, 4, 2, 1), ("relu",), ("conv", 9, 5, 3, 2), ("relu",), ("fc", 3)], (1, 29, 31)),
+    ([("conv", 6, 4, 2, 0), ("relu",), ("conv", 12, 3, 1, 0), ("relu",), ("fc", 3)], (1, 28, 20)),
+    ([("conv", 8, 3, 1, 1), ("relu",), ("conv", 16, 1, 2, 0), ("relu",), ("conv", 11, 3, 1, 2), ("relu",),
+      ("fc", 3)], (3, 21, 20)),
+    ([("conv", 4, 7, 1, 3), ("relu",), ("conv", 3, 3, 2, 1), ("relu",), ("fc", 3)], (2, 6, 40)),
+])
+def test_row_convolutions(Context, layers, shape):
+    layers, C, d, lo, hi, prep = _case(dict(seed=61, in_shape=shape, layers=layers), 0.01)
+    net, lo_t, hi_t, l, u, S, _, _ = prep
+    SD = sum(l[i].numel() for i in l)
+    rng = np.random.default_rng(6)
+    nodes = [random_node(prep, rng, n_splits=2 * j, row=j % 2) for j in range(3)]
+    refs = []
+    for on in nodes:
+        on.split_layer = net.R
+        refs.append(core.bound_and_grad(net, on, on.alpha, on.beta, on.gamma, None, lo_t, hi_t))
+    with Context(node_capacity=1024, gemm_path=1) as ctx:
+        gnet = ctx.load_network(layers)
+        prop = ctx.set_property(gnet, lo, hi, C, d)
+        for i in l:
+            gl, gu = ctx.root_bounds(prop, i)
+            assert close(gl, l[i].numpy()).all() and close(gu, u[i].numpy()).all(), i
+        gids = []
+        for on in nodes:
+            gids.append(ctx.node_root(prop, on.row))
+            ctx.import_params(gids[-1], to_params(on, net.R))
+        for batch in ([0], [1, 2], [j % 3 for j in range(160)]):
+            lb, ga, gb, _ = ctx.bound_grad([gids[j] for j in batch], SD, 0)
+            for i in list(range(min(3, len(batch)))) + [len(batch) - 1]:
+                ref, _, oa, ob, _ = refs[batch[i]]
+                assert close(lb[i], float(ref)).all(), (batch[i], lb[i], float(ref))
+                o = np.concatenate([concat(oa, net.R), concat(ob, net.R)])
+                g = np.concatenate([ga[i], gb[i]])
+                assert np.abs(g - o).max() <= TOL * (1 + np.abs(o).max())
