@@ -1680,10 +1680,197 @@ static bool ig_preferred(const LayerDev& L) {
   return (double)L.co * L.ho * L.wo * L.ci * L.k * L.k >= 512.0 * 1024.0;
 }
 
+// Transposed convolution of stride 1 to at most three channels (a network's input):
+// a warp computes 128 consecutive positions of one row, a thread four of them and
+// all N channels, in the implicit GEMM's order of taps (o, kh, kw) and of offset
+// sums (a channel's four positions, the 32 lanes, then the channels), so that both
+// give the same bits.  G warps share the source rows they read, which are staged
+// OC channels at a time by asynchronous copies while the previous ones are summed.
+// The implicit GEMM gives such a layer one channel per thread and gathers each tap's
+// coefficients into shared memory: nine copies of the row for three FMAs each.  Here
+// six loaded coefficients serve 36 FMAs.  Measured, 32 channels of 32 x 32 through a
+// 3x3 kernel to three: 64 rows 102 us with the implicit GEMM, 14.5 here; 256 rows 214
+// and 24, 1024 rows 657 and 74 (reading the coefficients once would take 20).  What
+// is left is instructions: 108 of a channel's 130 or so per thread are the FMAs.
+constexpr int NARROW_OC = 8;   // source channels per stage
+constexpr int NARROW_ST = 2;   // stages
+
+struct NarrowCfg {
+  int G;       // warps (128 positions each) per CTA
+  int nchunk;  // 128-position chunks of a row
+  int rows;    // staged source rows of a CTA (at most)
+  int sw;      // their stride
+  int smem;
+};
+
+template <int K, int N, int EM>
+__global__ void __launch_bounds__(128) k_convT_narrow(const float* __restrict__ in, int ld_in,
+                                                      float* out, int ld_out, LayerDev L, Epi e,
+                                                      NarrowCfg g) {
+  extern __shared__ __align__(16) float nsm[];
+  const int stage = NARROW_OC * g.rows * g.sw;
+  float* Wn = nsm + NARROW_ST * stage;  // [o][kh][kw][4]
+  const int m = blockIdx.y, nthr = blockDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int P = L.hi * L.wi, hwo = L.ho * L.wo;
+  const int p_lo = blockIdx.x * g.G * 128, p_hi = min(P, p_lo + g.G * 128) - 1;
+  const FDiv dw = f_div_of(L.wi);
+  const int y_lo = f_div(p_lo, dw), y_hi = f_div(p_hi, dw);
+  // staged source rows: yb .. ye of the plane, yb + i at row i; columns shifted by
+  // K - 1 - p; what lies outside the plane stays zero
+  const int yb = y_lo + L.p - K + 1, v_lo = max(0, yb), v_hi = min(L.ho - 1, y_hi + L.p);
+  const int nrow = max(0, v_hi - v_lo + 1);
+  for (int i = threadIdx.x; i < NARROW_ST * stage / 4; i += nthr)
+    reinterpret_cast<float4*>(nsm)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int i = threadIdx.x; i < L.co * K * K * 4; i += nthr)
+    Wn[i] = (i & 3) < N ? __ldg(L.Wb + (i >> 2) * N + (i & 3)) : 0.f;
+  __syncthreads();
+  const float* src = in + (size_t)m * ld_in + v_lo * L.wo;
+  const int nel = nrow * L.wo;  // staged elements of a channel: consecutive in memory
+  const FDiv dwo = f_div_of(L.wo);
+  auto load = [&](int c) {  // channels c OC .. of the row into stage c mod ST
+    const int o0 = c * NARROW_OC, no = min(NARROW_OC, L.co - o0);
+    const unsigned base = static_cast<unsigned>(__cvta_generic_to_shared(
+        nsm + c % NARROW_ST * stage + (v_lo - yb) * g.sw + K - 1 - L.p));
+    const float* s0 = src + (size_t)o0 * hwo;
+    const unsigned dstep = (unsigned)(g.rows * g.sw) * 4u;
+    for (int q = threadIdx.x; q < nel; q += nthr) {
+      const int r = f_div(q, dwo);
+      unsigned d = base + (unsigned)(r * g.sw + q - r * L.wo) * 4u;
+      const float* s = s0 + q;
+#pragma unroll 4
+      for (int o = 0; o < no; ++o, d += dstep, s += hwo)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(s) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int nc = (L.co + NARROW_OC - 1) / NARROW_OC;
+  const int chunk = blockIdx.x * g.G + warp, pos = chunk * 128 + lane * 4;
+  const bool act = pos < P;  // (P is a multiple of four)
+  const int y = act ? f_div(pos, dw) : y_lo, x = act ? pos - y * L.wi : 0;
+  float acc[N][4];
+#pragma unroll
+  for (int n = 0; n < N; ++n)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[n][i] = 0.f;
+  load(0);
+  for (int c = 0; c < nc; ++c) {
+    if (c + 1 < nc) {
+      load(c + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    const float* sp = nsm + c % NARROW_ST * stage + (y - y_lo + K - 1) * g.sw + x;
+    const float* wp = Wn + c * NARROW_OC * K * K * 4;
+    const int no = min(NARROW_OC, L.co - c * NARROW_OC);
+#pragma unroll 1
+    for (int o = 0; o < no; ++o, sp += g.rows * g.sw, wp += K * K * 4) {
+#pragma unroll
+      for (int a = 0; a < K; ++a) {
+        // coefficient x + i + p - b lies at column x + i + K - 1 - b
+        constexpr int NV = (K + 3 + 1) / 2 * 2;
+        float v[NV];
+#pragma unroll
+        for (int u = 0; u < NV; u += 4) {
+          if (u + 4 <= NV) {
+            const float4 q = *reinterpret_cast<const float4*>(sp - a * g.sw + u);
+            v[u] = q.x;
+            v[u + 1] = q.y;
+            v[u + 2] = q.z;
+            v[u + 3] = q.w;
+          } else {
+            const float2 q = *reinterpret_cast<const float2*>(sp - a * g.sw + u);
+            v[u] = q.x;
+            v[u + 1] = q.y;
+          }
+        }
+#pragma unroll
+        for (int b = 0; b < K; ++b) {
+          const float4 w4 = *reinterpret_cast<const float4*>(wp + (a * K + b) * 4);
+          const float w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+          for (int n = 0; n < N; ++n)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[n][i] = fmaf(v[i + K - 1 - b], w[n], acc[n][i]);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  float tot = 0.f;
+  const int rn = e.row_node[m];
+  const PropDev* rp = epi_prop(e, rn);
+#pragma unroll
+  for (int n = 0; n < N; ++n) {
+    float part = 0.f;
+    if (act) {
+      int j[4];
+      EpiIn pin[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        j[i] = n * P + pos + i;
+        epi_load_m<EM>(e, rn, rp, m, j[i], pin[i]);
+      }
+      epi_finish_block<EM, 4>(e, m, j, acc[n], pin, 15u, part);
+      if (out) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) out[(size_t)m * ld_out + j[i]] = acc[n][i];
+      }
+    }
+    for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    tot += part;
+  }
+  if (epi_has_part(e) && lane == 0 && chunk < g.nchunk)
+    e.part[(size_t)m * e.nslot + e.slot_base + chunk] = tot;
+}
+
+// Whether k_convT_narrow takes what the implicit GEMM's plan g would do: whole
+// 128-position chunks (from 38 rows of 1024 positions on; with fewer rows the plan's
+// shorter chunks spread a row over more SMs).
+static bool narrow_plan(const LayerDev& L, int dir, int M, const IgCfg& g, NarrowCfg* c) {
+  if (dir != 1 || L.s != 1 || (L.k != 3 && L.k != 5) || L.ci > 3 || (L.wi & 3) || L.p > L.k - 1 ||
+      g.pc != 128 || g.ngrp != 1)
+    return false;
+  c->nchunk = g.nchunk;
+  // CTAs of four warps while they fill the SMs, else of two (one: 15.8 us for 64 rows)
+  c->G = 4;
+  while (c->G > 2 && (long)M * ((c->nchunk + c->G - 1) / c->G) < 2 * 152) c->G >>= 1;
+  c->rows = (c->G * 128 + L.wi - 2) / L.wi + L.k;
+  c->sw = (L.wi + L.k - 1 + 3) / 4 * 4;
+  c->smem = (NARROW_ST * NARROW_OC * c->rows * c->sw + L.co * L.k * L.k * 4) * 4;
+  return c->smem <= 96 * 1024;
+}
+
+static void launch_narrow(const LayerDev& L, int M, const float* in, int ld_in, float* out,
+                          int ld_out, const Epi& e, const NarrowCfg& c, cudaStream_t st) {
+  dim3 grid((c.nchunk + c.G - 1) / c.G, M);
+  epi_dispatch_back(e, [&](auto em) {
+    constexpr int EM = decltype(em)::value;
+    auto go = [&](auto kern) {
+      set_smem(kern, c.smem);
+      kern<<<grid, 32 * c.G, c.smem, st>>>(in, ld_in, out, ld_out, L, e, c);
+    };
+    auto by_n = [&](auto k) {
+      constexpr int K = decltype(k)::value;
+      if (L.ci == 1) go(k_convT_narrow<K, 1, EM>);
+      else if (L.ci == 2) go(k_convT_narrow<K, 2, EM>);
+      else go(k_convT_narrow<K, 3, EM>);
+    };
+    if (L.k == 3) by_n(std::integral_constant<int, 3>{});
+    else by_n(std::integral_constant<int, 5>{});
+  });
+}
+
 // launches the implicit-GEMM kernel; returns the partial-sum slots (transposed)
 static int launch_ig(const LayerDev& L, int dir, int M, const float* in, int ld_in, float* out,
                      int ld_out, const Epi& e, cudaStream_t st) {
   const IgCfg g = ig_plan(L, dir, M);
+  NarrowCfg nc;
+  if (narrow_plan(L, dir, M, g, &nc)) {
+    launch_narrow(L, M, in, ld_in, out, ld_out, e, nc, st);
+    return g.nchunk;
+  }
   const int smem = ig_smem(g);
   dim3 grid(g.ncls * g.nchunk * g.ngrp, (M + g.RB - 1) / g.RB);
   const int thr = g.RB * g.tpr;

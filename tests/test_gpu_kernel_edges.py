@@ -242,3 +242,42 @@ def test_row_convolutions(Context, layers, shape):
                 o = np.concatenate([concat(oa, net.R), concat(ob, net.R)])
                 g = np.concatenate([ga[i], gb[i]])
                 assert np.abs(g - o).max() <= TOL * (1 + np.abs(o).max())
+
+
+# stride-1 convolutions back to at most three input channels (128-position chunks per
+# warp, many rows): 3x3 and 5x5 kernels, padding from none to the kernel's reach,
+# planes that are no multiple of a chunk or of a CTA's chunks, chunks that start inside
+# a row, source channels that are no multiple of a stage; a plane width that is no
+# multiple of four takes the other kernel
+@pytest.mark.parametrize("layers,shape", [
+    ([("conv", 21, 3, 1, 1), ("relu",), ("conv", 4, 2, 2, 0), ("relu",), ("fc", 3)], (3, 30, 36)),
+    ([("conv", 16, 5, 1, 2), ("relu",), ("conv", 4, 3, 3, 0), ("relu",), ("fc", 3)], (2, 27, 28)),
+    ([("conv", 30, 5, 1, 4), ("relu",), ("conv", 4, 4, 4, 0), ("relu",), ("fc", 3)], (1, 28, 28)),
+    ([("conv", 23, 3, 1, 0), ("relu",), ("conv", 4, 2, 2, 0), ("relu",), ("fc", 3)], (3, 32, 32)),
+    ([("conv", 20, 3, 1, 1), ("relu",), ("conv", 4, 2, 2, 0), ("relu",), ("fc", 3)], (3, 31, 34)),
+])
+def test_convolution_to_few_channels(Context, layers, shape):
+    layers, C, d, lo, hi, prep = _case(dict(seed=71, in_shape=shape, layers=layers), 0.01)
+    net, lo_t, hi_t, l, u, S, _, _ = prep
+    SD = sum(l[i].numel() for i in l)
+    rng = np.random.default_rng(8)
+    nodes = [random_node(prep, rng, n_splits=3 * j, row=j % 2) for j in range(2)]
+    refs = []
+    for on in nodes:
+        on.split_layer = net.R
+        refs.append(core.bound_and_grad(net, on, on.alpha, on.beta, on.gamma, None, lo_t, hi_t))
+    with Context(node_capacity=1024, gemm_path=1) as ctx:
+        gnet = ctx.load_network(layers)
+        prop = ctx.set_property(gnet, lo, hi, C, d)
+        gids = []
+        for on in nodes:
+            gids.append(ctx.node_root(prop, on.row))
+            ctx.import_params(gids[-1], to_params(on, net.R))
+        for batch in ([0, 1], [j % 2 for j in range(90)], [j % 2 for j in range(400)]):
+            lb, ga, gb, _ = ctx.bound_grad([gids[j] for j in batch], SD, 0)
+            for i in (0, 1, len(batch) - 1):
+                ref, _, oa, ob, _ = refs[batch[i]]
+                assert close(lb[i], float(ref)).all(), (batch[i], lb[i], float(ref))
+                o = np.concatenate([concat(oa, net.R), concat(ob, net.R)])
+                g = np.concatenate([ga[i], gb[i]])
+                assert np.abs(g - o).max() <= TOL * (1 + np.abs(o).max())
