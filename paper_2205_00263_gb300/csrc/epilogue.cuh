@@ -313,6 +313,13 @@ inline void epi_dispatch_fwd(const Epi& e, F&& go) {
   }
 }
 
+// calls go(mode as a constant) for any epilogue
+template <typename F>
+inline void epi_dispatch(const Epi& e, F&& go) {
+  if (e.kind == EPI_ADJ || e.kind == EPI_FWD_RELU) epi_dispatch_fwd(e, go);
+  else epi_dispatch_back(e, go);
+}
+
 // whether a zero coefficient passes the epilogue as a zero that adds nothing to
 // the row's offset
 template <int EM>

@@ -640,129 +640,203 @@ void launch_win_rows(const NetDev& net, const WinPlan& wp, const RowsDev& rows, 
 }
 
 // ---------------------------------------------------------------------------
-// dense GEMM C = A B (+ bias) with a fused epilogue; SIMT FP32, 64x64x16 tiles
+// dense GEMM C = A B (+ bias) with a fused epilogue; SIMT FP32
 // ---------------------------------------------------------------------------
 constexpr int GBK = 16;
+constexpr int GLA = GBK + 4;  // stride of a staged row of A (float4 reads without bank conflicts)
 
-// BM x BN tile, 256 threads as 16 x 16, each thread (BM/16) x (BN/16) outputs.
-template <int BM, int BN>
-__global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const float* __restrict__ A,
-                                              int lda, const float* __restrict__ B, int ldb,
-                                              const float* __restrict__ bias, int bias_div,
-                                              float* C, int ldc, Epi e) {
-  constexpr int TM = BM / 16, TN = BN / 16;
-  __shared__ float As[GBK][BM + 4];
-  __shared__ float Bs[GBK][BN + 4];
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  float acc[TM][TN];
+// A BM x BN tile over the reduction range [kb, ke): TM x TN outputs per thread
+// (rows ty + TY i, columns TN tx + j), each summed over k in order.  Steps of GBK go
+// through a ring of ST stages filled by asynchronous copies: the small products of
+// a few rows are bound by the latency of their loads (about 2 us for each step of
+// 16 when a step waited for its own loads), so ST - 1 steps are in flight, and a
+// thread takes 8 or 16 outputs (with four, shared-memory reads fed one FMA each).
+// Measured before and now: 64 x 512 x 4096 split in ten 56 and 18 us, 64 x 4096 x 512
+// split in two 36 and 14; 32 x 32 tiles, 256 x 4096 x 512 126 and 46, 9 x 100 x 100
+// 16.7 and 7.5; 64 x 64 tiles, 1024 x 4096 x 512 273 and 123.
+template <int BM, int BN, int TM, int TN, int ST>
+__device__ __forceinline__ void gemm_tile(int M, int N, int kb, int ke, const float* __restrict__ A,
+                                          int lda, const float* __restrict__ B, int ldb, int m0,
+                                          int n0, float* sm, float (&acc)[TM][TN]) {
+  constexpr int TX = BN / TN, TY = BM / TM, NT = TX * TY;
+  constexpr int STAGE = BM * GLA + GBK * BN;
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+  const bool va = ((reinterpret_cast<uintptr_t>(A) | (uintptr_t)lda * 4) & 15) == 0;
+  const bool vb = ((reinterpret_cast<uintptr_t>(B) | (uintptr_t)ldb * 4) & 15) == 0;
+  const unsigned s0 = static_cast<unsigned>(__cvta_generic_to_shared(sm));
+  // `n` of four floats (the others zero); one by one where 16-byte copies are not aligned
+  auto copy4 = [](unsigned d, const float* s, const float* base, int n, bool vec) {
+    if (vec) {
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(n > 0 ? s : base),
+                   "r"(n * 4)
+                   : "memory");
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d + 4u * u),
+                     "l"(u < n ? s + u : base), "r"(u < n ? 4 : 0)
+                     : "memory");
+    }
+  };
+  auto load = [&](int it) {
+    const int k0 = kb + it * GBK;
+    const unsigned sa = s0 + (unsigned)(it % ST * STAGE) * 4u, sb = sa + (unsigned)(BM * GLA) * 4u;
+#pragma unroll
+    for (int c = tid; c < BM * GBK / 4; c += NT) {
+      const int r = c / (GBK / 4), k = c % (GBK / 4) * 4, gm = m0 + r;
+      const int n = gm < M ? max(0, min(4, ke - (k0 + k))) : 0;
+      copy4(sa + (unsigned)(r * GLA + k) * 4u, A + (size_t)gm * lda + k0 + k, A, n, va);
+    }
+#pragma unroll
+    for (int c = tid; c < GBK * BN / 4; c += NT) {
+      const int r = c / (BN / 4), q = c % (BN / 4) * 4, gk = k0 + r;
+      const int n = gk < ke ? max(0, min(4, N - (n0 + q))) : 0;
+      copy4(sb + (unsigned)(r * BN + q) * 4u, B + (size_t)gk * ldb + n0 + q, B, n, vb);
+    }
+  };
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
     for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
-  for (int k0 = 0; k0 < K; k0 += GBK) {
-    for (int q = tid; q < BM * GBK; q += 256) {
-      const int r = q >> 4, cc = q & 15;
-      const int gm = m0 + r, gk = k0 + cc;
-      As[cc][r] = (gm < M && gk < K) ? A[(size_t)gm * lda + gk] : 0.f;
+  const int nk = (ke - kb + GBK - 1) / GBK;
+#pragma unroll
+  for (int it = 0; it < ST - 1; ++it) {
+    if (it < nk) load(it);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  for (int it = 0; it < nk; ++it) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(ST - 2) : "memory");
+    __syncthreads();
+    if (it + ST - 1 < nk) load(it + ST - 1);  // into the stage of step it - 1
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const float* as = sm + it % ST * STAGE + ty * GLA;
+    const float* bs = sm + it % ST * STAGE + BM * GLA + tx * TN;
+#pragma unroll
+    for (int k = 0; k < GBK; k += 4) {
+      float a[TM][4], b[4][TN];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(as + i * TY * GLA + k);
+        a[i][0] = v.x;
+        a[i][1] = v.y;
+        a[i][2] = v.z;
+        a[i][3] = v.w;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if constexpr (TN == 4) {
+          const float4 v = *reinterpret_cast<const float4*>(bs + (k + u) * BN);
+          b[u][0] = v.x;
+          b[u][1] = v.y;
+          b[u][2] = v.z;
+          b[u][3] = v.w;
+        } else {
+          const float2 v = *reinterpret_cast<const float2*>(bs + (k + u) * BN);
+          b[u][0] = v.x;
+          b[u][1] = v.y;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i][u], b[u][j], acc[i][j]);
     }
-    for (int q = tid; q < BN * GBK; q += 256) {
-      const int r = q / BN, cc = q % BN;
-      const int gk = k0 + r, gn = n0 + cc;
-      Bs[r][cc] = (gk < K && gn < N) ? B[(size_t)gk * ldb + gn] : 0.f;
-    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+constexpr int gemm_smem(int BM, int BN, int ST) { return ST * (BM * GLA + GBK * BN) * 4; }
+
+// BM x BN tile, BM BN / (TM TN) threads.  The outputs pass through shared memory to
+// the epilogue's threads: 16 per row, columns tx + 16 j, so that a row's offset
+// partial is summed in that order whatever tile computed it.
+template <int BM, int BN, int TM, int TN, int ST, int EM>
+__global__ void __launch_bounds__(BM * BN / (TM * TN)) k_gemm(
+    int M, int N, int K, const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
+    const float* __restrict__ bias, int bias_div, float* C, int ldc, Epi e) {
+  extern __shared__ __align__(16) float gsm[];
+  constexpr int NT = BM * BN / (TM * TN), TX = BN / TN, TY = BM / TM, LC = BN + 1;
+  constexpr int RPT = BM * 16 / NT, NJ = BN / 16;  // epilogue: rows and columns per thread
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN, tid = threadIdx.x;
+  {
+    float acc[TM][TN];
+    gemm_tile<BM, BN, TM, TN, ST>(M, N, 0, K, A, lda, B, ldb, m0, n0, gsm, acc);
     __syncthreads();
 #pragma unroll
-    for (int kk = 0; kk < GBK; ++kk) {
-      float a[TM], b[TN];
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
+      for (int j = 0; j < TN; ++j)
+        gsm[(tid / TX + TY * i) * LC + tid % TX * TN + j] = acc[i][j];
     __syncthreads();
   }
-  float part[TM];
+  const int tx = tid & 15, ty = tid >> 4;
+  int cn[NJ];
+  float cb[NJ];
+  unsigned okn = 0;
 #pragma unroll
-  for (int i = 0; i < TM; ++i) part[i] = 0.f;
-#pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    const int m = m0 + ty + 16 * i;
-    if (m >= M) continue;
-#pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      const int n = n0 + tx + 16 * j;
-      if (n >= N) continue;
-      float v = acc[i][j];
-      if (bias) v += bias[n / bias_div];
-      const float o = epi_apply(e, m, n, v, part[i]);
-      if (C) C[(size_t)m * ldc + n] = o;
-    }
+  for (int j = 0; j < NJ; ++j) {
+    const int n = n0 + tx + 16 * j;
+    cn[j] = min(n, N - 1);
+    if (n < N) okn |= 1u << j;
+    cb[j] = bias ? bias[cn[j] / bias_div] : 0.f;
   }
-  if (epi_has_part(e)) {
+#pragma unroll 2
+  for (int i = 0; i < RPT; ++i) {
+    const int r = ty + NT / 16 * i, m = m0 + r;
+    float part = 0.f;
+    if (m < M) {
+      const int rn = EM == EM_STORE || EM == EM_FWD ? 0 : e.row_node[m];
+      const PropDev* rp = epi_prop(e, rn);
+      float v[NJ];
+      EpiIn in[NJ];
 #pragma unroll
-    for (int i = 0; i < TM; ++i) {
-      float p = part[i];
-      for (int o = 8; o; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o, 16);
-      const int m = m0 + ty + 16 * i;
-      if (tx == 0 && m < M) e.part[(size_t)m * e.nslot + e.slot_base + blockIdx.x] = p;
+      for (int j = 0; j < NJ; ++j) {
+        epi_load_m<EM>(e, rn, rp, m, cn[j], in[j]);
+        v[j] = gsm[r * LC + tx + 16 * j];
+        if (bias) v[j] += cb[j];
+      }
+      epi_finish_block<EM, NJ>(e, m, cn, v, in, okn, part);
+      if (C) {
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+          if (okn >> j & 1u) C[(size_t)m * ldc + cn[j]] = v[j];
+      }
+    }
+    if (epi_has_part(e)) {
+      for (int o = 8; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o, 16);
+      if (tx == 0 && m < M) e.part[(size_t)m * e.nslot + e.slot_base + blockIdx.x] = part;
     }
   }
 }
 
 // Split-K partial products: CTA z computes K range [z*kc, (z+1)*kc) of a
 // 32 x 32 tile into ws[z][m][n] (no epilogue).
-__global__ void __launch_bounds__(256) k_gemm_splitk(int M, int N, int K, int kc,
+__global__ void __launch_bounds__(128) k_gemm_splitk(int M, int N, int K, int kc,
                                                      const float* __restrict__ A, int lda,
                                                      const float* __restrict__ B, int ldb,
                                                      float* __restrict__ ws) {
-  __shared__ float As[GBK][32 + 4];
-  __shared__ float Bs[GBK][32 + 4];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * 32, n0 = blockIdx.x * 32;
+  extern __shared__ __align__(16) float gsm[];
+  const int m0 = blockIdx.y * 32, n0 = blockIdx.x * 32, tid = threadIdx.x;
   const int kb = blockIdx.z * kc, ke = min(K, kb + kc);
-  float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-  for (int k0 = kb; k0 < ke; k0 += GBK) {
-    for (int q = tid; q < 32 * GBK; q += 256) {
-      const int r = q >> 4, cc = q & 15;
-      const int gm = m0 + r, gk = k0 + cc;
-      As[cc][r] = (gm < M && gk < ke) ? A[(size_t)gm * lda + gk] : 0.f;
-    }
-    for (int q = tid; q < 32 * GBK; q += 256) {
-      const int r = q >> 5, cc = q & 31;
-      const int gk = k0 + r, gn = n0 + cc;
-      Bs[r][cc] = (gk < ke && gn < N) ? B[(size_t)gk * ldb + gn] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < GBK; ++kk) {
-      const float a0 = As[kk][ty], a1 = As[kk][ty + 16];
-      const float b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
-      acc[0][0] = fmaf(a0, b0, acc[0][0]);
-      acc[0][1] = fmaf(a0, b1, acc[0][1]);
-      acc[1][0] = fmaf(a1, b0, acc[1][0]);
-      acc[1][1] = fmaf(a1, b1, acc[1][1]);
-    }
-    __syncthreads();
-  }
+  float acc[4][2];
+  gemm_tile<32, 32, 4, 2, 6>(M, N, kb, ke, A, lda, B, ldb, m0, n0, gsm, acc);
   float* w = ws + (size_t)blockIdx.z * M * N;
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const int m = m0 + ty + 16 * i, n = n0 + tx + 16 * j;
+      const int m = m0 + tid / 16 + 8 * i, n = n0 + tid % 16 * 2 + j;
       if (m < M && n < N) w[(size_t)m * N + n] = acc[i][j];
     }
 }
 
 // Sum of the split-K partials (fixed order) + bias, then the epilogue; a CTA
 // covers 8 rows x 32 columns, one warp per row, and writes one offset partial
-// per (row, 32-column tile).
+// per (row, 32-column tile).  An output's partials (at most 16) and its epilogue's
+// inputs are loaded together.
+template <int EM>
 __global__ void __launch_bounds__(256) k_splitk_epi(int M, int N, int S, const float* __restrict__ ws,
                                                     const float* __restrict__ bias, int bias_div,
                                                     float* C, int ldc, Epi e) {
@@ -770,11 +844,21 @@ __global__ void __launch_bounds__(256) k_splitk_epi(int M, int N, int S, const f
   const int n = blockIdx.x * 32 + (threadIdx.x & 31);
   float part = 0.f;
   if (m < M && n < N) {
-    float v = 0.f;
-    for (int z = 0; z < S; ++z) v += ws[((size_t)z * M + m) * N + n];
-    if (bias) v += bias[n / bias_div];
-    const float o = epi_apply(e, m, n, v, part);
-    if (C) C[(size_t)m * ldc + n] = o;
+    const int rn = EM == EM_STORE || EM == EM_FWD ? 0 : e.row_node[m];
+    float w[16];
+#pragma unroll
+    for (int z = 0; z < 16; ++z) w[z] = z < S ? ws[((size_t)z * M + m) * N + n] : 0.f;
+    const float b = bias ? bias[n / bias_div] : 0.f;
+    EpiIn in[1];
+    const int j[1] = {n};
+    epi_load_m<EM>(e, rn, epi_prop(e, rn), m, n, in[0]);
+    float v[1] = {0.f};
+#pragma unroll
+    for (int z = 0; z < 16; ++z)
+      if (z < S) v[0] += w[z];
+    if (bias) v[0] += b;
+    epi_finish_block<EM, 1>(e, m, j, v, in, 1u, part);
+    if (C) C[(size_t)m * ldc + n] = v[0];
   }
   if (epi_has_part(e)) {
     for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
@@ -801,19 +885,30 @@ static int gemm_variant(int v, int M, int N, int K, const float* A, int lda, con
     const int kc = ((K + S - 1) / S + GBK - 1) / GBK * GBK;
     S = (K + kc - 1) / kc;
     dim3 g1((N + 31) / 32, (M + 31) / 32, S);
-    k_gemm_splitk<<<g1, 256, 0, st>>>(M, N, K, kc, A, lda, B, ldb, e.ws);
+    constexpr int sm = gemm_smem(32, 32, 6);
+    k_gemm_splitk<<<g1, 128, sm, st>>>(M, N, K, kc, A, lda, B, ldb, e.ws);
     dim3 g2((N + 31) / 32, (M + 7) / 8);
-    k_splitk_epi<<<g2, 256, 0, st>>>(M, N, S, e.ws, bias, bias_div, C, ldc, e);
+    epi_dispatch(e, [&](auto em) {
+      k_splitk_epi<decltype(em)::value><<<g2, 256, 0, st>>>(M, N, S, e.ws, bias, bias_div, C, ldc, e);
+    });
     return g2.x;
   }
   if (v == V_G64) {
     dim3 grid((N + 63) / 64, (M + 63) / 64);
-    k_gemm<64, 64><<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, bias, bias_div, C, ldc, e);
+    constexpr int sm = gemm_smem(64, 64, 4);
+    epi_dispatch(e, [&](auto em) {
+      k_gemm<64, 64, 4, 4, 4, decltype(em)::value>
+          <<<grid, 256, sm, st>>>(M, N, K, A, lda, B, ldb, bias, bias_div, C, ldc, e);
+    });
     return grid.x;
   }
   if (v == V_G32) {
     dim3 grid((N + 31) / 32, (M + 31) / 32);
-    k_gemm<32, 32><<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, bias, bias_div, C, ldc, e);
+    constexpr int sm = gemm_smem(32, 32, 6);
+    epi_dispatch(e, [&](auto em) {
+      k_gemm<32, 32, 4, 2, 6, decltype(em)::value>
+          <<<grid, 128, sm, st>>>(M, N, K, A, lda, B, ldb, bias, bias_div, C, ldc, e);
+    });
     return grid.x;
   }
   return -1;

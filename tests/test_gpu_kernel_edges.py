@@ -281,3 +281,42 @@ def test_convolution_to_few_channels(Context, layers, shape):
                 o = np.concatenate([concat(oa, net.R), concat(ob, net.R)])
                 g = np.concatenate([ga[i], gb[i]])
                 assert np.abs(g - o).max() <= TOL * (1 + np.abs(o).max())
+
+
+# dense products of a few rows (gemm_path 1): widths that are no multiple of four (no
+# 16-byte copies), of a tile or of a step of the reduction, reductions shorter than a
+# step and than the ring of steps, split reductions with a short last part; one row,
+# rows that end inside a tile, and enough for 64 x 64 tiles
+@pytest.mark.parametrize("dims", [(13, 9, 5, 3), (50, 129, 70, 4), (64, 304, 68, 3), (31, 515, 257, 6),
+                                  (520, 1040, 33, 3)])
+def test_dense_products(Context, dims):
+    layers = []
+    for n in dims[1:]:
+        layers += [("fc", n), ("relu",)]
+    layers, C, d, lo, hi, prep = _case(dict(seed=81, in_shape=(1, 1, dims[0]), layers=layers[:-1]), 0.02)
+    net, lo_t, hi_t, l, u, S, _, _ = prep
+    SD = sum(l[i].numel() for i in l)
+    rng = np.random.default_rng(9)
+    nodes = [random_node(prep, rng, n_splits=2 * j, row=j % 2) for j in range(2)]
+    refs = []
+    for on in nodes:
+        on.split_layer = net.R
+        refs.append(core.bound_and_grad(net, on, on.alpha, on.beta, on.gamma, None, lo_t, hi_t))
+    with Context(node_capacity=4096, gemm_path=1) as ctx:
+        gnet = ctx.load_network(layers)
+        prop = ctx.set_property(gnet, lo, hi, C, d)
+        for i in l:
+            gl, gu = ctx.root_bounds(prop, i)
+            assert close(gl, l[i].numpy()).all() and close(gu, u[i].numpy()).all(), i
+        gids = []
+        for on in nodes:
+            gids.append(ctx.node_root(prop, on.row))
+            ctx.import_params(gids[-1], to_params(on, net.R))
+        for batch in ([1], [j % 2 for j in range(45)], [j % 2 for j in range(1300)]):
+            lb, ga, gb, _ = ctx.bound_grad([gids[j] for j in batch], SD, 0)
+            for i in {0, min(1, len(batch) - 1), len(batch) - 1}:
+                ref, _, oa, ob, _ = refs[batch[i]]
+                assert close(lb[i], float(ref)).all(), (batch[i], lb[i], float(ref))
+                o = np.concatenate([concat(oa, net.R), concat(ob, net.R)])
+                g = np.concatenate([ga[i], gb[i]])
+                assert np.abs(g - o).max() <= TOL * (1 + np.abs(o).max())
