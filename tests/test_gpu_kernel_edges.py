@@ -288,7 +288,7 @@ def test_convolution_to_few_channels(Context, layers, shape):
 # step and than the ring of steps, split reductions with a short last part; one row,
 # rows that end inside a tile, and enough for 64 x 64 tiles
 @pytest.mark.parametrize("dims", [(13, 9, 5, 3), (50, 129, 70, 4), (64, 304, 68, 3), (31, 515, 257, 6),
-                                  (520, 1040, 33, 3)])
+                                  (520, 1300, 33, 3)])
 def test_dense_products(Context, dims):
     layers = []
     for n in dims[1:]:
@@ -312,7 +312,7 @@ def test_dense_products(Context, dims):
         for on in nodes:
             gids.append(ctx.node_root(prop, on.row))
             ctx.import_params(gids[-1], to_params(on, net.R))
-        for batch in ([1], [j % 2 for j in range(45)], [j % 2 for j in range(1300)]):
+        for batch in ([1], [j % 2 for j in range(45)], [j % 2 for j in range(1000)]):
             lb, ga, gb, _ = ctx.bound_grad([gids[j] for j in batch], SD, 0)
             for i in {0, min(1, len(batch) - 1), len(batch) - 1}:
                 ref, _, oa, ob, _ = refs[batch[i]]
