@@ -2343,75 +2343,50 @@ __device__ __forceinline__ int layer_of(const NetDev& net, int f) {
 }
 
 // gamma^T P and gamma^T Phat per neuron (CSR by neuron), and gamma^T p per row.
-// The CTAs of a row: GP_SPLIT that sum a share of gamma^T p each (k_reduce_lb adds
-// the shares), `nzero` that write the zeros of neurons without entries, and the
-// others, which take eight of the layers' listed neurons (those with entries) at
-// a time: each warp brings one neuron's entries to shared memory, all loads in
-// flight (a neuron in three groups of 150 rows has 450), then two lanes per neuron
-// of one warp sum them, gamma^T P and gamma^T Phat, in entry order.  Bound by the
-// latency of those loads and the chain of FMAs.  64 rows of the 3x32x32 network with
-// 135k constraint rows, and 9 of the 784-100-100-10 one: 335 and 79 us with one
-// thread per neuron that loads its own entries, 409 and 12 with one warp per neuron
-// for the sums too (two lanes of 32 busy), 234 and 60 with 64-entry chunks.
+// A CTA serves RB consecutive rows.  The CTAs of such a group: RB x GP_SPLIT that sum
+// a share of one row's gamma^T p each (k_reduce_lb adds the shares), RB x `nzero`
+// that write the zeros of neurons without entries, and the others, which take eight
+// of the layers' listed neurons (those with entries) at a time: each warp brings
+// one neuron's entries to shared memory, all loads in flight (a neuron in three
+// groups of 150 rows has 450), then two lanes per neuron and row sum them, gamma^T P
+// and gamma^T Phat, in entry order.  Rows of one property share the entries: an
+// entry's index and two coefficients are loaded once for the RB rows (of a group
+// of different properties, a CTA takes one row).  Bound by the latency of those
+// loads and the chain of FMAs.  64 rows of the 3x32x32 network with 135k constraint
+// rows: 113 us with one row per CTA, 70 with four; 9 rows of the 784-100-100-10 one
+// 7.4 with one (their CTAs would not fill the SMs in groups).  20 steps of 64 such
+// rows, with the gradients' kernel below: 13.4 and 11.8 ms; 14.0 where two properties
+// alternate row by row, the order that groups gain nothing from.
 constexpr int GP_THREADS = 256;
-constexpr int GP_CHUNK = 480;  // entries of a chunk (15 per lane)
+constexpr int GP_GROUP = 4;        // rows of a group
+constexpr int GP_GROUP_MIN = 32;   // rows from which on they are grouped
 
-__global__ void __launch_bounds__(GP_THREADS) k_gamma_proj(
-    int M, const int* __restrict__ row_node, PoolDev pool, const PropDev* __restrict__ props,
-    NetDev net, int nzero, float* __restrict__ GP, float* __restrict__ GPh,
-    float* __restrict__ gp0) {
-  const int m = blockIdx.y;
-  const int n = row_node[m];
-  const PropDev& P = props[pool.prop[n]];
-  const float* gam = pool.GAM + (size_t)n * pool.EC;
-  if (blockIdx.x < GP_SPLIT) {
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    constexpr int step = GP_THREADS * GP_SPLIT;
-    for (int i = 1; i <= net.R; ++i) {
-      const MncDev& mc = P.mnc[i];
-      const float* g = gam + mc.goff;
-      const float* pv = mc.p;
-      const int e1 = mc.e;
-      for (int e = blockIdx.x * GP_THREADS + threadIdx.x; e < e1; e += 4 * step) {
-        float gv[4], p[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const bool in = e + u * step < e1;
-          gv[u] = in ? g[e + u * step] : 0.f;
-          p[u] = in ? pv[e + u * step] : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc[u] = fmaf(gv[u], p[u], acc[u]);
-      }
-    }
-    const float tot = block_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
-    if (threadIdx.x == 0) gp0[(size_t)m * GP_SPLIT + blockIdx.x] = tot;
-    return;
-  }
-  if (blockIdx.x < GP_SPLIT + nzero) {
-    for (int f = (blockIdx.x - GP_SPLIT) * GP_THREADS + threadIdx.x; f < net.SD;
-         f += nzero * GP_THREADS) {
-      const int i = layer_of(net, f), j = f - net.off[i];
-      const int* cptr = P.mnc[i].e > 0 ? P.mnc[i].cptr : nullptr;
-      if (!cptr || cptr[j + 1] == cptr[j]) {
-        GP[(size_t)m * net.SD + f] = 0.f;
-        GPh[(size_t)m * net.SD + f] = 0.f;
-      }
-    }
-    return;
-  }
-  constexpr int NW = GP_THREADS / 32, LD = GP_CHUNK + 4;
-  __shared__ __align__(16) float s_ent[NW][3][LD];  // gamma, P, Phat
-  __shared__ int s_len[NW], s_f[NW];
+// The sums of `rows` rows (at most R; all of one property) from row m on: CTA b of nb
+// takes listed neurons NW b .., NW nb further on.  s_ent: a warp's staged entries (P,
+// Phat, the rows' gamma; CHUNK + 4 floats each).
+template <int R, int CHUNK>
+__device__ __forceinline__ void gamma_proj_rows(int m, int rows, int b, int nb,
+                                                const int* __restrict__ row_node,
+                                                const PoolDev& pool,
+                                                const PropDev* __restrict__ props,
+                                                const NetDev& net, float* s_ent, int* s_len,
+                                                int* s_f, float* __restrict__ GP,
+                                                float* __restrict__ GPh) {
+  constexpr int NW = GP_THREADS / 32, LD = CHUNK + 4, WS = (2 + R) * LD;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nb = gridDim.x - GP_SPLIT - nzero, b = blockIdx.x - GP_SPLIT - nzero;
+  const PropDev& P = props[pool.prop[row_node[m]]];
+  const float* gam[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    gam[r] = pool.GAM + (size_t)row_node[m + (r < rows ? r : 0)] * pool.EC;
+  float* own = s_ent + warp * WS;
   int total = 0;
   for (int i = 1; i <= net.R; ++i) total += P.mnc[i].n_act;
   for (int a0 = b * NW; a0 < total; a0 += nb * NW) {
     // this warp's neuron and its entries
-    int q0 = 0, len = 0;
+    int q0 = 0, len = 0, goff = 0;
     const int *ce_ = nullptr;
-    const float *cP_ = nullptr, *cPh_ = nullptr, *g = nullptr;
+    const float *cP_ = nullptr, *cPh_ = nullptr;
     if (a0 + warp < total) {
       int i = 1, a = a0 + warp;
       while (a >= P.mnc[i].n_act) a -= P.mnc[i++].n_act;
@@ -2422,38 +2397,43 @@ __global__ void __launch_bounds__(GP_THREADS) k_gamma_proj(
       ce_ = mc.ce + q0;
       cP_ = mc.cP + q0;
       cPh_ = mc.cPh + q0;
-      g = gam + mc.goff;
+      goff = mc.goff;
       if (lane == 0) s_f[warp] = net.off[i] + j;
     }
     if (lane == 0) s_len[warp] = len;
     __syncthreads();
     int most = 0;
     for (int w = 0; w < NW; ++w) most = max(most, s_len[w]);
-    const int mine = (threadIdx.x >> 1) % NW, which = threadIdx.x & 1;
+    // lanes of the sums: row, P or Phat, neuron
+    const int row = threadIdx.x % R, which = threadIdx.x / R & 1;
+    const int mine = threadIdx.x / (2 * R) % NW;
     float acc = 0.f;
-    for (int c0 = 0; c0 < most; c0 += GP_CHUNK) {
-      int ce[GP_CHUNK / 32];
-      float cp[GP_CHUNK / 32], cph[GP_CHUNK / 32];
+    for (int c0 = 0; c0 < most; c0 += CHUNK) {
+      int ce[CHUNK / 32];
+      float cp[CHUNK / 32], cph[CHUNK / 32];
 #pragma unroll
-      for (int v = 0; v < GP_CHUNK / 32; ++v) {
+      for (int v = 0; v < CHUNK / 32; ++v) {
         const int k = c0 + 32 * v + lane;
         ce[v] = k < len ? ce_[k] : -1;
         cp[v] = k < len ? cP_[k] : 0.f;
         cph[v] = k < len ? cPh_[k] : 0.f;
       }
 #pragma unroll
-      for (int v = 0; v < GP_CHUNK / 32; ++v) {
-        s_ent[warp][0][32 * v + lane] = ce[v] >= 0 ? g[ce[v]] : 0.f;
-        s_ent[warp][1][32 * v + lane] = cp[v];
-        s_ent[warp][2][32 * v + lane] = cph[v];
+      for (int v = 0; v < CHUNK / 32; ++v) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          own[(2 + r) * LD + 32 * v + lane] =
+              ce[v] >= 0 && (R == 1 || r < rows) ? gam[r][goff + ce[v]] : 0.f;
+        own[32 * v + lane] = cp[v];
+        own[LD + 32 * v + lane] = cph[v];
       }
       __syncthreads();
-      if (threadIdx.x < 2 * NW) {
-        const float* eg = s_ent[mine][0];
-        const float* ec = s_ent[mine][1 + which];
-        const int cnt = min(GP_CHUNK, s_len[mine] - c0);
+      if (threadIdx.x < 2 * R * NW) {
+        const float* eg = s_ent + mine * WS + (2 + row) * LD;
+        const float* ec = s_ent + mine * WS + which * LD;
+        const int num = min(CHUNK, s_len[mine] - c0);
         int k = 0;
-        for (; k + 8 <= cnt; k += 8) {
+        for (; k + 8 <= num; k += 8) {
           const float4 x0 = *reinterpret_cast<const float4*>(eg + k);
           const float4 x1 = *reinterpret_cast<const float4*>(eg + k + 4);
           const float4 y0 = *reinterpret_cast<const float4*>(ec + k);
@@ -2467,94 +2447,209 @@ __global__ void __launch_bounds__(GP_THREADS) k_gamma_proj(
           acc = fmaf(x1.z, y1.z, acc);
           acc = fmaf(x1.w, y1.w, acc);
         }
-        for (; k < cnt; ++k) acc = fmaf(eg[k], ec[k], acc);
+        for (; k < num; ++k) acc = fmaf(eg[k], ec[k], acc);
       }
       __syncthreads();
     }
-    if (threadIdx.x < 2 * NW && a0 + mine < total)
-      (which ? GPh : GP)[(size_t)m * net.SD + s_f[mine]] = acc;
+    if (threadIdx.x < 2 * R * NW && a0 + mine < total && row < rows)
+      (which ? GPh : GP)[(size_t)(m + row) * net.SD + s_f[mine]] = acc;
     __syncthreads();
   }
 }
 
-// CTAs per row for the listed neurons: one pass over up to 1024 of them
+template <int RB>
+__global__ void __launch_bounds__(GP_THREADS, 4) k_gamma_proj(
+    int M, const int* __restrict__ row_node, PoolDev pool, const PropDev* __restrict__ props,
+    NetDev net, int nzero, float* __restrict__ GP, float* __restrict__ GPh,
+    float* __restrict__ gp0) {
+  const int mg = blockIdx.y * RB;
+  if (blockIdx.x < GP_SPLIT * RB) {
+    const int m = mg + blockIdx.x / GP_SPLIT, share = blockIdx.x % GP_SPLIT;
+    if (m >= M) return;
+    const int n = row_node[m];
+    const PropDev& P = props[pool.prop[n]];
+    const float* gam = pool.GAM + (size_t)n * pool.EC;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    constexpr int step = GP_THREADS * GP_SPLIT;
+    for (int i = 1; i <= net.R; ++i) {
+      const MncDev& mc = P.mnc[i];
+      const float* g = gam + mc.goff;
+      const float* pv = mc.p;
+      const int e1 = mc.e;
+      for (int e = share * GP_THREADS + threadIdx.x; e < e1; e += 4 * step) {
+        float gv[4], p[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const bool in = e + u * step < e1;
+          gv[u] = in ? g[e + u * step] : 0.f;
+          p[u] = in ? pv[e + u * step] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] = fmaf(gv[u], p[u], acc[u]);
+      }
+    }
+    const float tot = block_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
+    if (threadIdx.x == 0) gp0[(size_t)m * GP_SPLIT + share] = tot;
+    return;
+  }
+  if (blockIdx.x < (GP_SPLIT + nzero) * RB) {
+    const int z = blockIdx.x - GP_SPLIT * RB, m = mg + z / nzero;
+    if (m >= M) return;
+    const PropDev& P = props[pool.prop[row_node[m]]];
+    for (int f = z % nzero * GP_THREADS + threadIdx.x; f < net.SD; f += nzero * GP_THREADS) {
+      const int i = layer_of(net, f), j = f - net.off[i];
+      const int* cptr = P.mnc[i].e > 0 ? P.mnc[i].cptr : nullptr;
+      if (!cptr || cptr[j + 1] == cptr[j]) {
+        GP[(size_t)m * net.SD + f] = 0.f;
+        GPh[(size_t)m * net.SD + f] = 0.f;
+      }
+    }
+    return;
+  }
+  // (RB = 4: rows of different properties get longer chunks in the same space)
+  constexpr int NW = GP_THREADS / 32, C1 = RB == 1 ? 480 : 448, CG = 224;
+  constexpr int W1 = 3 * (C1 + 4), WG = RB == 1 ? 0 : (2 + RB) * (CG + 4);
+  __shared__ __align__(16) float s_ent[NW * (W1 > WG ? W1 : WG)];
+  __shared__ int s_len[NW], s_f[NW];
+  const int nother = (GP_SPLIT + nzero) * RB;
+  const int nb = gridDim.x - nother, b = blockIdx.x - nother;
+  const int nr = min(RB, M - mg);
+  if (RB > 1) {
+    bool same = true;
+    const int prop0 = pool.prop[row_node[mg]];
+    for (int r = 1; r < nr; ++r) same = same && pool.prop[row_node[mg + r]] == prop0;
+    if (same) {
+      gamma_proj_rows<RB, CG>(mg, nr, b, nb, row_node, pool, props, net, s_ent, s_len, s_f, GP, GPh);
+      return;
+    }
+  }
+  const int r = b % nr;  // (nb >= RB)
+  gamma_proj_rows<1, C1>(mg + r, 1, b / nr, (nb - r + nr - 1) / nr, row_node, pool, props, net,
+                         s_ent, s_len, s_f, GP, GPh);
+}
+
 void launch_gamma_proj(int M, const int* row_node, PoolDev pool, const PropDev* props,
                        const NetDev& net, float* GP, float* GPh, float* gp0, cudaStream_t st) {
   if (M <= 0) return;
   const int per = GP_THREADS / 32;
   const int nact = std::min(128, (net.SD + per - 1) / per);
   const int nzero = (net.SD + 4 * GP_THREADS - 1) / (4 * GP_THREADS);
-  dim3 grid(GP_SPLIT + nzero + nact, M);
-  k_gamma_proj<<<grid, GP_THREADS, 0, st>>>(M, row_node, pool, props, net, nzero, GP, GPh, gp0);
+  auto go = [&](auto kern, int rb) {
+    dim3 grid((GP_SPLIT + nzero) * rb + std::max(nact, rb), (M + rb - 1) / rb);
+    kern<<<grid, GP_THREADS, 0, st>>>(M, row_node, pool, props, net, nzero, GP, GPh, gp0);
+  };
+  if (M >= GP_GROUP_MIN) go(k_gamma_proj<GP_GROUP>, GP_GROUP);
+  else go(k_gamma_proj<1>, 1);
 }
 
 // d lb / d gamma_e = sum_k P_ek (d lb / d a')_idx + Phat_ek (d lb / d ahat)_idx - p_e.
+// A CTA serves RB consecutive rows; rows of one property share a constraint row's
+// neurons and coefficients (28 bytes of 52 per row, at three neurons), which were
+// two thirds of the time at one row per CTA.  64 rows, 135k constraint rows: 63 us,
+// 32 in groups of four.
 constexpr int GAMMA_NPT = 4;
-// A CTA serves one row (node and property looked up once); each thread takes
-// GAMMA_NPT constraint rows, loading every row's entries before the gathers.
-__global__ void k_gamma_grad(int M, const int* __restrict__ row_node, PoolDev pool,
-                             const PropDev* __restrict__ props, NetDev net,
-                             const float* __restrict__ Gz, const float* __restrict__ Hz,
-                             float* __restrict__ GG) {
-  const int m = blockIdx.y;
-  __shared__ const PropDev* s_P;
-  __shared__ int s_goff[MNBAB_MAXR + 1], s_e[MNBAB_MAXR + 1];
-  if (threadIdx.x == 0) s_P = props + pool.prop[row_node[m]];
+template <int RB>
+__global__ void __launch_bounds__(256) k_gamma_grad(
+    int M, const int* __restrict__ row_node, PoolDev pool, const PropDev* __restrict__ props,
+    NetDev net, const float* __restrict__ Gz, const float* __restrict__ Hz, float* __restrict__ GG) {
+  constexpr int NPT = GAMMA_NPT / (RB == 1 ? 1 : 2);  // constraint rows per thread
+  const int mg = blockIdx.y * RB, nr = min(RB, M - mg);
+  __shared__ const PropDev* s_P[RB];
+  __shared__ int s_goff[RB][MNBAB_MAXR + 1], s_e[RB][MNBAB_MAXR + 1];
+  if (threadIdx.x < RB)
+    s_P[threadIdx.x] = props + pool.prop[row_node[mg + min((int)threadIdx.x, nr - 1)]];
   __syncthreads();
-  const PropDev& P = *s_P;
-  if (threadIdx.x <= net.R) {
-    s_goff[threadIdx.x] = threadIdx.x >= 1 ? P.mnc[threadIdx.x].goff : 0;
-    s_e[threadIdx.x] = threadIdx.x >= 1 ? P.mnc[threadIdx.x].e : 0;
+  for (int q = threadIdx.x; q < RB * (net.R + 1); q += blockDim.x) {
+    const int r = q / (net.R + 1), t = q % (net.R + 1);
+    s_goff[r][t] = t >= 1 ? s_P[r]->mnc[t].goff : 0;
+    s_e[r][t] = t >= 1 ? s_P[r]->mnc[t].e : 0;
   }
   __syncthreads();
-  const int E = P.E;
-  const int e0 = blockIdx.x * (blockDim.x * GAMMA_NPT) + threadIdx.x;
+  bool same = true;
 #pragma unroll
-  for (int u = 0; u < GAMMA_NPT; ++u) {
-    const int ef = e0 + u * blockDim.x;
-    if (ef >= E) break;
+  for (int r = 1; r < RB; ++r) same = same && s_P[r] == s_P[0];
+  const int e0 = blockIdx.x * (blockDim.x * NPT) + threadIdx.x;
+  // the gradients at constraint row ef of `rows` rows (at most R) from row r0 of the group on
+  auto grad = [&](int r0, int rows, int ef, auto rc) {
+    constexpr int R = decltype(rc)::value;
+    const PropDev& P = *s_P[r0];
+    if (ef >= P.E) return;
     int i = 0;
     for (int t = 1; t <= net.R; ++t)
-      if (s_e[t] > 0 && ef >= s_goff[t] && ef < s_goff[t] + s_e[t]) i = t;
-    if (i == 0) continue;
+      if (s_e[r0][t] > 0 && ef >= s_goff[r0][t] && ef < s_goff[r0][t] + s_e[r0][t]) i = t;
+    if (i == 0) return;
     const MncDev& mc = P.mnc[i];
-    const int e = ef - s_goff[i];
-    const float* gz = Gz + (size_t)m * net.SD + net.off[i];
-    const float* hz = Hz + (size_t)m * net.SD + net.off[i];
+    const int e = ef - s_goff[r0][i];
+    const size_t z0 = (size_t)(mg + r0) * net.SD + net.off[i];
     const int k = mc.k;
-    float g = -mc.p[e];
+    const float p = mc.p[e];
     if (k == 3) {
-      const int j0 = mc.idx[(size_t)e * 3], j1 = mc.idx[(size_t)e * 3 + 1],
-                j2 = mc.idx[(size_t)e * 3 + 2];
-      const float p0 = mc.P[(size_t)e * 3], p1 = mc.P[(size_t)e * 3 + 1],
-                  p2 = mc.P[(size_t)e * 3 + 2];
-      const float h0 = mc.Ph[(size_t)e * 3], h1 = mc.Ph[(size_t)e * 3 + 1],
-                  h2 = mc.Ph[(size_t)e * 3 + 2];
-      const float z0 = gz[j0], z1 = gz[j1], z2 = gz[j2];
-      const float y0 = hz[j0], y1 = hz[j1], y2 = hz[j2];
-      g = fmaf(p0, z0, g);
-      g = fmaf(h0, y0, g);
-      g = fmaf(p1, z1, g);
-      g = fmaf(h1, y1, g);
-      g = fmaf(p2, z2, g);
-      g = fmaf(h2, y2, g);
+      int j[3];
+      float pc[3], hc[3];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        j[q] = mc.idx[(size_t)e * 3 + q];
+        pc[q] = mc.P[(size_t)e * 3 + q];
+        hc[q] = mc.Ph[(size_t)e * 3 + q];
+      }
+      float z[R][3], y[R][3];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const size_t o = z0 + (size_t)(r < rows ? r : 0) * net.SD;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          z[r][q] = Gz[o + j[q]];
+          y[r][q] = Hz[o + j[q]];
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        float g = -p;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          g = fmaf(pc[q], z[r][q], g);
+          g = fmaf(hc[q], y[r][q], g);
+        }
+        if (r < rows) GG[(size_t)(mg + r0 + r) * pool.EC + ef] = g;
+      }
     } else {
-      for (int kk = 0; kk < k; ++kk) {
-        const int j = mc.idx[(size_t)e * k + kk];
-        g = fmaf(mc.P[(size_t)e * k + kk], gz[j], g);
-        g = fmaf(mc.Ph[(size_t)e * k + kk], hz[j], g);
+      for (int r = 0; r < rows; ++r) {
+        const size_t o = z0 + (size_t)r * net.SD;
+        float g = -p;
+        for (int kk = 0; kk < k; ++kk) {
+          const int j = mc.idx[(size_t)e * k + kk];
+          g = fmaf(mc.P[(size_t)e * k + kk], Gz[o + j], g);
+          g = fmaf(mc.Ph[(size_t)e * k + kk], Hz[o + j], g);
+        }
+        GG[(size_t)(mg + r0 + r) * pool.EC + ef] = g;
       }
     }
-    GG[(size_t)m * pool.EC + ef] = g;
+  };
+  if (RB > 1 && same) {
+#pragma unroll
+    for (int u = 0; u < NPT; ++u)
+      grad(0, nr, e0 + u * blockDim.x, std::integral_constant<int, RB>{});
+    return;
   }
+  // (gridDim.x >= RB)
+  const int r = blockIdx.x % nr, nb = ((int)gridDim.x - r + nr - 1) / nr;
+  const int E = s_P[r]->E, tile = blockDim.x * GAMMA_NPT;
+  for (int t0 = (int)blockIdx.x / nr * tile + (int)threadIdx.x; t0 < E; t0 += nb * tile)
+#pragma unroll
+    for (int u = 0; u < GAMMA_NPT; ++u)
+      grad(r, 1, t0 + u * blockDim.x, std::integral_constant<int, 1>{});
 }
 
 void launch_gamma_grad(int M, const int* row_node, PoolDev pool, const PropDev* props,
                        const NetDev& net, const float* Gz, const float* Hz, float* GG,
                        cudaStream_t st) {
   if (M <= 0 || pool.EC <= 0) return;
-  dim3 grid((pool.EC + 256 * GAMMA_NPT - 1) / (256 * GAMMA_NPT), M);
-  k_gamma_grad<<<grid, 256, 0, st>>>(M, row_node, pool, props, net, Gz, Hz, GG);
+  auto go = [&](auto kern, int rb, int npt) {
+    dim3 grid(std::max((pool.EC + 256 * npt - 1) / (256 * npt), rb), (M + rb - 1) / rb);
+    kern<<<grid, 256, 0, st>>>(M, row_node, pool, props, net, Gz, Hz, GG);
+  };
+  if (M >= GP_GROUP_MIN) go(k_gamma_grad<GP_GROUP>, GP_GROUP, GAMMA_NPT / 2);
+  else go(k_gamma_grad<1>, 1, GAMMA_NPT);
 }
 
 // Projected Adam ascent step (Sec. 3.1): alpha in [0, 1], beta, gamma >= 0.

@@ -320,3 +320,39 @@ def test_dense_products(Context, dims):
                 o = np.concatenate([concat(oa, net.R), concat(ob, net.R)])
                 g = np.concatenate([ga[i], gb[i]])
                 assert np.abs(g - o).max() <= TOL * (1 + np.abs(o).max())
+
+
+# gamma terms of rows in groups (from 32 rows on): groups of one property and of
+# several, a last group that is not full, a property without constraints among them
+@pytest.mark.parametrize("order", ["blocks", "alternating"])
+def test_gamma_terms_of_row_groups(Context, order):
+    spec = dict(seed=33, in_shape=(1, 5, 5), layers=[("fc", 21), ("relu",), ("fc", 9), ("relu",), ("fc", 3)])
+    cases = [_case(spec, 0.05, _rows_per_neuron(5, (300, 1, 40, 0, 229), 3)),
+             _case(spec, 0.04, _rows_per_neuron(6, (7, 230), 2)), _case(spec, 0.06)]
+    rng = np.random.default_rng(12)
+    E = [sum(v.idx.shape[0] for v in (c[5][6] or {}).values()) for c in cases]
+    with Context(node_capacity=512, max_mnc_rows=max(E)) as ctx:
+        gnet = ctx.load_network(cases[0][0])
+        gids, refs = [], []
+        for layers, C, d, lo, hi, prep in cases:
+            net, lo_t, hi_t, l, u, S, m, dense = prep
+            prop = ctx.set_property(gnet, lo, hi, C, d)
+            for t in sorted(m or {}):
+                ctx.set_mnc(prop, t, m[t].idx, m[t].P, m[t].Ph, m[t].p)
+            on = random_node(prep, rng, n_splits=2, row=1)
+            on.split_layer = net.R
+            refs.append(core.bound_and_grad(net, on, on.alpha, on.beta, on.gamma, dense, lo_t, hi_t))
+            gids.append(ctx.node_root(prop, on.row))
+            ctx.import_params(gids[-1], to_params(on, net.R))
+        SD = sum(v.numel() for v in l.values())
+        which = [0] * 14 + [1] * 15 + [2] * 9 if order == "blocks" else [j % 3 for j in range(39)]
+        lb, ga, gb, gg = ctx.bound_grad([gids[j] for j in which], SD, max(E))
+        flat, at = np.concatenate([ga, gb, gg], 1).reshape(-1), 0  # a node: alpha, beta, its gammas
+        for i, j in enumerate(which):
+            ref, _, oa, ob, og = refs[j]
+            assert close(lb[i], float(ref)).all(), (i, j, lb[i], float(ref))
+            o = np.concatenate([concat(oa, net.R), concat(ob, net.R),
+                                *(og[t].numpy() for t in sorted(og or {}))])
+            g = flat[at:at + 2 * SD + E[j]]
+            at += g.size
+            assert np.abs(g - o).max() <= TOL * (1 + np.abs(o).max())
