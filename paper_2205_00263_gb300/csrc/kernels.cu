@@ -2271,45 +2271,88 @@ void launch_reduce_lb(int M, const float* part, int nslot, int used, const float
 }
 
 // Rows (+e_j, -e_j) for every unstable (l < 0 < u) unsplit neuron of a layer,
-// ascending j within a node.
-__global__ void k_collect_rows(const int* nodes, PoolDev pool, int off, int d, int* counter,
-                               int* row_node, int* row_j, float* row_sign) {
+// ascending j within a node.  One CTA per node (its rows lie together), bound by the
+// latency of its loads: a thread has COLLECT_U neurons in flight, 32 consecutive ones
+// per warp, and a tile's segments of 32 are numbered by one scan.  One node of 32768
+// neurons took 65 us with 256 threads and two barriers for each 256 neurons, now 15.6.
+constexpr int COLLECT_T = 1024, COLLECT_U = 8;
+__global__ void __launch_bounds__(COLLECT_T) k_collect_rows(const int* nodes, PoolDev pool, int off,
+                                                            int d, int* counter, int* row_node,
+                                                            int* row_j, float* row_sign) {
+  constexpr int NW = COLLECT_T / 32, SEG = NW * COLLECT_U;  // segments of a tile
   const int n = nodes[blockIdx.x];
   const size_t base = (size_t)n * pool.SD + off;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  __shared__ int s_seg[SEG], s_cnt[NW], s_start, s_run;
+  // bit u: neuron j0 + 32 (NW u + w) + lane gets rows
+  auto flags = [&](int j0) {
+    float l[COLLECT_U], u[COLLECT_U];
+    int sp[COLLECT_U];
+#pragma unroll
+    for (int v = 0; v < COLLECT_U; ++v) {
+      const size_t q = base + min(j0 + 32 * (NW * v + w) + lane, d - 1);
+      l[v] = pool.L[q];
+      u[v] = pool.U[q];
+      sp[v] = pool.S[q];
+    }
+    unsigned f = 0;
+#pragma unroll
+    for (int v = 0; v < COLLECT_U; ++v)
+      if (j0 + 32 * (NW * v + w) + lane < d && l[v] < 0.f && u[v] > 0.f && sp[v] == 0) f |= 1u << v;
+    return f;
+  };
   int cnt = 0;
-  for (int j = threadIdx.x; j < d; j += blockDim.x) {
-    const float l = pool.L[base + j], u = pool.U[base + j];
-    cnt += (l < 0.f && u > 0.f && pool.S[base + j] == 0) ? 1 : 0;
-  }
-  const int tot = (int)block_sum((float)cnt);
-  __shared__ int start;
-  if (threadIdx.x == 0) start = atomicAdd(counter, 2 * tot);
+  for (int j0 = 0; j0 < d; j0 += COLLECT_T * COLLECT_U) cnt += __popc(flags(j0));
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  if (lane == 0) s_cnt[w] = cnt;
   __syncthreads();
-  __shared__ int wsum[32];
-  int run = 0;  // rows emitted before this chunk
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int j0 = 0; j0 < d; j0 += blockDim.x) {
-    const int j = j0 + threadIdx.x;
-    bool f = false;
-    if (j < d) {
-      const float l = pool.L[base + j], u = pool.U[base + j];
-      f = l < 0.f && u > 0.f && pool.S[base + j] == 0;
+  if (threadIdx.x == 0) {
+    int tot = 0;
+    for (int i = 0; i < NW; ++i) tot += s_cnt[i];
+    s_start = atomicAdd(counter, 2 * tot);
+    s_run = 0;
+  }
+  for (int j0 = 0; j0 < d; j0 += COLLECT_T * COLLECT_U) {
+    const unsigned f = flags(j0);
+    unsigned bal[COLLECT_U];
+#pragma unroll
+    for (int v = 0; v < COLLECT_U; ++v) {
+      bal[v] = __ballot_sync(0xffffffffu, f >> v & 1u);
+      if (lane == 0) s_seg[NW * v + w] = __popc(bal[v]);
     }
-    const unsigned bal = __ballot_sync(0xffffffffu, f);
-    const int before_lane = __popc(bal & ((1u << lane) - 1u));
-    if (lane == 0) wsum[w] = __popc(bal);
     __syncthreads();
-    int before_warp = 0, chunk = 0;
-    for (int i = 0; i < nw; ++i) {
-      if (i < w) before_warp += wsum[i];
-      chunk += wsum[i];
+    if (w == 0) {  // exclusive scan of the segments, 8 per lane
+      constexpr int PL = SEG / 32;
+      int c[PL], sum = 0;
+#pragma unroll
+      for (int i = 0; i < PL; ++i) {
+        c[i] = s_seg[lane * PL + i];
+        sum += c[i];
+      }
+      int inc = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += x;
+      }
+      int run = s_run + inc - sum;
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < PL; ++i) {
+        s_seg[lane * PL + i] = run;
+        run += c[i];
+      }
+      if (lane == 31) s_run = run;
     }
-    if (f) {
-      const int r = start + 2 * (run + before_warp + before_lane);
-      row_node[r] = n; row_j[r] = j; row_sign[r] = 1.f;
-      row_node[r + 1] = n; row_j[r + 1] = j; row_sign[r + 1] = -1.f;
-    }
-    run += chunk;
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v < COLLECT_U; ++v)
+      if (f >> v & 1u) {
+        const int j = j0 + 32 * (NW * v + w) + lane;
+        const int r = s_start + 2 * (s_seg[NW * v + w] + __popc(bal[v] & ((1u << lane) - 1u)));
+        row_node[r] = n; row_j[r] = j; row_sign[r] = 1.f;
+        row_node[r + 1] = n; row_j[r + 1] = j; row_sign[r + 1] = -1.f;
+      }
     __syncthreads();
   }
 }
@@ -2317,7 +2360,7 @@ __global__ void k_collect_rows(const int* nodes, PoolDev pool, int off, int d, i
 void launch_collect_rows(int nb, const int* nodes, PoolDev pool, int off, int d, int* counter,
                          int* row_node, int* row_j, float* row_sign, cudaStream_t st) {
   if (nb <= 0) return;
-  k_collect_rows<<<nb, 256, 0, st>>>(nodes, pool, off, d, counter, row_node, row_j, row_sign);
+  k_collect_rows<<<nb, COLLECT_T, 0, st>>>(nodes, pool, off, d, counter, row_node, row_j, row_sign);
 }
 
 __global__ void k_update_bounds(int npairs, const int* row_node, const int* row_j,

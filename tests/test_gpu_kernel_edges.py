@@ -356,3 +356,20 @@ def test_gamma_terms_of_row_groups(Context, order):
             g = flat[at:at + 2 * SD + E[j]]
             at += g.size
             assert np.abs(g - o).max() <= TOL * (1 + np.abs(o).max())
+
+
+# rows of unstable neurons: a second layer of 8649 neurons (a tile of 8192 and a ragged
+# one), of 7 and of 33
+@pytest.mark.parametrize("layers,shape", [
+    ([("conv", 9, 3, 1, 1), ("relu",), ("conv", 9, 1, 1, 0), ("relu",), ("fc", 3)], (1, 31, 31)),
+    ([("fc", 40), ("relu",), ("fc", 7), ("relu",), ("fc", 33), ("relu",), ("fc", 3)], (1, 5, 5)),
+])
+def test_rows_of_unstable_neurons(Context, layers, shape):
+    layers, C, d, lo, hi, prep = _case(dict(seed=91, in_shape=shape, layers=layers), 0.05)
+    l, u = prep[3], prep[4]
+    with Context(node_capacity=64) as ctx:
+        gnet = ctx.load_network(layers)
+        prop = ctx.set_property(gnet, lo, hi, C, d)
+        for i in l:
+            gl, gu = ctx.root_bounds(prop, i)
+            assert close(gl, l[i].numpy()).all() and close(gu, u[i].numpy()).all(), i
