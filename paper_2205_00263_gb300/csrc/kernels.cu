@@ -29,9 +29,14 @@ __device__ float block_sum(float v) {
   return r;
 }
 
+// Allows a kernel `bytes` of dynamic shared memory.  The 48 KB that need no leave
+// include the kernel's static shared memory (up to 9 KB here).  The limit is the same
+// for every launch of a kernel, so that host threads do not lower it for one another.
 template <typename F>
 static void set_smem(F f, int bytes) {
-  if (bytes > 48 * 1024) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (bytes > 32 * 1024)
+    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         std::max(bytes, 208 * 1024));
 }
 
 // ---------------------------------------------------------------------------

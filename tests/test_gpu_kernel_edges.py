@@ -373,3 +373,50 @@ def test_rows_of_unstable_neurons(Context, layers, shape):
         for i in l:
             gl, gu = ctx.root_bounds(prop, i)
             assert close(gl, l[i].numpy()).all() and close(gu, u[i].numpy()).all(), i
+
+
+# the fused optimisation loop: FC outputs that give a warp one, two, four and seven
+# at a time and more than one round of them, FC inputs that are no multiple of four,
+# stride classes of one, two and three taps, planes whose last pair of positions is
+# half empty; on both the SIMT (1) and the tensor-core (0) form
+@pytest.mark.parametrize("path", [0, 1])
+@pytest.mark.parametrize("layers,shape", [
+    ([("fc", 130), ("relu",), ("fc", 65), ("relu",), ("fc", 33), ("relu",), ("fc", 17), ("relu",), ("fc", 3)],
+     (1, 5, 6)),
+    ([("conv", 6, 5, 2, 2), ("relu",), ("conv", 8, 3, 3, 1), ("relu",), ("fc", 113), ("relu",), ("fc", 4)],
+     (1, 13, 11)),
+    ([("conv", 8, 3, 1, 1), ("relu",), ("conv", 4, 2, 3, 0), ("relu",), ("fc", 31), ("relu",), ("fc", 3)],
+     (2, 9, 7)),
+])
+def test_fused_optimisation_layers(Context, layers, shape, path):
+    layers, C, d, lo, hi, prep = _case(dict(seed=95, in_shape=shape, layers=layers), 0.03)
+    net, lo_t, hi_t = prep[:3]
+    dense = prep[7]
+    rng = np.random.default_rng(13)
+    with Context(node_capacity=64, gemm_path=path) as ctx:
+        gnet = ctx.load_network(layers)
+        prop = ctx.set_property(gnet, lo, hi, C, d)
+        nodes = [random_node(prep, rng, n_splits=j, row=j % 2, gamma_scale=0.0) for j in range(4)]
+        gids = []
+        for on in nodes:
+            on.split_layer = net.R
+            gids.append(ctx.node_root(prop, on.row))
+            ctx.import_params(gids[-1], to_params(on, net.R))
+        best = ctx.optimize(gids, steps=5)
+        for j, on in enumerate(nodes):
+            top, *_ = core.optimize(net, on, dense, lo_t, hi_t, core.AdamHP(steps=5))
+            assert close(best[j], top).all(), (j, best[j], top)
+
+
+def test_autotune_first_thing(Context):
+    """Every variant of every layer runs in a context that has launched nothing
+    else: layers whose staging takes exactly 48 KB of dynamic shared memory beside
+    their kernel's static variables (stride-2 transposed convolutions from 64 x 8 x 8
+    and 32 x 16 x 16)."""
+    layers = synth.make_network(dict(seed=97, in_shape=(32, 32, 32), layers=[
+        ("conv", 32, 4, 2, 1), ("relu",), ("conv", 64, 3, 1, 1), ("relu",), ("conv", 64, 4, 2, 1),
+        ("relu",), ("fc", 3)]))
+    with Context(node_capacity=512) as ctx:
+        net = ctx.load_network(layers)
+        recs = ctx.autotune(net, max_rows=64)
+        assert recs and all(r["variant"] != "auto" for r in recs)
