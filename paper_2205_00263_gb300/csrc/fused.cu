@@ -73,10 +73,24 @@ __device__ __forceinline__ int f_split(int items) {
   return ks;
 }
 
+// x / d by the rounded-up reciprocal m = ceil(2^32 / d), exact for x d < 2^32 (the
+// fused kernels' indices stay below 2^16, their layers fit in shared memory), without
+// the general form's correction; a convolution step decodes its item with ten
+// divisions by layer sizes.
+struct SDiv {
+  unsigned d, m;
+};
+__host__ __device__ inline SDiv s_div_of(int d) {
+  return SDiv{(unsigned)d, d <= 1 ? 0u : 0xffffffffu / (unsigned)d + 1u};
+}
+__device__ __forceinline__ int s_div(int x, SDiv v) {
+  return v.m ? (int)__umulhi((unsigned)x, v.m) : x;
+}
+
 struct FusedIdx {
   struct Layer {
-    FDiv pp, w2, s;   // transposed step: first positions, those of a row, stride
-    FDiv p, wo;       // forward step: output positions, their columns
+    SDiv pp, w2, s;   // transposed step: first positions, those of a row, stride
+    SDiv p, wo;       // forward step: output positions, their columns
   } l[MNBAB_MAXR + 2];
 };
 
@@ -86,8 +100,8 @@ static FusedIdx fused_idx(const NetDev& net) {
     const LayerDev& L = net.aff[t];
     if (L.kind != MNBAB_CONV2D) continue;
     const int w2 = (L.wi + 2 * L.s - 1) / (2 * L.s) * L.s;
-    x.l[t] = {f_div_of(L.hi * w2), f_div_of(w2), f_div_of(L.s), f_div_of(L.ho * L.wo),
-              f_div_of(L.wo)};
+    x.l[t] = {s_div_of(L.hi * w2), s_div_of(w2), s_div_of(L.s), s_div_of(L.ho * L.wo),
+              s_div_of(L.wo)};
   }
   return x;
 }
@@ -287,16 +301,16 @@ __device__ void f_conv_back(const LayerDev& L, const FusedIdx::Layer& X, const f
     int grp = 0, ih = 0, iw = 0;
     bool two = false;
     if (act) {
-      grp = f_div(it, X.pp);
+      grp = s_div(it, X.pp);
       const int q = it - grp * PP;
-      ih = f_div(q, X.w2);
-      const int qw = q - ih * W2, qs = f_div(qw, X.s);
+      ih = s_div(q, X.w2);
+      const int qw = q - ih * W2, qs = s_div(qw, X.s);
       iw = qs * S + qw;
       act = iw < L.wi;
       two = iw + S < L.wi;
     }
     if (act) {
-      const int oh0 = f_div(ih + L.p, X.s), ow0 = f_div(iw + L.p, X.s);
+      const int oh0 = s_div(ih + L.p, X.s), ow0 = s_div(iw + L.p, X.s);
       const int kh0 = ih + L.p - oh0 * S, kw0 = iw + L.p - ow0 * S;
       const int da = ks * hwo, dw = ks * (int)wco, n = (L.co - k0 + ks - 1) >> lg;
       for (int kh = kh0, oh = oh0; kh < L.k && oh >= 0; kh += S, --oh) {
@@ -392,9 +406,9 @@ __device__ void f_conv_fwd_cb(const LayerDev& L, const FusedIdx::Layer& X, const
     for (int u = 0; u < C2; ++u) acc[u] = make_float2(0.f, 0.f);
     int grp = 0, pos = 0;
     if (act) {
-      grp = f_div(it, X.p);
+      grp = s_div(it, X.p);
       pos = it - grp * P;
-      const int oh = f_div(pos, X.wo), ow = pos - oh * L.wo;
+      const int oh = s_div(pos, X.wo), ow = pos - oh * L.wo;
       const int ih0 = oh * L.s - L.p, iw0 = ow * L.s - L.p;
       const int kh_lo = max(0, -ih0), kh_hi = min(L.k, L.hi - ih0);
       const int kw_lo = max(0, -iw0), kw_hi = min(L.k, L.wi - iw0);

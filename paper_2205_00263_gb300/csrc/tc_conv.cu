@@ -18,20 +18,27 @@
 //    class as [K / 4][N][4] in HBM and staged by TMA (a 3-D tiled tensor map,
 //    cp.async.bulk.tensor), which lands it in the canonical no-swizzle K-major
 //    layout (core matrices along K N x 16 B apart, along N 128 B apart);
-//  - A is the implicit im2col operand: each thread gathers its position's 32
-//    reduction values of a K block from the coefficient rows (L2), splits
-//    them into hi / lo and stores them in the canonical layout;
-//  - two stages: the threads gather block k + 1 while the tensor core runs
-//    block k (3 MMAs of K = 8 per K step: hi.hi + hi.lo + lo.hi, FP32
-//    accumulation in tensor memory);
+//  - A is the implicit im2col operand and lives in tensor memory (a GEMM row is a
+//    TMEM lane): each of the 256 gather threads takes 16 of a K block's 32 reduction
+//    values of its position from the coefficient rows (L2), splits them into hi / lo
+//    and stores them with tcgen05.st into one of TC_AST stages; block k + 1's loads
+//    are in flight meanwhile;
+//  - one thread of a control warp streams the weights through a ring of TC_WST
+//    stages and issues each block's MMAs (3 of K = 8 per K step: lo.hi + hi.lo +
+//    hi.hi, FP32 accumulation in tensor memory, in that order);
 //  - the epilogue reads each warp's 32 TMEM lanes (one objective row) with
-//    tcgen05.ld and applies the same epilogue functions as the SIMT kernels, one
-//    instantiation per kind and a rolled loop over eight channels: unrolled with
-//    a switch on the kind at every output, the CTAs waited for instructions (64
-//    rows: conv_tc 10.0 ms of 20 Adam steps of the 3x32x32 network, now 6.6; 128
-//    rows of the residual one 10.2, now 6.3);
+//    tcgen05.ld, eight channels at a time whose inputs are loaded together, one
+//    instantiation per kind of epilogue and rolled: unrolled with a switch on the kind
+//    at every output, the CTAs waited for instructions, and loads behind a branch per
+//    output followed one another;
 //    a row's offset partial is a warp reduction in a fixed order, written to
 //    slot (class, position chunk), so it does not depend on the other rows.
+// What bounds a CTA now is its chain of accumulating MMAs: about 125 cycles each
+// whatever N <= 64 is, twelve to a K block.  Measured, 20 Adam steps: 64 rows of
+// conv_big_32's convolutions 10.0 ms at first, 6.6 with the rolled epilogues, 5.4
+// now; 128 rows of resnet_32's 10.2, 6.3 and 5.1.  Splitting the chain over two
+// accumulators would change the order of the sums; more CTAs per SM do not fit beside
+// two of 256 TMEM columns.
 // Every wait is bounded; on timeout the kernel sets the device error flag,
 // gives its MMAs one more bounded wait, frees its tensor memory and returns.
 #include <cuda.h>
