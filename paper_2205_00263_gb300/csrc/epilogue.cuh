@@ -126,9 +126,9 @@ __device__ __forceinline__ float epi_apply(const Epi& e, int m, int j, float v, 
 }
 
 // Two-phase form of epi_apply for kernels that finish several outputs per
-// thread: epi_load issues every global load an output's epilogue needs (so the
-// loads of all of a thread's outputs are in flight together), epi_finish does
-// the same arithmetic as epi_apply on the loaded values.
+// thread: epi_load_node and epi_load_own issue every global load an output's
+// epilogue needs (so the loads of all of a thread's outputs are in flight together),
+// epi_finish does the same arithmetic as epi_apply on the loaded values.
 struct EpiIn {
   float acc, l, u, al, be, gp, gph;
   float cb;  // bias of the consuming affine layer at j (ReLU step)
@@ -144,36 +144,8 @@ __device__ __forceinline__ float epi_colbias(const Epi& e, int j) {
   return e.kind == EPI_RELU ? e.bias[j / e.bias_div] : 0.f;
 }
 
-// every input of output (m, j) except the column bias (in.cb)
-__device__ __forceinline__ void epi_load_row(const Epi& e, int n, const PropDev* P, int m, int j,
-                                             EpiIn& in) {
-  in.acc = e.acc_in ? e.acc_in[(size_t)m * e.acc_ld + j] : 0.f;
-  in.al = in.be = in.gp = in.gph = 0.f;
-  in.s = 0;
-  if (e.kind == EPI_RELU || e.kind == EPI_ADJ) {
-    const size_t q = (size_t)n * e.SD + e.off + j;
-    const size_t qm = (size_t)m * e.SD + e.off + j;
-    in.l = e.pool.L[q];
-    in.u = e.pool.U[q];
-    in.s = e.pool.S[q];
-    if (e.kind == EPI_RELU) {
-      if (e.final_mode) {
-        in.al = e.pool.ALPHA[q];
-        in.be = e.pool.BETA[q];
-      }
-      if (e.GP) in.gp = e.GP[qm];
-      if (e.GPh) in.gph = e.GPh[qm];
-    } else {
-      in.al = e.pool.ALPHA[q];
-      in.gp = e.AP[qm];
-    }
-  } else if (e.kind == EPI_CONC) {
-    in.l = P->lo[j];
-    in.u = P->hi[j];
-  }
-}
-
-// epi_load_row in two parts: the inputs that depend on the node and column only
+// every input of output (m, j) except the column bias (in.cb), in two parts: the
+// inputs that depend on the node and column only
 // (bounds, split, slope, multiplier; the input box), which rows of one node can
 // share, and those of the row itself
 __device__ __forceinline__ void epi_load_node(const Epi& e, int n, const PropDev* P, int j,
@@ -203,12 +175,6 @@ __device__ __forceinline__ void epi_load_own(const Epi& e, int m, int j, EpiIn& 
   } else if (e.kind == EPI_ADJ) {
     in.gp = e.AP[qm];
   }
-}
-
-__device__ __forceinline__ void epi_load(const Epi& e, int n, const PropDev* P, int m, int j,
-                                         EpiIn& in) {
-  epi_load_row(e, n, P, m, j, in);
-  in.cb = epi_colbias(e, j);
 }
 
 __device__ __forceinline__ float epi_finish(const Epi& e, int m, int j, float v, const EpiIn& in,
