@@ -70,7 +70,6 @@ struct mnbab_net {
   PoolDev pool{};
   int cap = 0;
   std::vector<int> free_slots;
-  int held = 0;  // free slots kept for the row root nodes of started properties
   std::vector<int> slot_split;  // host metadata per slot
   std::vector<int> slot_row;
   std::vector<int> slot_prop;
@@ -140,7 +139,7 @@ struct mnbab_prop {
   std::vector<mnbab_trace_rec> trace;
   int mnc_set[MNBAB_MAXR + 1] = {0};
   bool root_pending = false;         // root bounds not computed yet
-  bool rows_pending = false;         // started, row root nodes not created yet
+  std::vector<int> root_row_slots;   // its row root nodes, initialised with the bounds
   bool admitted = true;              // false while queued in the request loop
   bool materialized = false;         // node slots allocated
   int inter_steps = 0;               // Adam steps of optimised root intermediate bounds
@@ -457,12 +456,8 @@ double layer_wbytes(const LayerDev& L) {
 // ---------------------------------------------------------------------------
 // node pool
 // ---------------------------------------------------------------------------
-int free_count(const mnbab_net* n) { return std::max(0, (int)n->free_slots.size() - n->held); }
-
-// `own`: the slot is one of those held for row root nodes
-int alloc_slot(mnbab_net* n, bool own = false) {
-  if (own ? n->free_slots.empty() : free_count(n) < 1)
-    fail(MNBAB_E_BUDGET, "node pool exhausted");
+int alloc_slot(mnbab_net* n) {
+  if (n->free_slots.empty()) fail(MNBAB_E_BUDGET, "node pool exhausted");
   const int s = n->free_slots.back();
   n->free_slots.pop_back();
   n->slot_used[s] = 1;
@@ -1415,7 +1410,7 @@ void attack_layers(mnbab_ctx* c, const mnbab_prop* p, int n_starts, int steps, c
                    float* best_out, float* x_out, std::vector<double>* f64_out) {
   mnbab_net* n = p->net;
   const int nr = p->n_rows, d0 = n->d0, Q = nr * n_starts;
-  const int Qc = std::min({Q, n->B, n->chunk, free_count(n)});
+  const int Qc = std::min({Q, n->B, n->chunk, (int)n->free_slots.size()});
   if (Qc < 1) fail(MNBAB_E_BUDGET, "node pool exhausted");
   const size_t need = (size_t)n_starts * d0 + (size_t)Qc * (2 * (size_t)d0 + 1);
   if (n->atk_cap < need) {
@@ -1473,7 +1468,7 @@ void attack_layers(mnbab_ctx* c, const mnbab_prop* p, int n_starts, int steps, c
   if (!f64_out) return;
   // FP64 margins of the chosen points (row r's point in a slot of row r)
   f64_out->assign(nr, 0.0);
-  const int Rc = std::min({nr, n->B, free_count(n)});
+  const int Rc = std::min({nr, n->B, (int)n->free_slots.size()});
   if (Rc < 1) fail(MNBAB_E_BUDGET, "node pool exhausted");
   for (int r0 = 0; r0 < nr; r0 += Rc) {
     const int M = std::min(Rc, nr - r0);
@@ -1620,18 +1615,19 @@ bool pre_attack(mnbab_ctx* c, mnbab_prop* p) {
   return false;
 }
 
-// Starts a property: its root-bound slot (l = -inf, u = +inf, re-bounded from
-// layer 1 with the next batch of admissions).  Its row root nodes are open from
-// here on and their slots are held, but they are created by its first BaB step
-// (open_rows): a caller that reads root bounds only writes none of them (9 rows
-// of the 3x32x32 network are 10 MB and 10 slots a property).
+// Starts a property.  It takes its node slots together or, where the pool cannot
+// hold them all, none of them: the root-bound slot (l = -inf, u = +inf, re-bounded
+// from layer 1 with the other properties started by the call) and one root node per
+// row.  ensure_roots, which starts properties, also writes these nodes, so that a
+// queued node is always a written one.
 void materialize(mnbab_net* n, mnbab_prop* p) {
   mnbab_ctx* c = n->ctx;
   if (p->atk_starts > 0 && pre_attack(c, p)) {
     p->materialized = true;  // falsified before any node: nothing to bound
     return;
   }
-  const int rs = alloc_slot(n, true);
+  if ((int)n->free_slots.size() < p->n_rows + 1) fail(MNBAB_E_BUDGET, "node pool exhausted");
+  const int rs = alloc_slot(n);
   p->root_slot = rs;
   n->slot_prop[rs] = p->index;
   n->slot_row[rs] = 0;
@@ -1640,47 +1636,17 @@ void materialize(mnbab_net* n, mnbab_prop* p) {
   // properties started together, in one launch (ensure_roots)
   n->new_roots.push_back(rs);
   n->new_root_props.push_back(p->index);
-  for (int r = 0; r < p->n_rows; ++r) p->row_open[r]++;
-  n->held += p->n_rows;
-  p->rows_pending = true;
+  for (int r = 0; r < p->n_rows; ++r) {
+    const int sl = alloc_slot(n);
+    n->slot_prop[sl] = p->index;
+    n->slot_row[sl] = r;
+    n->slot_split[sl] = n->R;
+    p->root_row_slots.push_back(sl);
+    p->queue.push_back(QNode{sl, p->next_seq++, r, 0, n->R});
+    p->row_open[r]++;
+  }
   p->root_pending = true;
   p->materialized = true;
-}
-
-// The row root nodes of the given started properties that have none yet, from
-// their root bounds, queued in row order.
-void open_rows(mnbab_net* n, mnbab_prop* const* props, int n_props) {
-  mnbab_ctx* c = n->ctx;
-  std::vector<int> dst, src, row;
-  auto flush = [&]() {
-    if (dst.empty()) return;
-    h2d(c, n->ri_dst, dst.data(), dst.size());
-    h2d(c, n->ri_src, src.data(), src.size());
-    h2d(c, n->ri_row, row.data(), row.size());
-    Scope sc(c, C_BOOK, 0.0, 25.0 * dst.size() * n->SD);
-    launch_root_init((int)dst.size(), n->ri_dst, n->ri_src, n->ri_row, n->pool, c->st);
-    // the index vectors were staged when they were enqueued: they can be reused
-    dst.clear(); src.clear(); row.clear();
-  };
-  for (int i = 0; i < n_props; ++i) {
-    mnbab_prop* p = props[i];
-    if (!p->rows_pending) continue;
-    if ((int)n->free_slots.size() < p->n_rows) fail(MNBAB_E_BUDGET, "node pool exhausted");
-    for (int r = 0; r < p->n_rows; ++r) {
-      if ((int)dst.size() == 2 * n->B) flush();
-      const int sl = alloc_slot(n, true);
-      n->slot_prop[sl] = p->index;
-      n->slot_row[sl] = r;
-      n->slot_split[sl] = n->R;
-      p->queue.push_back(QNode{sl, p->next_seq++, r, 0, n->R});
-      dst.push_back(sl);
-      src.push_back(p->root_slot);
-      row.push_back(r);
-    }
-    n->held -= p->n_rows;
-    p->rows_pending = false;
-  }
-  flush();
 }
 
 // Optimised intermediate bounds (Sec. 3.1, parameter sharing).  For ReLU
@@ -1928,7 +1894,28 @@ void ensure_roots(mnbab_net* n, mnbab_prop* const* only = nullptr, int n_only = 
     a.steps = steps;
     optimize_intermediate_impl(n, grp, 2, a);
   }
-  for (auto* p : pend) p->root_pending = false;
+  std::vector<int> dst, src, row;
+  auto flush = [&]() {
+    if (dst.empty()) return;
+    h2d(c, n->ri_dst, dst.data(), dst.size());
+    h2d(c, n->ri_src, src.data(), src.size());
+    h2d(c, n->ri_row, row.data(), row.size());
+    Scope sc(c, C_BOOK, 0.0, 25.0 * dst.size() * n->SD);
+    launch_root_init((int)dst.size(), n->ri_dst, n->ri_src, n->ri_row, n->pool, c->st);
+    // the index vectors were staged when they were enqueued: they can be reused
+    dst.clear(); src.clear(); row.clear();
+  };
+  for (auto* p : pend) {
+    for (size_t r = 0; r < p->root_row_slots.size(); ++r) {
+      if ((int)dst.size() == 2 * n->B) flush();
+      dst.push_back(p->root_row_slots[r]);
+      src.push_back(p->root_slot);
+      row.push_back((int)r);
+    }
+    p->root_pending = false;
+    p->root_row_slots.clear();
+  }
+  flush();
 }
 
 // Uploads the constraint rows of one ReLU layer of a property (row form and
@@ -2128,7 +2115,6 @@ void bab_step_impl(mnbab_ctx* c, mnbab_prop* const* props, int n_props, int max_
   max_nodes = std::max(1, std::min(max_nodes, n->B));
   HostTimer ht(c);
   ensure_roots(n, props, n_props);
-  open_rows(n, props, n_props);
   ht.lap(H_ROOTS);
   {
     const double t = now_s();
@@ -3437,7 +3423,7 @@ mnbab_status mnbab_queue_size(const mnbab_ctx* cc, const mnbab_prop* p, int32_t*
   mnbab_ctx* c = const_cast<mnbab_ctx*>(cc);
   API_BEGIN(c)
   if (!p || !n_out) fail(MNBAB_E_INVALID_ARG, "null argument");
-  *n_out = p->rows_pending ? p->n_rows : (int)p->queue.size();
+  *n_out = (int)p->queue.size();
   API_END(c)
 }
 
