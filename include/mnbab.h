@@ -355,7 +355,10 @@ mnbab_status mnbab_score_branches(mnbab_ctx* ctx, const mnbab_node_id* nodes, in
  * every property set on the network.  A caller can so upload many properties
  * ahead of time and step a window of them.  cfg may be
  * NULL (20 steps, default rates).  max_nodes is clamped to the context's batch
- * capacity. */
+ * capacity.  A step that fails settles no node that it would have branched:
+ * without room for the children of all of them (MNBAB_E_BUDGET) these nodes are
+ * open again, at the head of their queues and with the parameters that the step
+ * reached; the nodes that it verified or falsified are settled. */
 mnbab_status mnbab_bab_step(mnbab_ctx* ctx, mnbab_prop* const* props, int32_t n_props,
                             int32_t max_nodes, const mnbab_adam* cfg, mnbab_step_stats* out);
 

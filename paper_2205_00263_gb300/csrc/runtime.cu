@@ -2100,6 +2100,31 @@ struct Picked {
   QNode q;
 };
 
+// The popped nodes of a step, until they are settled.  A step that fails (no slots for
+// the children, a device error) puts the others back at the head of their queues, in
+// their order: a property that lost open nodes would read as verified once its queue
+// is empty.
+struct Popped {
+  std::vector<Picked> v;
+  std::vector<char> settled;
+  void add(mnbab_prop* p) {
+    v.push_back({p, p->queue.front()});
+    settled.push_back(0);
+    p->queue.pop_front();
+    p->bounded++;
+    p->row_open[v.back().q.row]--;
+  }
+  ~Popped() {
+    for (size_t i = v.size(); i-- > 0;) {
+      if (settled[i]) continue;
+      mnbab_prop* p = v[i].p;
+      p->queue.push_front(v[i].q);
+      p->bounded--;
+      p->row_open[v[i].q.row]++;
+    }
+  }
+};
+
 void bab_step_impl(mnbab_ctx* c, mnbab_prop* const* props, int n_props, int max_nodes,
                    const mnbab_adam& adam, mnbab_step_stats* st) {
   std::memset(st, 0, sizeof(*st));
@@ -2122,17 +2147,14 @@ void bab_step_impl(mnbab_ctx* c, mnbab_prop* const* props, int n_props, int max_
       if (props[i]->materialized && props[i]->t_start == 0.0) props[i]->t_start = t;
   }
   // pop FIFO
-  std::vector<Picked> picked;
+  Popped popped;
+  const std::vector<Picked>& picked = popped.v;
   for (int i = 0; i < n_props && (int)picked.size() < max_nodes; ++i) {
     mnbab_prop* p = props[i];
     if (!p->materialized) continue;
     while (!p->done && !p->queue.empty() && p->bounded < p->budget &&
-           (int)picked.size() < max_nodes) {
-      picked.push_back({p, p->queue.front()});
-      p->queue.pop_front();
-      p->bounded++;
-      p->row_open[picked.back().q.row]--;
-    }
+           (int)picked.size() < max_nodes)
+      popped.add(p);
   }
   const int M = (int)picked.size();
   st->nodes_bounded = M;
@@ -2291,11 +2313,12 @@ void bab_step_impl(mnbab_ctx* c, mnbab_prop* const* props, int n_props, int max_
     std::vector<int> par, lay, neu;
     std::vector<int> kidslots;
     std::vector<std::pair<int, int>> branch_of;  // (picked index, opt index)
+    std::vector<mnbab_trace_rec> recs(M);
     int oi = 0;
     for (int i = 0; i < M; ++i) {
       mnbab_prop* p = picked[i].p;
       const QNode& q = picked[i].q;
-      mnbab_trace_rec rec{};
+      mnbab_trace_rec& rec = recs[i];
       rec.seq = q.seq;
       rec.row = q.row;
       rec.depth = q.depth;
@@ -2366,11 +2389,16 @@ void bab_step_impl(mnbab_ctx* c, mnbab_prop* const* props, int n_props, int max_
           }
         }
       }
-      p->trace.push_back(rec);
+      popped.settled[i] = release;
       if (release) free_slot(n, q.slot);
     }
-    // children
+    // children; without room for all of them no node is branched, and the nodes to
+    // branch are open again
     const int nb = (int)par.size();
+    const bool room = 2 * (size_t)nb <= n->free_slots.size();
+    for (int i = 0; i < M; ++i)
+      if (room || popped.settled[i]) picked[i].p->trace.push_back(recs[i]);
+    if (!room) fail(MNBAB_E_BUDGET, "node pool exhausted");
     if (nb > 0) {
       kidslots.resize(2 * nb);
       for (int b = 0; b < nb; ++b) {
@@ -2396,6 +2424,7 @@ void bab_step_impl(mnbab_ctx* c, mnbab_prop* const* props, int n_props, int max_
           pk.p->queue.push_back(QNode{s, pk.p->next_seq++, pk.q.row, pk.q.depth + 1, lay[b]});
           pk.p->row_open[pk.q.row]++;
         }
+        popped.settled[branch_of[b].first] = 1;
       }
       // no synchronisation: a freed parent slot is reused only by later work on
       // the same stream, after the children have copied it

@@ -1,6 +1,6 @@
 """Node pools that are too small: a call that finds too few slots is refused with
-MNBAB_E_BUDGET and leaves every property as it was, so that later calls give what
-they give in a large pool."""
+MNBAB_E_BUDGET and leaves every property's open nodes open, so that later calls end as
+in a large pool."""
 import numpy as np
 import pytest
 import torch
@@ -67,3 +67,27 @@ def test_refused_start_leaves_the_started_ones(Context, refused_by):
             assert ctx.queue_size(p) == big.queue_size(ref) == ROWS + 1
         _refused(lambda: ctx.bab_step([c], max_nodes=1, steps=STEPS))
         assert ctx.queue_size(c) == 0 and _key(ctx, c) == []
+
+
+def test_refused_children_leave_their_nodes_open(Context):
+    """A step whose nodes branch finds room for one child: its nodes are open again and
+    nothing is decided.  With room the property ends as in a large pool (falsified, where
+    a queue that had lost its nodes read as verified)."""
+    case = _case()
+    cap = 64
+    with Context(node_capacity=cap) as ctx, Context(node_capacity=256) as big:
+        net, ref_net = ctx.load_network(case[0]), big.load_network(case[0])
+        a, ref = _property(ctx, net, case), _property(big, ref_net, case)
+        extra = [ctx.node_root(a, 0) for _ in range(cap - 1 - (ROWS + 1) - 1)]
+        _refused(lambda: ctx.bab_step([a], max_nodes=ROWS, steps=STEPS))
+        assert ctx.queue_size(a) == ROWS and _key(ctx, a) == []
+        assert ctx.status(a)[0] == 0
+        assert [ctx.verdict(a, r)[0] for r in range(-1, ROWS)] == [0] * (ROWS + 1)
+        for n in extra:
+            ctx.node_free(n)
+        for c, p in ((ctx, a), (big, ref)):
+            while c.bab_step([p], max_nodes=ROWS, steps=STEPS)["nodes_bounded"]:
+                pass
+        assert ctx.verdict(a)[0] == big.verdict(ref)[0] == -1
+        seqs = [k[0] for k in _key(ctx, a)]
+        assert seqs == sorted(seqs) and seqs[:ROWS] == list(range(ROWS))
