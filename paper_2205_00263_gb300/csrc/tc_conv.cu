@@ -429,7 +429,7 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-int conv_tc_smem(int NP, int Kp) {
+constexpr int conv_tc_smem(int NP, int Kp) {
   return 1024 + TC_WST * 2 * NP * KC * 4 + Kp * (int)sizeof(int2);
 }
 
@@ -516,7 +516,11 @@ int launch_tc_conv(const LayerDev& L, int dir, int M, const float* in, int ld_in
   const dim3 grid(t->ncls[dir] * t->nchunk[dir], (M + TROWS - 1) / TROWS);
   const int NP = t->NP[dir], smem = conv_tc_smem(NP, t->Kp[dir]);
   auto go = [&](auto kern) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // the most that any layer takes (17 to 73 KB), for every layer: the limit belongs to the
+    // kernel, and a host thread that set its own layer's size between another thread's
+    // set and launch made that launch fail
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         conv_tc_smem(64, TC_KMAX));
     kern<<<grid, TC_THREADS, smem, st>>>(t->hi[dir], t->lo[dir], L, dir, NP, M, t->nchunk[dir], in,
                                          ld_in, out, ld_out, e, e.err);
   };
