@@ -31,12 +31,13 @@ __device__ float block_sum(float v) {
 
 // Allows a kernel `bytes` of dynamic shared memory.  The 48 KB that need no leave
 // include the kernel's static shared memory (up to 9 KB here).  The limit is the same
-// for every launch of a kernel, so that host threads do not lower it for one another.
+// for every launch of a kernel, the most that any launch of this file takes
+// (win_plan), so that host threads do not lower it for one another.
+constexpr int SMEM_MOST = 216 * 1024;
 template <typename F>
 static void set_smem(F f, int bytes) {
   if (bytes > 32 * 1024)
-    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         std::max(bytes, 208 * 1024));
+    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MOST);
 }
 
 // ---------------------------------------------------------------------------
@@ -303,8 +304,8 @@ bool win_plan(const NetDev& net, int t, WinPlan& wp) {
     wp.wide = wp.wide || (ci & 3) == 0 || ci == 2 || ci == 3;
   }
   const int most = !wp.wide && wp.vt == 256 ? 4 : WIN_RB_MAX;
-  wp.rb = bytes(most) <= 104 * 1024 ? most : bytes(4) <= 216 * 1024 ? 4 : 1;
-  return bytes(wp.rb) <= 216 * 1024;
+  wp.rb = bytes(most) <= 104 * 1024 ? most : bytes(4) <= SMEM_MOST ? 4 : 1;
+  return bytes(wp.rb) <= SMEM_MOST;
 }
 
 // x / d for the small operands of window indices (x d < 2^32), by the rounded-up

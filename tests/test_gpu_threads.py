@@ -11,9 +11,6 @@ import synth
 
 pytestmark = pytest.mark.gpu
 
-CALLS = 10000
-
-
 @pytest.fixture(scope="module")
 def Context():
     if not torch.cuda.is_available():
@@ -24,27 +21,28 @@ def Context():
     return Context
 
 
-def _calls(Context, spec, gemm_path, fused, calls, go=lambda i: True):
-    """The values of `calls` calls that re-bound a root node and bound it (and optimise and
-    attack it), which are all the same; go(i): whether to make call i."""
+def _calls(Context, spec, gemm_path, nodes, fused, calls, go=lambda i: True):
+    """The values of `calls` calls that re-bound root nodes, two rows a launch, and bound
+    them (and optimise and attack), which are all the same; go(i): whether to make call i."""
     layers = synth.make_network(spec)
     x = synth.make_image(spec["seed"], spec["in_shape"]).reshape(-1)
     lo, hi = synth.input_box(x, 0.02)
     C, d = synth.property_rows(0, 3)
     first = None
-    with Context(node_capacity=16, gemm_path=gemm_path) as ctx:
+    with Context(node_capacity=32, gemm_path=gemm_path, row_chunk=2) as ctx:
         net = ctx.load_network(layers)
         prop = ctx.set_property(net, lo, hi, C, d)
-        node = ctx.node_root(prop, 0)
-        start = ctx.export_params(node)
+        ids = [ctx.node_root(prop, 0) for _ in range(nodes)]
+        start = ctx.export_params(ids[0])
         start.split_layer = 1  # the layers above are bounded again
         for i in range(calls):
             if not go(i):
                 break
-            ctx.import_params(node, start)
-            got = list(ctx.bound_batch([node]))
+            for n in ids:
+                ctx.import_params(n, start)
+            got = list(ctx.bound_batch(ids))
             if fused:
-                got += [ctx.optimize([node], steps=1), ctx.attack(prop, np.stack([lo, hi]), 1)[0]]
+                got += [ctx.optimize(ids, steps=1), ctx.attack(prop, np.stack([lo, hi]), 1)[0]]
             got = np.concatenate([np.ravel(g) for g in got])
             first = got if first is None else first
             assert (got == first).all(), (i, got, first)
@@ -52,19 +50,26 @@ def _calls(Context, spec, gemm_path, fused, calls, go=lambda i: True):
 
 
 # a pair of networks: the first one's launches take more than the second one's limit
-@pytest.mark.parametrize("gemm_path,fused,large,small", [
+@pytest.mark.parametrize("gemm_path,nodes,fused,calls,large,small", [
     # tensor-core convolutions: 73 KB (64 channels, a reduction of 1024) and 17 KB
-    pytest.param(2, False, dict(seed=3, in_shape=(64, 6, 6), layers=[("conv", 64, 4, 2, 1), ("relu",), ("fc", 3)]),
+    pytest.param(2, 1, False, 10000, dict(seed=3, in_shape=(64, 6, 6), layers=[("conv", 64, 4, 2, 1), ("relu",), ("fc", 3)]),
                  dict(seed=4, in_shape=(8, 6, 6), layers=[("conv", 9, 3, 1, 1), ("relu",), ("fc", 3)]),
                  id="tensor_core_convolutions"),
+    # windowed rows: 209 KB (four rows of 54 x 54 values of 4 channels and 12 x 12 of 12)
+    # and 81 KB
+    pytest.param(1, 8, False, 200, dict(seed=5, in_shape=(4, 54, 54), layers=[("conv", 12, 10, 4, 0), ("relu",),
+                                                                      ("conv", 16, 12, 1, 0), ("relu",), ("fc", 3)]),
+                 dict(seed=6, in_shape=(4, 34, 34), layers=[("conv", 12, 10, 4, 0), ("relu",), ("conv", 16, 7, 1, 0),
+                                                            ("relu",), ("fc", 3)]),
+                 id="windowed_rows"),
 ])
-def test_two_threads(Context, gemm_path, fused, large, small):
-    alone = [_calls(Context, s, gemm_path, fused, 1) for s in (large, small)]
+def test_two_threads(Context, gemm_path, nodes, fused, calls, large, small):
+    alone = [_calls(Context, s, gemm_path, nodes, fused, 1) for s in (large, small)]
     failed, ready = [], threading.Barrier(2)
 
     def run(spec, want):
         try:
-            got = _calls(Context, spec, gemm_path, fused, CALLS,
+            got = _calls(Context, spec, gemm_path, nodes, fused, calls,
                          lambda i: not failed and (i > 0 or ready.wait(60) >= 0))
             assert failed or (got == want).all(), (got, want)
         except BaseException as e:  # noqa: BLE001 - handed to the test's thread
