@@ -1329,7 +1329,7 @@ void launch_opt_chain(int M, const NetDev& net, const PoolDev& pool, const PropD
   const int lsm = (pool.SD + 1) / 2 * 4;
   const int use_list = smem + lsm <= (smem <= kTwoPerSm ? kTwoPerSm : 220 * 1024) ? 1 : 0;
   if (use_list) smem += lsm;
-  if (smem > 48 * 1024)
+  if (smem > 32 * 1024)  // (48 KB without leave, the kernel's static shared memory included)
     cudaFuncSetAttribute(k_opt_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   const int maxw = fused_maxw(net, pool.d0);
   k_opt_chain<<<M, FT, smem, st>>>(net, pool, props, row_node, row_j, hp, AP_out, GA_out, GB_out, maxw,
@@ -1357,7 +1357,7 @@ void launch_sweep_chain(const NetDev& net, const PoolDev& pool, const PropDev* p
   for (int t = 1; t < t0; ++t) maxw = std::max(maxw, net.d[t]);
   maxw = (maxw + 3) / 4 * 4;
   const int smem = (sweep_wfloats(net, t0) + 2 * SWEEP_RB * maxw) * (int)sizeof(float);
-  if (smem > 48 * 1024)
+  if (smem > 32 * 1024)  // (48 KB without leave, the kernel's static shared memory included)
     cudaFuncSetAttribute(k_sweep_chain<SWEEP_RB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          smem);
   static int sms = 0;
@@ -1398,7 +1398,7 @@ void launch_attack_chain(const NetDev& net, const PropDev* props, int prop, int 
                          float* bx_out, cudaStream_t st) {
   if (n_rows <= 0 || n_starts <= 0) return;
   const int smem = attack_smem_bytes(net);
-  if (smem > 48 * 1024)
+  if (smem > 32 * 1024)  // (48 KB without leave, the kernel's static shared memory included)
     cudaFuncSetAttribute(k_attack_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   k_attack_chain<<<n_rows * n_starts, FT, smem, st>>>(net, props, prop, starts, n_starts, steps,
                                                       best_out, bx_out, fused_maxw(net, net.d[0]), fused_idx(net));
