@@ -25,8 +25,8 @@ def _calls(Context, spec, gemm_path, nodes, fused, calls, go=lambda i: True):
     """The values of `calls` calls that re-bound root nodes, two rows a launch, and bound
     them (and optimise and attack), which are all the same; go(i): whether to make call i."""
     layers = synth.make_network(spec)
-    x = synth.make_image(spec["seed"], spec["in_shape"]).reshape(-1)
-    lo, hi = synth.input_box(x, 0.02)
+    x = np.random.default_rng(spec["seed"]).uniform(0.2, 0.8, spec["in_shape"]).reshape(-1)
+    lo, hi = synth.input_box(x, 0.05)
     C, d = synth.property_rows(0, 3)
     first = None
     with Context(node_capacity=32, gemm_path=gemm_path, row_chunk=2) as ctx:
@@ -62,6 +62,12 @@ def _calls(Context, spec, gemm_path, nodes, fused, calls, go=lambda i: True):
                  dict(seed=6, in_shape=(4, 34, 34), layers=[("conv", 12, 10, 4, 0), ("relu",), ("conv", 16, 7, 1, 0),
                                                             ("relu",), ("fc", 3)]),
                  id="windowed_rows"),
+    # fused kernels: dense-row sweeps (198 and 134 KB), the optimisation loop (93 and 63 KB)
+    # and the pre-attack (74 and 50 KB)
+    pytest.param(0, 2, True, 60, dict(seed=7, in_shape=(30,), layers=[("fc", 6200), ("relu",), ("fc", 64), ("relu",),
+                                                                        ("fc", 3)]),
+                 dict(seed=8, in_shape=(30,), layers=[("fc", 4200), ("relu",), ("fc", 64), ("relu",), ("fc", 3)]),
+                 id="fused_kernels"),
 ])
 def test_two_threads(Context, gemm_path, nodes, fused, calls, large, small):
     alone = [_calls(Context, s, gemm_path, nodes, fused, 1) for s in (large, small)]
