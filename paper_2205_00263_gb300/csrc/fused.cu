@@ -1251,14 +1251,11 @@ __global__ void __launch_bounds__(FT) k_attack_chain(NetDev net, const PropDev* 
 constexpr int kTwoPerSm = 112 * 1024;  // dynamic shared memory of two CTAs per SM
 
 // Allows a fused kernel `bytes` of dynamic shared memory (48 KB without leave, the
-// kernel's static shared memory included).  The limit belongs to the kernel, not to a
-// context: it is the most that any network's plan admits, for every launch, so that
-// host threads do not lower it for one another.
-constexpr int kMostSmem = 220 * 1024;
+// kernel's static shared memory included).
+constexpr int kMostSmem = 220 * 1024;  // of any network's plan
 template <typename F>
-static void allow_smem(F kern, int bytes) {
-  if (bytes > 32 * 1024)
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
+static void set_smem(F kern, int bytes) {
+  if (bytes > 32 * 1024) allow_smem<kMostSmem>(kern);
 }
 
 static int fused_maxw(const NetDev& net, int d0) {
@@ -1340,7 +1337,7 @@ void launch_opt_chain(int M, const NetDev& net, const PoolDev& pool, const PropD
   const int lsm = (pool.SD + 1) / 2 * 4;
   const int use_list = smem + lsm <= (smem <= kTwoPerSm ? kTwoPerSm : kMostSmem) ? 1 : 0;
   if (use_list) smem += lsm;
-  allow_smem(k_opt_chain, smem);
+  set_smem(k_opt_chain, smem);
   const int maxw = fused_maxw(net, pool.d0);
   k_opt_chain<<<M, FT, smem, st>>>(net, pool, props, row_node, row_j, hp, AP_out, GA_out, GB_out, maxw,
                                    ft, fused_idx(net), use_list, err, skip_lb);
@@ -1367,7 +1364,7 @@ void launch_sweep_chain(const NetDev& net, const PoolDev& pool, const PropDev* p
   for (int t = 1; t < t0; ++t) maxw = std::max(maxw, net.d[t]);
   maxw = (maxw + 3) / 4 * 4;
   const int smem = (sweep_wfloats(net, t0) + 2 * SWEEP_RB * maxw) * (int)sizeof(float);
-  allow_smem(k_sweep_chain<SWEEP_RB>, smem);
+  set_smem(k_sweep_chain<SWEEP_RB>, smem);
   static int sms = 0;
   if (!sms && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0) != cudaSuccess)
     sms = 152;
@@ -1406,7 +1403,7 @@ void launch_attack_chain(const NetDev& net, const PropDev* props, int prop, int 
                          float* bx_out, cudaStream_t st) {
   if (n_rows <= 0 || n_starts <= 0) return;
   const int smem = attack_smem_bytes(net);
-  allow_smem(k_attack_chain, smem);
+  set_smem(k_attack_chain, smem);
   k_attack_chain<<<n_rows * n_starts, FT, smem, st>>>(net, props, prop, starts, n_starts, steps,
                                                       best_out, bx_out, fused_maxw(net, net.d[0]), fused_idx(net));
 }

@@ -30,14 +30,11 @@ __device__ float block_sum(float v) {
 }
 
 // Allows a kernel `bytes` of dynamic shared memory.  The 48 KB that need no leave
-// include the kernel's static shared memory (up to 9 KB here).  The limit is the same
-// for every launch of a kernel, the most that any launch of this file takes
-// (win_plan), so that host threads do not lower it for one another.
-constexpr int SMEM_MOST = 216 * 1024;
+// include the kernel's static shared memory (up to 9 KB here).
+constexpr int SMEM_MOST = 216 * 1024;  // of any launch of this file (win_plan)
 template <typename F>
 static void set_smem(F f, int bytes) {
-  if (bytes > 32 * 1024)
-    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MOST);
+  if (bytes > 32 * 1024) allow_smem<SMEM_MOST>(f);
 }
 
 // ---------------------------------------------------------------------------

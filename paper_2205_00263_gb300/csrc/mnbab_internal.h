@@ -15,6 +15,18 @@
 
 namespace mnbab {
 
+// Allows a kernel LIMIT bytes of dynamic shared memory.  The limit belongs to the kernel
+// on the device, not to a context: LIMIT is the most that any launch of the kernel takes,
+// so that host threads do not lower it for one another.  A successful set clears the
+// thread's last error, and with it the error of an earlier launch that was refused (its
+// results were then taken as written): while one is pending nothing is set, and the
+// call's synchronisation reports it.
+template <int LIMIT, typename F>
+inline void allow_smem(F kern) {
+  if (cudaPeekAtLastError() == cudaSuccess)
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, LIMIT);
+}
+
 struct LayerDev {
   int kind;  // 1 fc, 2 conv
   int d_in, d_out;

@@ -516,11 +516,7 @@ int launch_tc_conv(const LayerDev& L, int dir, int M, const float* in, int ld_in
   const dim3 grid(t->ncls[dir] * t->nchunk[dir], (M + TROWS - 1) / TROWS);
   const int NP = t->NP[dir], smem = conv_tc_smem(NP, t->Kp[dir]);
   auto go = [&](auto kern) {
-    // the most that any layer takes (17 to 73 KB), for every layer: the limit belongs to the
-    // kernel, and a host thread that set its own layer's size between another thread's
-    // set and launch made that launch fail
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         conv_tc_smem(64, TC_KMAX));
+    allow_smem<conv_tc_smem(64, TC_KMAX)>(kern);  // 73 KB; layers take 17 KB and more
     kern<<<grid, TC_THREADS, smem, st>>>(t->hi[dir], t->lo[dir], L, dir, NP, M, t->nchunk[dir], in,
                                          ld_in, out, ld_out, e, e.err);
   };

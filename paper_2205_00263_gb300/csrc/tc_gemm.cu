@@ -435,11 +435,7 @@ static int launch_bn(const TcFc* t, int dir, int M, int N, int K, const float* A
                      const float* bias, int bias_div, float* C, int ldc, const Epi& e, int* err,
                      cudaStream_t st) {
   constexpr int smem = Pipe<BN>::SMEM;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_gemm_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    attr = true;
-  }
+  allow_smem<smem>(k_gemm_tc<BN>);
   // split the coefficient rows into the workspace, then the GEMM
   const int Kp = t->Kp[dir];
   const int Rg = (M + 7) / 8 * 8;
