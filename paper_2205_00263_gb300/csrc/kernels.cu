@@ -372,8 +372,7 @@ struct PhaseIdx {
 // both [channel][position][RB rows].  An item is one output position x CB
 // channels x four rows: a 16-byte load brings a coefficient of the four rows,
 // and its CB weights serve all of them, so three loads feed 32 FMAs (CB = 8).
-// Where the items leave threads idle, 2 or 4 adjacent lanes split an item's
-// reduction.  SM: the weights are in shared memory, else in global memory.
+// SM: the weights are in shared memory, else in global memory.
 template <int THREADS, int RG, int CB, bool SM>
 __device__ __forceinline__ void win_conv(const LayerDev& L, const float* __restrict__ Wt, int wci,
                                          const float* A, float* B, int RB, int h, int w,
@@ -456,10 +455,10 @@ __device__ __forceinline__ void win_conv(const LayerDev& L, const float* __restr
   }
 }
 
-// RB = 8, 4 or (windows beyond 56 KB a row) 1 rows per CTA, their windows in shared memory with the rows of a
-// position adjacent.  Bound by the latency of the weight and bound loads (FMA
-// pipe 34% busy) and FP32 FMAs: on the 3x32x32 network's layers 3 and 4 (32768
-// and 8192 rows, 31 GFLOP) 1.2 and 2.9 ms; a thread per output element of one
+// RB = 8, 4 or (where four rows' windows and weights exceed 216 KB) 1 rows per CTA, their
+// windows in shared memory with the rows of a position adjacent.  Bound by the latency
+// of the weight and bound loads (FMA pipe 34% busy) and FP32 FMAs: on the 3x32x32
+// network's layers 3 and 4 (32768 and 8192 rows, 31 GFLOP) 1.2 and 2.9 ms; a thread per output element of one
 // row took 16.3 ms together.  Few items leave threads idle in the deep layers'
 // first steps; splitting their reductions over lanes gained 0.7 ms and changed the
 // order of the sums, which stays that of one row alone.  Four columns of one row
@@ -2390,7 +2389,8 @@ __device__ __forceinline__ int layer_of(const NetDev& net, int f) {
 
 // gamma^T P and gamma^T Phat per neuron (CSR by neuron), and gamma^T p per row.
 // A CTA serves RB consecutive rows.  The CTAs of such a group: RB x GP_SPLIT that sum
-// a share of one row's gamma^T p each (k_reduce_lb adds the shares), RB x `nzero`
+// a share of one row's gamma^T p each (k_reduce_lb adds the shares in a tree: another
+// order than that of one CTA for the row, about 5e-8 of the sum apart), RB x `nzero`
 // that write the zeros of neurons without entries, and the others, which take eight
 // of the layers' listed neurons (those with entries) at a time: each warp brings
 // one neuron's entries to shared memory, all loads in flight (a neuron in three
