@@ -50,9 +50,9 @@ def _rows_per_neuron(seed, counts, k):
     return fn
 
 
-# gamma terms: neurons with no entry, around a warp's width and around a warp's
-# four loads in flight, in a network of a few neurons per CTA and in one of more
-# than 8192 neurons (256 per CTA, a ragged last one); rows over 2 and 3 neurons
+# gamma terms: neurons with no entry (written as zeros by CTAs of their own) and with
+# entries around one and four widths of the warp that stages them, in a network of a few
+# listed neurons and in one of more than 8192 neurons; rows over 2 and 3 neurons
 @pytest.mark.parametrize("spec,k", [
     (dict(seed=31, in_shape=(12,), layers=[("fc", 33), ("relu",), ("fc", 9), ("relu",), ("fc", 3)]), 3),
     (dict(seed=32, in_shape=(1, 33, 33), layers=[("conv", 8, 3, 1, 1), ("relu",), ("fc", 17), ("relu",),
@@ -96,8 +96,8 @@ def test_gamma_terms(Context, spec, k):
             assert close(best[j], top).all()
 
 
-# windowed rows: stride classes of one to more than three taps (two passes over
-# the reduction), kernels smaller than the stride, 1, 2, 3, 4, 5 and 8 input
+# windowed rows: stride classes of one to more than three taps,
+# kernels smaller than the stride, 1, 2, 3, 4, 5 and 8 input
 # channels, windows cut by the padding, a row count that is not a multiple of
 # the rows per CTA, splits in the layers that the rows pass
 @pytest.mark.parametrize("layers,shape", [
@@ -164,7 +164,7 @@ def test_row_roots_are_created_by_the_first_step(Context):
 # tensor-core convolutions in both directions (forced by gemm_path 2): strides
 # 1 to 4, kernels below and above the stride, padding beyond the kernel's reach, planes
 # smaller than a tile and rows across tiles, channel counts that are not multiples of 8 or 16,
-# several channel chunks and class groups; one row and enough rows for two tiles per CTA
+# one to four chunks of 16 channels and 1 to 16 stride classes; one row and 700, four to a CTA
 @pytest.mark.parametrize("layers,shape", [
     ([("conv", 9, 5, 3, 2), ("relu",), ("conv", 17, 2, 4, 1), ("relu",), ("fc", 3)], (8, 22, 15)),
     ([("conv", 24, 3, 1, 2), ("relu",), ("conv", 48, 5, 2, 2), ("relu",), ("fc", 3)], (10, 6, 9)),
